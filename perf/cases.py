@@ -389,3 +389,145 @@ def _run_chunks(st):
     for u0, c, q, k, v, o, lse in st["chunks"]:
         ug.unigist_prefill_chunk(st["p"], u0, c, q, k, v, st["kc"], st["vc"], st["table"], st["lens"], o, lse, st["ws"])
     return [x[5] for x in st["chunks"]], [x[6] for x in st["chunks"]], st["kc"], st["vc"], st["lens"]
+
+
+# ----------------------------------------------------------------------------------------------------------------
+# The same results in 64 bits, from the definition: torch alone, on the sequence as it is (no gist shift, no tiles).
+def exact(case, seed):
+    st = prepare(case, seed)  # for the inputs
+    return {"decode": _exact_decode, "loop": _exact_loop, "train": _exact_train, "packed": _exact_packed,
+            "prefill": _exact_prefill, "chunks": _exact_chunks}[case["kind"]](case, st)
+
+
+def _one_query64(q, k, v):
+    """q [Hq, 128] over k, v [Hkv, tokens, 128]."""
+    hkv = k.shape[0]
+    s = torch.einsum("hgd,htd->hgt", q.double().reshape(hkv, -1, 128), k.double()) / math.sqrt(128)
+    lse = torch.logsumexp(s, -1)
+    return torch.einsum("hgt,htd->hgd", (s - lse[..., None]).exp(), v.double()).reshape(-1, 128), lse.reshape(-1)
+
+
+def _cached(pages, row, length):
+    """The first `length` tokens of one sequence: [Hkv, length, 128]."""
+    return pages[row.long()].transpose(0, 1).flatten(1, 2)[:, :length]
+
+
+def _exact_decode(case, st):
+    rows = [_one_query64(st["q"][i], _cached(st["kc"], st["table"][i], n), _cached(st["vc"], st["table"][i], n))
+            for i, n in enumerate(_decode_lens(case))]
+    return torch.stack([o for o, _ in rows]), torch.stack([lse for _, lse in rows])
+
+
+def _exact_loop(case, st):
+    s, _, r, n, _ = _lens(case)
+    length, steps = _compact_len(case), len(st["q"])
+    live = torch.ones(steps, length + steps, dtype=torch.bool, device=DEV).tril(length)
+    if n >= -(-case["window"] // r):  # the second unit's first token: the oldest unit of the window is gone
+        live[r + 1:, s + n:s + n + r] = False
+    o, lse = [], []
+    for b in range(case["batch"]):
+        k, v = (torch.cat([_cached(st[pages], st["table"][b], length)] + [x[b][:, None] for x in st[new]], 1)
+                for pages, new in (("kc", "k"), ("vc", "v")))
+        rows = [_one_query64(st["q"][i][b], k[:, live[i]], v[:, live[i]]) for i in range(steps)]
+        o.append([x for x, _ in rows])
+        lse.append([x for _, x in rows])
+    return [torch.stack(x) for x in zip(*o)], [torch.stack(x) for x in zip(*lse)], None, None, None
+
+
+def _kinds(case, raw_len, device=DEV):
+    """Of every token of a sequence: its unit (-1: a sink) and whether it is a gist; and the shifted order's tokens."""
+    s, t, r, n, _ = _lens(case, raw_len)
+    i = torch.arange(s + t + n, device=device) - s
+    unit = torch.where(i < 0, -1, i // (r + 1))
+    gist = (i >= 0) & (i % (r + 1) == r)
+    return unit, gist, torch.argsort(gist, stable=True)
+
+
+def _sequence64(case, q, k, v, do=None, raw_len=None):
+    """One sequence, q, do [N, Hq, D], k, v [N, Hkv, D] -> o [N, Hq, D], lse [Hq, N] in shifted order, and with do the
+    gradients dq, dk, dv."""
+    s, _, r, _, w = _lens(case, raw_len)
+    unit, gist, order = _kinds(case, raw_len)
+    (total, hq, d), hkv, scale = q.shape, k.shape[1], 1 / math.sqrt(q.shape[2])
+    out = {name: torch.zeros(x.shape, dtype=torch.float64, device=DEV)
+           for name, x in (("o", q), ("dq", q), ("dk", k), ("dv", v)) if do is not None or name == "o"}
+    lse = torch.empty(hq, total, dtype=torch.float64, device=DEV)
+    at = torch.arange(total, device=DEV)
+    for a in range(0, total, 1024):
+        rows = at[a:a + 1024]
+        first = max((a - s) // (r + 1) - w, 0)  # the first unit whose raw tokens the block's first row sees
+        cols = at[:rows[-1] + 1]
+        cols = cols[(unit[cols] < 0) | gist[cols] | (unit[cols] >= first)]
+        seen = (cols <= rows[:, None]) & ((unit[cols] < 0) | gist[cols] | (unit[cols] >= unit[rows][:, None] - w))
+        for h in range(hkv):
+            heads = slice(h * hq // hkv, (h + 1) * hq // hkv)
+            qh = q[rows, heads].double().transpose(0, 1)
+            kh, vh = k[cols, h].double(), v[cols, h].double()
+            p = (qh @ kh.T * scale).masked_fill_(~seen, -math.inf)
+            norm = torch.logsumexp(p, -1)
+            lse[heads, rows] = norm
+            p = p.sub_(norm[..., None]).exp_()
+            oh = p @ vh
+            out["o"][rows, heads] = oh.transpose(0, 1)
+            if do is not None:
+                doh = do[rows, heads].double().transpose(0, 1)
+                out["dv"][cols, h] += p.flatten(0, 1).T @ doh.flatten(0, 1)
+                p *= (doh @ vh.T).sub_((doh * oh).sum(-1, keepdim=True))
+                out["dq"][rows, heads] = (p @ kh * scale).transpose(0, 1)
+                out["dk"][cols, h] += p.flatten(0, 1).T @ qh.flatten(0, 1) * scale
+    return (out["o"], lse[:, order]) + ((out["dq"], out["dk"], out["dv"]) if do is not None else ())
+
+
+def _rotated64(case, x, sign):
+    """x [N, H, D]: feature j of the first half pairs with j + D / 2; a gist has the position of the raw token after it."""
+    s, _, r, _, _ = _lens(case)
+    unit, gist, _ = _kinds(case, case["raw_len"])
+    i = torch.arange(len(unit), device=DEV)
+    pos = torch.where(gist, s + (unit + 1) * r, i - unit.clamp_min(0)).double()
+    half = x.shape[2] // 2
+    angle = sign * pos[:, None, None] * ROPE_BASE ** (-torch.arange(half, device=DEV, dtype=torch.float64) / half)
+    a, b = x.double().split(half, 2)
+    return torch.cat([a * angle.cos() - b * angle.sin(), b * angle.cos() + a * angle.sin()], 2)
+
+
+def _exact_train(case, st):
+    rope, outs = case["tensors"] == "rope", []
+    for b in range(case["batch"]):
+        q, k = ((_rotated64(case, st[x][b], 1) if rope else st[x][b]) for x in ("q", "k"))
+        o, lse, dq, dk, dv = _sequence64(case, q, k, st["v"][b], st["do"][b])
+        if rope:
+            dq, dk = _rotated64(case, dq, -1), _rotated64(case, dk, -1)
+        outs.append((o, lse, dq, dk, dv))
+    return tuple(torch.stack(x) for x in zip(*outs))
+
+
+def _exact_packed(case, st):
+    outs, a = [], 0
+    for t in st["docs"]:
+        b = a + _tokens(case, t)
+        o, lse, dq, dk, dv = _sequence64(case, *(st[x][a:b] for x in ("q", "k", "v", "do")), raw_len=t)
+        outs.append((o, lse.flatten(), dq, dk, dv))
+        a = b
+    return tuple(torch.cat(x) for x in zip(*outs))
+
+
+def _exact_prefill(case, st):
+    outs = [_sequence64(case, st["q"][b], st["k"][b], st["v"][b]) for b in range(case["batch"])]
+    return torch.stack([o for o, _ in outs]), torch.stack([lse for _, lse in outs]), None, None, None
+
+
+def _exact_chunks(case, st):
+    s, t, r, _, _ = _lens(case)
+    order = _kinds(case, t)[2]  # the tokens in the order [sinks | raw | gists]
+    tokens, outs = [], []  # each chunk's tokens, in its own order of the same form
+    for u0, c, *_ in st["chunks"]:
+        tokens.append(torch.cat([order[:s if u0 == 0 else 0], order[s + u0 * r:s + (u0 + c) * r], order[s + t + u0:s + t + u0 + c]]))
+    place = torch.argsort(torch.cat(tokens))
+    for b in range(case["batch"]):
+        q, k, v = (torch.cat([x[j][b] for x in st["chunks"]])[place] for j in (2, 3, 4))
+        o, lse = _sequence64(case, q, k, v)
+        by_token = torch.empty_like(lse)
+        by_token[:, order] = lse
+        outs.append(([o[i] for i in tokens], [by_token[:, i] for i in tokens]))
+    return ([torch.stack(x) for x in zip(*(o for o, _ in outs))], [torch.stack(x) for x in zip(*(l for _, l in outs))], None,
+            None, None)
