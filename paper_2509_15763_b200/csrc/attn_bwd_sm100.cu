@@ -231,8 +231,8 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     mbar_init(bar_empty[1], 1);
     mbar_init(bar_S, 1);
     mbar_init(bar_dP, 1);
-    mbar_init(bar_P, 256);
-    mbar_init(bar_dS, 256);
+    mbar_init(bar_P, 8);
+    mbar_init(bar_dS, 8);
     mbar_init(bar_final, 1);
     mbar_fence_init();
   }
@@ -304,62 +304,63 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     if (!ok) atomicExch(&g_bwd_timeout, 1u);
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
+      const uint32_t leader = elect_one();
       constexpr uint32_t idesc_s = make_idesc_bf16(KV_BM, KV_BN, false, false);
       constexpr uint32_t idesc_acc = make_idesc_bf16(KV_BM, D, false, true);
       // A operand of the accumulating MMAs: bf16 pairs in TMEM; query columns [0,64) are packed at
       // columns [0,32) of the buffer, query columns [64,128) at columns [64,96)
       auto a_col = [](int kk) { return (kk / 4) * 64 + (kk % 4) * 8; };
-      ok = mbar_wait(bar_kv, 0);
+      ok = mbar_wait_warp(bar_kv, 0);
       for (int it = 0; it < n_iter && ok; ++it) {
         const int st = it & 1;
-        ok = mbar_wait(bar_full[st], (it >> 1) & 1);
+        ok = mbar_wait_warp(bar_full[st], (it >> 1) & 1);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t off = (kk / 4) * SM::kSlab + (kk % 4) * 32;
-          umma_ss(t_A, make_smem_desc(sK + off, 16, 1024), make_smem_desc(sQ[st] + off, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_A, make_smem_desc(sK + off, 16, 1024), make_smem_desc(sQ[st] + off, 16, 1024), idesc_s, kk > 0);
         }
-        umma_commit(bar_S);
+        umma_commit(leader, bar_S);
         if (it > 0) {
           const int ps = (it - 1) & 1;
-          ok = mbar_wait(bar_dS, (it - 1) & 1);
+          ok = mbar_wait_warp(bar_dS, (it - 1) & 1);
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < KV_BN / 16; ++kk)
-            umma_ts(t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
+            umma_ts(leader, t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
                     (it > 1 || kk > 0) ? 1u : 0u);
-          umma_commit(bar_empty[ps]);
+          umma_commit(leader, bar_empty[ps]);
         }
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t off = (kk / 4) * SM::kSlab + (kk % 4) * 32;
-          umma_ss(t_B, make_smem_desc(sV + off, 16, 1024), make_smem_desc(sDO[st] + off, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_B, make_smem_desc(sV + off, 16, 1024), make_smem_desc(sDO[st] + off, 16, 1024), idesc_s, kk > 0);
         }
-        umma_commit(bar_dP);
-        ok = mbar_wait(bar_P, it & 1);
+        umma_commit(leader, bar_dP);
+        ok = mbar_wait_warp(bar_P, it & 1);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < KV_BN / 16; ++kk)
-          umma_ts(t_dV, t_A + a_col(kk), make_smem_desc(sDO[st] + kk * 2048, SM::kSlab, 1024), idesc_acc,
+          umma_ts(leader, t_dV, t_A + a_col(kk), make_smem_desc(sDO[st] + kk * 2048, SM::kSlab, 1024), idesc_acc,
                   (it > 0 || kk > 0) ? 1u : 0u);
       }
       if (ok && n_iter > 0) {
         const int ps = (n_iter - 1) & 1;
-        ok = mbar_wait(bar_dS, (n_iter - 1) & 1);
+        ok = mbar_wait_warp(bar_dS, (n_iter - 1) & 1);
         if (ok) {
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < KV_BN / 16; ++kk)
-            umma_ts(t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
+            umma_ts(leader, t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
                     (n_iter > 1 || kk > 0) ? 1u : 0u);
-          umma_commit(bar_final);
+          umma_commit(leader, bar_final);
         }
       }
-      if (!ok) atomicExch(&g_bwd_timeout, 1u);
+      if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
     }
   } else {
     // ------------------------------------------------------------ compute: thread = key (TMEM lane), 64 query columns
@@ -417,7 +418,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(bar_P);
+      mbar_arrive_warp(bar_P);
       ok = mbar_wait_warp(bar_dP, it & 1);
       if (!ok) break;
       tc_fence_after();
@@ -441,7 +442,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(bar_dS);
+      mbar_arrive_warp(bar_dS);
     }
     if (ok && n_iter > 0) ok = mbar_wait_warp(bar_final, 0);
     if (ok) {
@@ -559,7 +560,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     mbar_init(bar_k, 1);
     mbar_init(bar_v, 1);
     mbar_init(bar_s, 1);
-    mbar_init(bar_p, 128);
+    mbar_init(bar_p, 4);
     mbar_init(bar_pv, 1);
     mbar_fence_init();
   }
@@ -600,35 +601,36 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       if (!ok) atomicExch(&g_bwd_timeout, 1u);
     }
   } else if (warp == 5) {
-    if (elect_one()) {
+    {
+      const uint32_t leader = elect_one();
       constexpr uint32_t idesc_s = make_idesc_bf16(DQ_BM, DQ_BN, false, false);
       constexpr uint32_t idesc_dq = make_idesc_bf16(DQ_BM, D, false, true);
-      ok = mbar_wait(bar_q, 0);
+      ok = mbar_wait_warp(bar_q, 0);
       for (int j = 0; j < nt && ok; ++j) {
-        ok = mbar_wait(bar_k, j & 1) && mbar_wait(bar_v, j & 1);
+        ok = mbar_wait_warp(bar_k, j & 1) && mbar_wait_warp(bar_v, j & 1);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t qoff = (kk / 4) * SM::kQSlab + (kk % 4) * 32, koff = (kk / 4) * SM::kKSlab + (kk % 4) * 32;
-          umma_ss(t_S, make_smem_desc(sQ + qoff, 16, 1024), make_smem_desc(sK + koff, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_S, make_smem_desc(sQ + qoff, 16, 1024), make_smem_desc(sK + koff, 16, 1024), idesc_s, kk > 0);
         }
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t qoff = (kk / 4) * SM::kQSlab + (kk % 4) * 32, koff = (kk / 4) * SM::kKSlab + (kk % 4) * 32;
-          umma_ss(t_dP, make_smem_desc(sDO + qoff, 16, 1024), make_smem_desc(sV + koff, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_dP, make_smem_desc(sDO + qoff, 16, 1024), make_smem_desc(sV + koff, 16, 1024), idesc_s, kk > 0);
         }
-        umma_commit(bar_s);
-        ok = mbar_wait(bar_p, j & 1);
+        umma_commit(leader, bar_s);
+        ok = mbar_wait_warp(bar_p, j & 1);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < DQ_BN / 16; ++kk)
-          umma_ts(t_dQ, t_S + kk * 8, make_smem_desc(sK + kk * 2048, SM::kKSlab, 1024), idesc_dq,
+          umma_ts(leader, t_dQ, t_S + kk * 8, make_smem_desc(sK + kk * 2048, SM::kKSlab, 1024), idesc_dq,
                   (j > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(bar_pv);
+        umma_commit(leader, bar_pv);
       }
-      if (!ok) atomicExch(&g_bwd_timeout, 1u);
+      if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
     }
   } else {
     const int r_in_tile = threadIdx.x;
@@ -685,7 +687,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(bar_p);
+      mbar_arrive_warp(bar_p);
     }
     if (ok) ok = mbar_wait_warp(bar_pv, (nt - 1) & 1);
     if (ok) {
@@ -914,11 +916,11 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
     mbar_init(bar_kv, 1);
     mbar_init(bar_S, 1);
     mbar_init(bar_dP, 1);
-    mbar_init(bar_P, 256);
-    mbar_init(bar_dS, 256);
+    mbar_init(bar_P, 8);
+    mbar_init(bar_dS, 8);
     mbar_init(bar_dSfree, 1);
     mbar_init(bar_dQ, 1);
-    mbar_init(bar_dQfree, 256);
+    mbar_init(bar_dQfree, 8);
     mbar_init(bar_final, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(full_q0 + 8 * i, 1);
@@ -1041,7 +1043,8 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
       if (!ok && lane == 0) atomicExch(&g_bwd_timeout, 1u);
     } else if (warp == kFuMmaWarp) {
       // ---------------------------------------------------------- MMA issuer
-      if (lane == 0) {
+      {
+      const uint32_t leader = elect_one();
         constexpr uint32_t idesc_s = make_idesc_bf16(128, 128, false, false);   // K-major A and B
         constexpr uint32_t idesc_acc = make_idesc_bf16(128, 128, false, true);  // K-major A, MN-major B
         constexpr uint32_t idesc_dq = make_idesc_bf16(128, 128, true, true);    // MN-major A and B
@@ -1061,23 +1064,23 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         auto issue_S = [&](int st) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            umma_ss(t_S, smem_desc_join(k_lo + koff(kk), kHi), smem_desc_join(q_lo + st * kStage + koff(kk), kHi),
+            umma_ss(leader, t_S, smem_desc_join(k_lo + koff(kk), kHi), smem_desc_join(q_lo + st * kStage + koff(kk), kHi),
                     idesc_s, kk > 0);
-          umma_commit(bar_S);
+          umma_commit(leader, bar_S);
         };
         auto issue_dP = [&]() {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            umma_ss(t_dP, smem_desc_join(v_lo + koff(kk), kHi), smem_desc_join(do_lo + koff(kk), kHi), idesc_s, kk > 0);
-          umma_commit(bar_dP);
+            umma_ss(leader, t_dP, smem_desc_join(v_lo + koff(kk), kHi), smem_desc_join(do_lo + koff(kk), kHi), idesc_s, kk > 0);
+          umma_commit(leader, bar_dP);
         };
-        ok = mbar_wait(bar_kv, 0);
+        ok = mbar_wait_warp(bar_kv, 0);
         if (ok && n_iter > 0) {
-          ok = mbar_wait(full_q0, 0);
+          ok = mbar_wait_warp(full_q0, 0);
           if (ok) {
             tc_fence_after();
             issue_S(0);
-            ok = mbar_wait(full_do, 0);
+            ok = mbar_wait_warp(full_do, 0);
           }
           if (ok) {
             tc_fence_after();
@@ -1087,43 +1090,43 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         for (int it = 0; it < n_iter && ok; ++it) {
           const int st = it & 1, ph = it & 1;
           const bool has_next = it + 1 < n_iter;
-          ok = mbar_wait(bar_P, ph);
+          ok = mbar_wait_warp(bar_P, ph);
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)  // dV += P^T dO
-            umma_ts(t_dV, t_S + a_col(kk), smem_desc_join(doT_lo + moff(kk), kHi), idesc_acc,
+            umma_ts(leader, t_dV, t_S + a_col(kk), smem_desc_join(doT_lo + moff(kk), kHi), idesc_acc,
                     (it > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(empty_do);
+          umma_commit(leader, empty_do);
           if (has_next) {
-            ok = mbar_wait(full_q0 + 8 * (st ^ 1), ((it + 1) >> 1) & 1);
+            ok = mbar_wait_warp(full_q0 + 8 * (st ^ 1), ((it + 1) >> 1) & 1);
             if (!ok) break;
             tc_fence_after();
             issue_S(st ^ 1);
           }
-          ok = mbar_wait(bar_dS, ph);
+          ok = mbar_wait_warp(bar_dS, ph);
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)  // dQ^T = K^T dS^T  (contraction over the 128 keys)
-            umma_ss(t_dP, smem_desc_join(kT_lo + moff(kk), kHi), smem_desc_join(dsT_lo + moff(kk), kHi), idesc_dq,
+            umma_ss(leader, t_dP, smem_desc_join(kT_lo + moff(kk), kHi), smem_desc_join(dsT_lo + moff(kk), kHi), idesc_dq,
                     kk > 0);
-          umma_commit(bar_dQ);
+          umma_commit(leader, bar_dQ);
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)  // dK += dS^T Q  (contraction over the 128 queries)
-            umma_ss(t_dK, smem_desc_join(ds_lo + koff(kk), kHi), smem_desc_join(qT_lo + st * kStage + moff(kk), kHi),
+            umma_ss(leader, t_dK, smem_desc_join(ds_lo + koff(kk), kHi), smem_desc_join(qT_lo + st * kStage + moff(kk), kHi),
                     idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(empty_q0 + 8 * st);
-          umma_commit(bar_dSfree);
+          umma_commit(leader, empty_q0 + 8 * st);
+          umma_commit(leader, bar_dSfree);
           if (has_next) {
-            ok = mbar_wait(bar_dQfree, ph) && mbar_wait(full_do, (it + 1) & 1);
+            ok = mbar_wait_warp(bar_dQfree, ph) && mbar_wait_warp(full_do, (it + 1) & 1);
             if (!ok) break;
             tc_fence_after();
             issue_dP();
           }
         }
-        if (ok) umma_commit(bar_final);
-        if (!ok) atomicExch(&g_bwd_timeout, 1u);
+        if (ok) umma_commit(leader, bar_final);
+        if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
       }
     }
   } else if (warp >= 8) {
@@ -1152,7 +1155,8 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
       tmem_ld32(t_dP + lane_base + col0 + 32, v1);
       tmem_wait_ld();
       tc_fence_before();
-      mbar_arrive_relaxed(bar_dQfree);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_relaxed(bar_dQfree);
       auto stage_rows = [&](const uint32_t (&v)[32]) {  // the reduction issued before has finished reading the staging buffer
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncwarp();
@@ -1233,7 +1237,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(bar_P);
+      mbar_arrive_warp(bar_P);
       ok = mbar_wait_warp(bar_dP, it & 1);
       if (ok && it > 0) ok = mbar_wait_warp(bar_dSfree, (it - 1) & 1);  // the previous dS^T has been consumed
       if (!ok) break;
@@ -1259,7 +1263,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
       }
       tc_fence_before();  // the dP^T columns may be overwritten (by dQ^T) once every thread has arrived
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // dS^T visible to the tensor core's reads
-      mbar_arrive(bar_dS);
+      mbar_arrive_warp(bar_dS);
     }
     if (ok && n_iter > 0) ok = mbar_wait_warp(bar_final, 0);
     if (ok) {

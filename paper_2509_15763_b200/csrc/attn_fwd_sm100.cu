@@ -324,8 +324,8 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
     mbar_init(bar_o, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_s[i], 1);
-      mbar_init(bar_p[i], 128);
-      mbar_init(bar_p2[i], 128);
+      mbar_init(bar_p[i], 4);
+      mbar_init(bar_p2[i], 4);
     }
     for (int i = 0; i < kStages; ++i) {
       mbar_init(bar_full + 8 * i, 1);
@@ -393,7 +393,10 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
+    // One lane runs the loop, unlike in the backward: this kernel is bound by the chain scores -> softmax -> P V of a
+    // stream, not by the issue (whole-warp issue measured slower: 616 against 601 us on the one-layer problem).
     if (elect_one()) {
+      constexpr uint32_t leader = 1;
       constexpr uint32_t idesc_qk = make_idesc_bf16(BM, BN, false, false);
       constexpr uint32_t idesc_pv = make_idesc_bf16(BM, D, false, true);
       int n_s[2] = {0, 0}, n_pv[2] = {0, 0};  // products issued so far per stream
@@ -405,10 +408,10 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t off = ((kk / 4) * SM::kSlab + (kk % 4) * 32) >> 4;
-          umma_ss(tmem + i * 128, smem_desc_join(q_lo[i] + off, kHi), smem_desc_join(k_lo + off, kHi), idesc_qk,
+          umma_ss(leader, tmem + i * 128, smem_desc_join(q_lo[i] + off, kHi), smem_desc_join(k_lo + off, kHi), idesc_qk,
                   kk > 0);
         }
-        umma_commit(bar_s[i]);
+        umma_commit(leader, bar_s[i]);
         ++n_s[i];
       };
       auto issue_pv = [&](int i, uint32_t sV, int half) {  // the k steps of one half of the keys of the tile
@@ -417,7 +420,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
 #pragma unroll
         for (int k4 = 0; k4 < BN / 32; ++k4) {
           const int kk = half * (BN / 32) + k4;
-          umma_ts(tmem + 256 + i * 128, tmem + i * 128 + kk * 8, smem_desc_join(v_lo + kk * (2048 >> 4), kHi),
+          umma_ts(leader, tmem + 256 + i * 128, tmem + i * 128 + kk * 8, smem_desc_join(v_lo + kk * (2048 >> 4), kHi),
                   idesc_pv, (n_pv[i] > 0 || kk > 0) ? 1u : 0u);
         }
         n_pv[i] += half;
@@ -433,7 +436,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
           tc_fence_after();
           if (str0.sees(sg, idx)) issue_s(0, ring + slot_of(0) * SM::kTile);
           if (str1.sees(sg, idx)) issue_s(1, ring + slot_of(0) * SM::kTile);
-          umma_commit(bar_empty + 8 * slot_of(0));
+          umma_commit(leader, bar_empty + 8 * slot_of(0));
         }
       }
       for (int j = 0; j < nt && ok; ++j) {
@@ -457,7 +460,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
             tc_fence_after();
             issue_pv(i, ring + slot_of(tv) * SM::kTile, 1);
           }
-          if (i == 1) umma_commit(bar_empty + 8 * slot_of(tv));
+          if (i == 1) umma_commit(leader, bar_empty + 8 * slot_of(tv));
           if (has_next) {
             if (i == 0) {
               ok = wait_full(tk);
@@ -465,11 +468,11 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
               tc_fence_after();
             }
             if (si.sees(nx_sg, nx_idx)) issue_s(i, ring + slot_of(tk) * SM::kTile);
-            if (i == 1) umma_commit(bar_empty + 8 * slot_of(tk));
+            if (i == 1) umma_commit(leader, bar_empty + 8 * slot_of(tk));
           }
         }
       }
-      if (ok) umma_commit(bar_o);
+      if (ok) umma_commit(leader, bar_o);
       if (!ok) atomicExch(&g_fwd_timeout, 1u);
     }
   }
@@ -549,13 +552,13 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
         // hand the first half of P over, so that its part of P V runs under the second half's exponentials
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar_p[i]);
+        mbar_arrive_warp(bar_p[i]);
         float unused;
         tile_sum += row_exp<1>(sc, tS, scale_log2, m_run == -INFINITY ? 0.f : m_run, unused);
         l_run += tile_sum;
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar_p2[i]);
+        mbar_arrive_warp(bar_p2[i]);
         ++cnt;
       }
       if (ok) ok = mbar_wait_warp(bar_o, 0);
