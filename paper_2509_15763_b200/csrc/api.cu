@@ -569,9 +569,8 @@ int32_t unigist_cache_append(const unigist_problem* p, const void* k_new, const 
 size_t unigist_decode_workspace_bytes(int32_t S, int32_t Hq, int32_t Hkv, int32_t D,
                                       int32_t max_blocks) {
   if (S < 1 || Hq < 1 || Hkv < 1 || D < 1 || max_blocks < 1) return 0;
-  const int splits = decode_num_splits(S, Hkv, max_blocks);
-  // per (seq, q head, split): D fp32 partial outputs + running max + running sum
-  return align_up((size_t)S * Hq * splits * (D + 2) * sizeof(float), 256);
+  // partial results of sequences that are cut: D fp32 partial outputs + running max + running sum each
+  return decode_scratch_bytes(S, Hq, Hkv, D, max_blocks);
 }
 
 int32_t unigist_decode(int32_t S, int32_t Hq, int32_t Hkv, int32_t D, float softmax_scale,
@@ -591,11 +590,11 @@ int32_t unigist_decode(int32_t S, int32_t Hq, int32_t Hkv, int32_t D, float soft
   if (!(softmax_scale >= 0.f) || std::isinf(softmax_scale))
     return fail(UNIGIST_ERR_INVALID_ARG, "softmax_scale must be finite and >= 0");
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D);
-  const size_t need = unigist_decode_workspace_bytes(S, Hq, Hkv, D, max_blocks);
+  const size_t need = decode_min_scratch_bytes(S, Hq, Hkv, D, max_blocks);
   if (!workspace || ws_bytes < need)
     return fail(UNIGIST_ERR_WORKSPACE, "decode needs %zu bytes of workspace, got %zu", need, ws_bytes);
   return launch_decode(S, Hq, Hkv, D, scale, q, kc, vc, num_blocks, table, max_blocks, seq_lens, o,
-                       lse, workspace, (cudaStream_t)stream);
+                       lse, workspace, ws_bytes, (cudaStream_t)stream);
 }
 
 int32_t unigist_decode_step(const unigist_problem* p, const void* q, const void* kc, const void* vc, int32_t num_blocks,
@@ -611,13 +610,13 @@ int32_t unigist_decode_step(const unigist_problem* p, const void* q, const void*
   if (!q || !kc || !vc || !table || !seq_lens || !state || !o) return fail(UNIGIST_ERR_INVALID_ARG, "a pointer is NULL");
   if (!aligned16(q) || !aligned16(kc) || !aligned16(vc) || !aligned16(o) || !aligned16(workspace))
     return fail(UNIGIST_ERR_ALIGNMENT, "tensor pointers must be 16-byte aligned");
-  const size_t need = unigist_decode_workspace_bytes(S, Hq, Hkv, D, max_blocks);
+  const size_t need = decode_min_scratch_bytes(S, Hq, Hkv, D, max_blocks);
   if (!workspace || ws_bytes < need)
     return fail(UNIGIST_ERR_WORKSPACE, "decode needs %zu bytes of workspace, got %zu", need, ws_bytes);
   int stride = 0, free_off = 0;
   cache_state_layout(g.r, decode_geom(p, g).k, &stride, &free_off);
   return launch_decode(S, Hq, Hkv, D, scale, q, kc, vc, num_blocks, table, max_blocks, seq_lens, o, lse, workspace,
-                       (cudaStream_t)stream, state, stride, free_off);
+                       ws_bytes, (cudaStream_t)stream, state, stride, free_off);
 }
 
 int32_t unigist_selftest_wait_timeout(void* stream) { return launch_selftest_wait((cudaStream_t)stream); }

@@ -116,6 +116,17 @@ __host__ __device__ inline int seg_row_to_token(const Geom& g, bool interleaved,
   return seg == kSegRaw ? g.s + row + row / g.r : g.s + row * (g.r + 1) + g.r;
 }
 
+// Programmatic dependent launch: the next kernel on the stream may become resident once every block has said so;
+// its pdl_wait() returns when this kernel has completed and its writes are visible.  Both do nothing in a kernel
+// that was launched without the attribute.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Both, where a kernel's prologue ends: before its first access to global memory.
+__device__ __forceinline__ void pdl_begin() {
+  pdl_launch_dependents();
+  pdl_wait();
+}
+
 // Host side helpers (api.cu).
 int32_t fail(int32_t code, const char* fmt, ...);
 int32_t check_problem(const unigist_problem* p, Geom* g, float* scale);
@@ -135,6 +146,32 @@ struct KernelScope {
   int slot;
   cudaStream_t st;
 };
+// Launches a kernel whose first access to global memory comes after pdl_wait() (every thread calls it): the kernel may
+// become resident while the one before it on the stream is still running, so that launch latency and prologue are
+// hidden.  cluster > 1: blocks along x in clusters of that many.  An error is picked up by check_launch.
+template <typename T>
+struct AsIs {
+  using type = T;
+};
+template <typename... KArgs>
+void launch_chained(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, int cluster,
+                    const typename AsIs<KArgs>::type&... args) {
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  void* params[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), params);
+}
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Kernel launchers (one per .cu file).
@@ -191,7 +228,7 @@ int32_t launch_compact_inplace(const Geom& g, const unigist_problem& p, void* kc
                                int32_t* kept_idx, void* ws, cudaStream_t st);
 int32_t launch_decode(int S, int Hq, int Hkv, int D, float scale, const void* q, const void* kc,
                       const void* vc, int num_blocks, const int32_t* table, int max_blocks,
-                      const int32_t* seq_lens, void* o, float* lse, void* ws, cudaStream_t st,
+                      const int32_t* seq_lens, void* o, float* lse, void* ws, size_t ws_bytes, cudaStream_t st,
                       const int32_t* holes = nullptr, int holes_stride = 0, int holes_off = 0);
 int32_t launch_prefill_chunk(const unigist_problem& p, const Geom& g_full, float scale, int u0, int c, const void* q,
                              const void* k, const void* v, void* kc, void* vc, int num_blocks, int32_t* table,
@@ -202,7 +239,9 @@ int32_t launch_cache_state_init(const Geom& g, int B, int units_done, int32_t* s
 int32_t launch_cache_append(const Geom& g, const unigist_problem& p, int is_gist, const void* k_new, const void* v_new,
                             void* kc, void* vc, int num_blocks, const int32_t* table, int max_blocks,
                             int32_t* seq_lens, int32_t* state, cudaStream_t st);
-int decode_num_splits(int S, int Hkv, int max_blocks);
+// Decode scratch: what the plan of a call uses at its best, and the least that is accepted.
+size_t decode_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks);
+size_t decode_min_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks);
 int32_t decode_take_timeout(bool* timed_out);
 int32_t launch_selftest_wait(cudaStream_t st);
 int32_t selftest_take_timeout(bool* timed_out);
