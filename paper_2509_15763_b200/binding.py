@@ -1,8 +1,9 @@
-"""Thin ctypes binding of ``libunigist.so``: argument marshalling only.
+"""Thin binding of ``libunigist.so``: argument marshalling only.
 
 Every function has the name of the C entry point it calls (``include/unigist.h``).  torch is
 used for device memory and streams; all arithmetic of the path runs in the library's kernels.
-A missing library is an error: there is no Python or CPU fallback.
+The calls that enqueue work go through ``_marshal`` (``csrc/marshal.cpp``), the size queries and measurement aids
+through ctypes.  A missing library is an error: there is no Python or CPU fallback.
 """
 from __future__ import annotations
 
@@ -67,6 +68,7 @@ class Problem:
 
 
 _lib = None
+_marshal = None
 
 
 def lib() -> ctypes.CDLL:
@@ -125,6 +127,18 @@ def _check(rc: int):
         raise UnigistError(rc, lib().unigist_last_error_string().decode())
 
 
+def _calls():
+    """The marshalling module.  Its functions take the arguments of the C call of that name in order, a tensor (or
+    None) for a pointer and what belongs to it (sizes, bytes of workspace), a stream or None for torch's current one;
+    they raise ValueError for a tensor that is not a contiguous CUDA tensor and return the call's status."""
+    global _marshal
+    if _marshal is None:
+        lib()
+        from . import _marshal as m
+        _marshal = m
+    return _marshal
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -133,12 +147,6 @@ def _stream(stream=None):
     if stream is None:
         stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
-
-
-def _dev(*ts):
-    for t in ts:
-        if t is not None and (not t.is_cuda or not t.is_contiguous()):
-            raise ValueError("tensors must be contiguous CUDA tensors")
 
 
 def unigist_total_len(p: Problem) -> int:
@@ -188,12 +196,7 @@ def unigist_decode_static(q, k_cache, v_cache, block_table, seq_lens, o, lse=Non
                           softmax_scale: float = 0.0, stream=None):
     """unigist_decode without a workspace argument: scratch is the library's built-in array, so
     nothing is allocated.  Calls on one device must not overlap; see include/unigist.h."""
-    _dev(q, k_cache, v_cache, block_table, seq_lens, o, lse)
-    S, Hq, D = q.shape
-    _check(lib().unigist_decode_static(S, Hq, k_cache.shape[1], D, softmax_scale, _ptr(q), _ptr(k_cache),
-                                       _ptr(v_cache), k_cache.shape[0], _ptr(block_table),
-                                       block_table.shape[1], _ptr(seq_lens), _ptr(o), _ptr(lse),
-                                       _stream(stream)))
+    _check(_calls().decode_static(q, k_cache, v_cache, block_table, seq_lens, o, lse, softmax_scale, stream))
 
 
 def unigist_device_status() -> None:
@@ -223,15 +226,11 @@ def unigist_layout(p: Problem, shift_perm=None, unshift_perm=None, pos_ids=None,
 
 
 def unigist_gist_shift(p: Problem, src, dst, stream=None):
-    _dev(src, dst)
-    _check(lib().unigist_gist_shift(ctypes.byref(p.c()), _ptr(src), _ptr(dst), src.shape[2],
-                                    src.element_size(), _stream(stream)))
+    _check(_calls().gist_shift(p, src, dst, stream))
 
 
 def unigist_gist_unshift(p: Problem, src, dst, stream=None):
-    _dev(src, dst)
-    _check(lib().unigist_gist_unshift(ctypes.byref(p.c()), _ptr(src), _ptr(dst), src.shape[2],
-                                      src.element_size(), _stream(stream)))
+    _check(_calls().gist_unshift(p, src, dst, stream))
 
 
 def _doc_array(doc_raw_len):
@@ -247,52 +246,31 @@ def unigist_docs_workspace_bytes(p: Problem, op: int, doc_raw_len) -> int:
 
 
 def unigist_attn_fwd_docs(p: Problem, doc_raw_len, q, k, v, o, lse, workspace=None, stream=None):
-    _dev(q, k, v, o, lse, workspace)
-    _check(lib().unigist_attn_fwd_docs(ctypes.byref(p.c()), len(doc_raw_len), _doc_array(doc_raw_len), _ptr(q), _ptr(k),
-                                       _ptr(v), _ptr(o), _ptr(lse), _ptr(workspace),
-                                       0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                       _stream(stream)))
+    _check(_calls().attn_fwd_docs(p, doc_raw_len, q, k, v, o, lse, workspace, stream))
 
 
 def unigist_attn_bwd_docs(p: Problem, doc_raw_len, q, k, v, o, lse, d_o, dq, dk, dv, workspace, stream=None):
-    _dev(q, k, v, o, lse, d_o, dq, dk, dv, workspace)
-    _check(lib().unigist_attn_bwd_docs(ctypes.byref(p.c()), len(doc_raw_len), _doc_array(doc_raw_len), _ptr(q), _ptr(k),
-                                       _ptr(v), _ptr(o), _ptr(lse), _ptr(d_o), _ptr(dq), _ptr(dk), _ptr(dv),
-                                       _ptr(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
+    _check(_calls().attn_bwd_docs(p, doc_raw_len, q, k, v, o, lse, d_o, dq, dk, dv, workspace, stream))
 
 
 ROPE_TO_SHIFTED, ROPE_FROM_SHIFTED, ROPE_INVERSE = 1, 2, 4
 
 
 def unigist_rope(p: Problem, src, dst, theta_base: float, flags: int = 0, stream=None):
-    _dev(src, dst)
-    _check(lib().unigist_rope(ctypes.byref(p.c()), _ptr(src), _ptr(dst), src.shape[2], float(theta_base), flags,
-                              _stream(stream)))
+    _check(_calls().rope(p, src, dst, theta_base, flags, stream))
 
 
 def unigist_attn_fwd(p: Problem, q, k, v, o, lse, workspace=None, stream=None):
-    _dev(q, k, v, o, lse, workspace)
-    _check(lib().unigist_attn_fwd(ctypes.byref(p.c()), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                  _ptr(workspace), 0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                  _stream(stream)))
+    _check(_calls().attn_fwd(p, q, k, v, o, lse, workspace, stream))
 
 
 def unigist_attn_bwd(p: Problem, q, k, v, o, lse, d_o, dq, dk, dv, workspace, stream=None):
-    _dev(q, k, v, o, lse, d_o, dq, dk, dv, workspace)
-    _check(lib().unigist_attn_bwd(ctypes.byref(p.c()), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                  _ptr(d_o), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(workspace),
-                                  0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                  _stream(stream)))
+    _check(_calls().attn_bwd(p, q, k, v, o, lse, d_o, dq, dk, dv, workspace, stream))
 
 
 def unigist_kv_compact(p: Problem, k, v, k_cache, v_cache, block_table, seq_lens, kept_idx=None,
                        workspace=None, stream=None):
-    _dev(k, v, k_cache, v_cache, block_table, seq_lens, kept_idx, workspace)
-    _check(lib().unigist_kv_compact(ctypes.byref(p.c()), _ptr(k), _ptr(v), _ptr(k_cache), _ptr(v_cache),
-                                    k_cache.shape[0], _ptr(block_table), block_table.shape[1],
-                                    _ptr(seq_lens), _ptr(kept_idx), _ptr(workspace),
-                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                    _stream(stream)))
+    _check(_calls().kv_compact(p, k, v, k_cache, v_cache, block_table, seq_lens, kept_idx, workspace, stream))
 
 
 def unigist_prefill_workspace_bytes(p: Problem, unit_begin: int, unit_count: int) -> int:
@@ -301,11 +279,8 @@ def unigist_prefill_workspace_bytes(p: Problem, unit_begin: int, unit_count: int
 
 def unigist_prefill_chunk(p: Problem, unit_begin: int, unit_count: int, q, k, v, k_cache, v_cache, block_table,
                           seq_lens, o, lse, workspace, stream=None):
-    _dev(q, k, v, k_cache, v_cache, block_table, seq_lens, o, lse, workspace)
-    _check(lib().unigist_prefill_chunk(ctypes.byref(p.c()), unit_begin, unit_count, _ptr(q), _ptr(k), _ptr(v),
-                                       _ptr(k_cache), _ptr(v_cache), k_cache.shape[0], _ptr(block_table),
-                                       block_table.shape[1], _ptr(seq_lens), _ptr(o), _ptr(lse), _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _stream(stream)))
+    _check(_calls().prefill_chunk(p, unit_begin, unit_count, q, k, v, k_cache, v_cache, block_table, seq_lens, o, lse,
+                                  workspace, stream))
 
 
 def unigist_cache_state_bytes(p: Problem) -> int:
@@ -313,26 +288,17 @@ def unigist_cache_state_bytes(p: Problem) -> int:
 
 
 def unigist_cache_state_init(p: Problem, units_done: int, state, stream=None):
-    _dev(state)
-    _check(lib().unigist_cache_state_init(ctypes.byref(p.c()), units_done, _ptr(state), _stream(stream)))
+    _check(_calls().cache_state_init(p, units_done, state, stream))
 
 
 def unigist_cache_append(p: Problem, k_new, v_new, is_gist: bool, k_cache, v_cache, block_table, seq_lens, state,
                          stream=None):
-    _dev(k_new, v_new, k_cache, v_cache, block_table, seq_lens, state)
-    _check(lib().unigist_cache_append(ctypes.byref(p.c()), _ptr(k_new), _ptr(v_new), int(bool(is_gist)),
-                                      _ptr(k_cache), _ptr(v_cache), k_cache.shape[0], _ptr(block_table),
-                                      block_table.shape[1], _ptr(seq_lens), _ptr(state), _stream(stream)))
+    _check(_calls().cache_append(p, k_new, v_new, bool(is_gist), k_cache, v_cache, block_table, seq_lens, state, stream))
 
 
 def unigist_decode_step(p: Problem, q, k_cache, v_cache, block_table, seq_lens, state, o, lse=None, workspace=None,
                         stream=None):
-    _dev(q, k_cache, v_cache, block_table, seq_lens, state, o, lse, workspace)
-    _check(lib().unigist_decode_step(ctypes.byref(p.c()), _ptr(q), _ptr(k_cache), _ptr(v_cache), k_cache.shape[0],
-                                     _ptr(block_table), block_table.shape[1], _ptr(seq_lens), _ptr(state), _ptr(o),
-                                     _ptr(lse), _ptr(workspace),
-                                     0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                     _stream(stream)))
+    _check(_calls().decode_step(p, q, k_cache, v_cache, block_table, seq_lens, state, o, lse, workspace, stream))
 
 
 def unigist_decode_workspace_bytes(num_seqs, num_q_heads, num_kv_heads, head_dim, max_blocks_per_seq) -> int:
@@ -342,10 +308,4 @@ def unigist_decode_workspace_bytes(num_seqs, num_q_heads, num_kv_heads, head_dim
 
 def unigist_decode(q, k_cache, v_cache, block_table, seq_lens, o, lse=None, workspace=None,
                    softmax_scale: float = 0.0, stream=None):
-    _dev(q, k_cache, v_cache, block_table, seq_lens, o, lse, workspace)
-    S, Hq, D = q.shape
-    _check(lib().unigist_decode(S, Hq, k_cache.shape[1], D, softmax_scale, _ptr(q), _ptr(k_cache),
-                                _ptr(v_cache), k_cache.shape[0], _ptr(block_table), block_table.shape[1],
-                                _ptr(seq_lens), _ptr(o), _ptr(lse), _ptr(workspace),
-                                0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                _stream(stream)))
+    _check(_calls().decode(q, k_cache, v_cache, block_table, seq_lens, o, lse, workspace, softmax_scale, stream))

@@ -1,4 +1,5 @@
-"""Build the C-ABI shared library ``libunigist.so`` in-tree with nvcc for sm_100a."""
+"""Build the C-ABI shared library ``libunigist.so`` (nvcc, sm_100a) and the Python binding's marshalling module
+``_marshal.so`` (g++, against torch) in-tree."""
 from __future__ import annotations
 
 import os
@@ -10,6 +11,7 @@ PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libunigist.so"
+MARSHAL = PKG / "_marshal.so"
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -21,17 +23,45 @@ def sources():
     return sorted(CSRC.glob("*.cu"))
 
 
-def _stale() -> bool:
-    if not LIB.exists():
+def _stale(target: Path, deps) -> bool:
+    if not target.exists():
         return True
-    t = LIB.stat().st_mtime
-    deps = list(CSRC.glob("*.cu")) + list(CSRC.glob("*.cuh")) + [ROOT / "include" / "unigist.h"]
+    t = target.stat().st_mtime
     return any(d.stat().st_mtime > t for d in deps)
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
+    """Build the library, then the marshalling module that links to it."""
+    build_library(force, verbose)
+    build_marshal(force)
+    return LIB
+
+
+def build_marshal(force: bool = False) -> Path:
+    src = CSRC / "marshal.cpp"
+    if not force and not _stale(MARSHAL, [src, ROOT / "include" / "unigist.h"]):
+        return MARSHAL
+    import sysconfig
+
+    import torch
+
+    t = Path(torch.__file__).resolve().parent
+    tmp = MARSHAL.with_suffix(f".tmp{os.getpid()}.so")
+    subprocess.check_call([
+        os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", str(ROOT / "include"),
+        "-I", str(t / "include"), "-I", str(t / "include" / "torch" / "csrc" / "api" / "include"),
+        "-I", "/usr/local/cuda/include", "-I", sysconfig.get_paths()["include"], str(src), "-o", str(tmp),
+        "-L", str(PKG), "-l:libunigist.so", "-Wl,-rpath,$ORIGIN", "-L", str(t / "lib"), "-ltorch_python", "-ltorch_cpu",
+        "-lc10", "-lc10_cuda"])
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
+def build_library(force: bool = False, verbose: bool = False) -> Path:
     """Compile every .cu under csrc/ into one shared library (objects built in parallel)."""
-    if not force and not _stale():
+    deps = list(CSRC.glob("*.cu")) + list(CSRC.glob("*.cuh")) + [ROOT / "include" / "unigist.h"]
+    if not force and not _stale(LIB, deps):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     objdir = PKG / "_build"

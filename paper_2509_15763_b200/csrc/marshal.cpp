@@ -1,0 +1,295 @@
+// Argument marshalling of the Python binding: takes torch tensors, checks that they are contiguous CUDA tensors, and
+// calls the C entry point of the same name (include/unigist.h).  Nothing is kept between calls.
+// A generation loop makes two of these calls per token and is bound by them: through ctypes, with a Python-level
+// check and a pointer object per tensor, a decode call took 14 us of host time against 6 this way.
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <c10/cuda/CUDAStream.h>
+
+#include <vector>
+
+#include "unigist.h"
+
+namespace {
+
+struct Failed {};  // a Python exception is set
+
+[[noreturn]] void raise(PyObject* type, const char* msg) {
+  PyErr_SetString(type, msg);
+  throw Failed{};
+}
+
+// The arguments of one call, read left to right (the caller holds a reference to each for the length of the call).
+struct Args {
+  PyObject* const* a;
+  Py_ssize_t n, at = 0;
+
+  PyObject* next() {
+    if (at >= n) raise(PyExc_TypeError, "too few arguments");
+    return a[at++];
+  }
+  const at::Tensor* tensor() {  // nullptr for None
+    PyObject* o = next();
+    if (o == Py_None) return nullptr;
+    if (!THPVariable_Check(o)) raise(PyExc_TypeError, "expected a torch.Tensor");
+    const at::Tensor& t = THPVariable_Unpack(o);
+    if (!t.is_cuda() || !t.is_contiguous()) raise(PyExc_ValueError, "tensors must be contiguous CUDA tensors");
+    return &t;
+  }
+  long long integer() {
+    const long long v = PyLong_AsLongLong(next());
+    if (v == -1 && PyErr_Occurred()) throw Failed{};
+    return v;
+  }
+  double real() {
+    const double v = PyFloat_AsDouble(next());
+    if (v == -1.0 && PyErr_Occurred()) throw Failed{};
+    return v;
+  }
+  void* stream() {  // None: torch's current stream
+    PyObject* o = next();
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    PyObject* h = PyObject_GetAttrString(o, "cuda_stream");
+    if (!h) throw Failed{};
+    void* p = PyLong_AsVoidPtr(h);
+    Py_DECREF(h);
+    if (!p && PyErr_Occurred()) throw Failed{};
+    return p;
+  }
+  unigist_problem problem() {
+    PyObject* o = next();
+    auto field = [&](const char* name) {
+      PyObject* v = PyObject_GetAttrString(o, name);
+      if (!v) throw Failed{};
+      if (!PyLong_Check(v)) {
+        Py_DECREF(v);
+        raise(PyExc_TypeError, "the fields of a problem are integers (softmax_scale: a number)");
+      }
+      const unsigned long long x = PyLong_AsUnsignedLongLongMask(v);
+      Py_DECREF(v);
+      if (PyErr_Occurred()) throw Failed{};
+      return x;
+    };
+    unigist_problem p;
+    p.batch = (int32_t)field("batch");
+    p.raw_len = (int32_t)field("raw_len");
+    p.num_sinks = (int32_t)field("num_sinks");
+    p.ratio = (int32_t)field("ratio");
+    p.window = (int32_t)field("window");
+    p.num_q_heads = (int32_t)field("num_q_heads");
+    p.num_kv_heads = (int32_t)field("num_kv_heads");
+    p.head_dim = (int32_t)field("head_dim");
+    PyObject* s = PyObject_GetAttrString(o, "softmax_scale");
+    if (!s) throw Failed{};
+    p.softmax_scale = (float)PyFloat_AsDouble(s);
+    Py_DECREF(s);
+    if (PyErr_Occurred()) throw Failed{};
+    p.flags = (uint32_t)field("flags");
+    return p;
+  }
+  std::vector<int32_t> int_list() {
+    PyObject* seq = PySequence_Fast(next(), "expected a sequence of document lengths");
+    if (!seq) throw Failed{};
+    std::vector<int32_t> v;
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(seq); ++i) {
+      PyObject* x = PyNumber_Long(PySequence_Fast_GET_ITEM(seq, i));
+      v.push_back(x ? (int32_t)PyLong_AsUnsignedLongLongMask(x) : 0);
+      Py_XDECREF(x);
+      if (PyErr_Occurred()) {
+        Py_DECREF(seq);
+        throw Failed{};
+      }
+    }
+    Py_DECREF(seq);
+    return v;
+  }
+};
+
+void* ptr(const at::Tensor* t) { return t ? t->data_ptr() : nullptr; }
+float* fptr(const at::Tensor* t) { return static_cast<float*>(ptr(t)); }
+int32_t* iptr(const at::Tensor* t) { return static_cast<int32_t*>(ptr(t)); }
+size_t bytes(const at::Tensor* t) { return t ? (size_t)t->numel() * t->element_size() : 0; }
+int32_t dim(const at::Tensor* t, int64_t i) {
+  if (!t) raise(PyExc_TypeError, "a tensor is missing");
+  if (i >= t->dim()) raise(PyExc_IndexError, "a tensor has too few dimensions");
+  return (int32_t)t->size(i);
+}
+
+// Runs a call with the interpreter lock released and hands its status back.
+template <typename Fn>
+int32_t unlocked(Fn fn) {
+  int32_t rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = fn();
+  Py_END_ALLOW_THREADS
+  return rc;
+}
+
+// A METH_FASTCALL function around `body(Args&) -> status`.
+template <int32_t (*kBody)(Args&)>
+PyObject* call(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  try {
+    Args args{a, n};
+    return PyLong_FromLong(kBody(args));
+  } catch (const Failed&) {
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+  }
+  return nullptr;
+}
+
+template <decltype(unigist_gist_shift)* kFn>
+int32_t shift(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *src = a.tensor(), *dst = a.tensor();
+  void* st = a.stream();
+  const int32_t heads = dim(src, 2), eb = (int32_t)src->element_size();
+  return unlocked([&] { return kFn(&p, ptr(src), ptr(dst), heads, eb, st); });
+}
+
+int32_t rope(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *src = a.tensor(), *dst = a.tensor();
+  const float base = (float)a.real();
+  const uint32_t flags = (uint32_t)a.integer();
+  void* st = a.stream();
+  const int32_t heads = dim(src, 2);
+  return unlocked([&] { return unigist_rope(&p, ptr(src), ptr(dst), heads, base, flags, st); });
+}
+
+int32_t attn_fwd(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  return unlocked([&] { return unigist_attn_fwd(&p, ptr(q), ptr(k), ptr(v), ptr(o), fptr(lse), ptr(ws), bytes(ws), st); });
+}
+
+int32_t attn_bwd(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *d_o = a.tensor(),
+                   *dq = a.tensor(), *dk = a.tensor(), *dv = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  return unlocked([&] {
+    return unigist_attn_bwd(&p, ptr(q), ptr(k), ptr(v), ptr(o), fptr(lse), ptr(d_o), ptr(dq), ptr(dk), ptr(dv), ptr(ws),
+                            bytes(ws), st);
+  });
+}
+
+int32_t attn_fwd_docs(Args& a) {
+  const unigist_problem p = a.problem();
+  const std::vector<int32_t> docs = a.int_list();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  return unlocked([&] {
+    return unigist_attn_fwd_docs(&p, (int32_t)docs.size(), docs.data(), ptr(q), ptr(k), ptr(v), ptr(o), fptr(lse), ptr(ws),
+                                 bytes(ws), st);
+  });
+}
+
+int32_t attn_bwd_docs(Args& a) {
+  const unigist_problem p = a.problem();
+  const std::vector<int32_t> docs = a.int_list();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *d_o = a.tensor(),
+                   *dq = a.tensor(), *dk = a.tensor(), *dv = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  return unlocked([&] {
+    return unigist_attn_bwd_docs(&p, (int32_t)docs.size(), docs.data(), ptr(q), ptr(k), ptr(v), ptr(o), fptr(lse), ptr(d_o),
+                                 ptr(dq), ptr(dk), ptr(dv), ptr(ws), bytes(ws), st);
+  });
+}
+
+int32_t kv_compact(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *k = a.tensor(), *v = a.tensor(), *kc = a.tensor(), *vc = a.tensor(), *table = a.tensor(),
+                   *lens = a.tensor(), *kept = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  const int32_t blocks = dim(kc, 0), width = dim(table, 1);
+  return unlocked([&] {
+    return unigist_kv_compact(&p, ptr(k), ptr(v), ptr(kc), ptr(vc), blocks, iptr(table), width, iptr(lens), iptr(kept), ptr(ws),
+                              bytes(ws), st);
+  });
+}
+
+int32_t prefill_chunk(Args& a) {
+  const unigist_problem p = a.problem();
+  const int32_t u0 = (int32_t)a.integer(), c = (int32_t)a.integer();
+  const at::Tensor *q = a.tensor(), *k = a.tensor(), *v = a.tensor(), *kc = a.tensor(), *vc = a.tensor(), *table = a.tensor(),
+                   *lens = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  const int32_t blocks = dim(kc, 0), width = dim(table, 1);
+  return unlocked([&] {
+    return unigist_prefill_chunk(&p, u0, c, ptr(q), ptr(k), ptr(v), ptr(kc), ptr(vc), blocks, iptr(table), width, iptr(lens),
+                                 ptr(o), fptr(lse), ptr(ws), bytes(ws), st);
+  });
+}
+
+int32_t cache_state_init(Args& a) {
+  const unigist_problem p = a.problem();
+  const int32_t units = (int32_t)a.integer();
+  const at::Tensor* state = a.tensor();
+  void* st = a.stream();
+  return unlocked([&] { return unigist_cache_state_init(&p, units, iptr(state), st); });
+}
+
+int32_t cache_append(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *k = a.tensor(), *v = a.tensor();
+  const int32_t is_gist = (int32_t)a.integer();
+  const at::Tensor *kc = a.tensor(), *vc = a.tensor(), *table = a.tensor(), *lens = a.tensor(), *state = a.tensor();
+  void* st = a.stream();
+  const int32_t blocks = dim(kc, 0), width = dim(table, 1);
+  return unlocked([&] {
+    return unigist_cache_append(&p, ptr(k), ptr(v), is_gist, ptr(kc), ptr(vc), blocks, iptr(table), width, iptr(lens),
+                                iptr(state), st);
+  });
+}
+
+int32_t decode_step(Args& a) {
+  const unigist_problem p = a.problem();
+  const at::Tensor *q = a.tensor(), *kc = a.tensor(), *vc = a.tensor(), *table = a.tensor(), *lens = a.tensor(),
+                   *state = a.tensor(), *o = a.tensor(), *lse = a.tensor(), *ws = a.tensor();
+  void* st = a.stream();
+  const int32_t blocks = dim(kc, 0), width = dim(table, 1);
+  return unlocked([&] {
+    return unigist_decode_step(&p, ptr(q), ptr(kc), ptr(vc), blocks, iptr(table), width, iptr(lens), iptr(state), ptr(o),
+                               fptr(lse), ptr(ws), bytes(ws), st);
+  });
+}
+
+template <bool kStatic>
+int32_t decode(Args& a) {
+  const at::Tensor *q = a.tensor(), *kc = a.tensor(), *vc = a.tensor(), *table = a.tensor(), *lens = a.tensor(),
+                   *o = a.tensor(), *lse = a.tensor(), *ws = kStatic ? nullptr : a.tensor();
+  const float scale = (float)a.real();
+  void* st = a.stream();
+  if (!q || q->dim() != 3) raise(PyExc_ValueError, "q must be [num_seqs, num_q_heads, head_dim]");
+  const int32_t S = dim(q, 0), Hq = dim(q, 1), D = dim(q, 2), Hkv = dim(kc, 1), blocks = dim(kc, 0), width = dim(table, 1);
+  return unlocked([&] {
+    return kStatic ? unigist_decode_static(S, Hq, Hkv, D, scale, ptr(q), ptr(kc), ptr(vc), blocks, iptr(table), width,
+                                           iptr(lens), ptr(o), fptr(lse), st)
+                   : unigist_decode(S, Hq, Hkv, D, scale, ptr(q), ptr(kc), ptr(vc), blocks, iptr(table), width, iptr(lens),
+                                    ptr(o), fptr(lse), ptr(ws), bytes(ws), st);
+  });
+}
+
+#define FN(name, ...) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&call<__VA_ARGS__>)), METH_FASTCALL, nullptr}
+PyMethodDef kMethods[] = {FN("gist_shift", shift<unigist_gist_shift>),
+                          FN("gist_unshift", shift<unigist_gist_unshift>),
+                          FN("rope", rope),
+                          FN("attn_fwd", attn_fwd),
+                          FN("attn_bwd", attn_bwd),
+                          FN("attn_fwd_docs", attn_fwd_docs),
+                          FN("attn_bwd_docs", attn_bwd_docs),
+                          FN("kv_compact", kv_compact),
+                          FN("prefill_chunk", prefill_chunk),
+                          FN("cache_state_init", cache_state_init),
+                          FN("cache_append", cache_append),
+                          FN("decode_step", decode_step),
+                          FN("decode", decode<false>),
+                          FN("decode_static", decode<true>),
+                          {nullptr, nullptr, 0, nullptr}};
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&kModule); }
