@@ -160,7 +160,10 @@ __device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key
 }
 
 // ------------------------------------------------------------------------------------------------
-// dK / dV kernel
+// dK / dV kernel.  Bound by the chain scores -> P -> dP -> dS of one step, not by the tensor pipe: with head_dim 64
+// tensor memory has room for a second S buffer and shared memory for four Q / dO stages, which take the scores and the
+// loads off that chain; with heavy tiles first over all heads, two sequences of 8190 raw tokens (ratio 7, 16 / 4
+// heads) took 0.70 ms before and 0.45 now.
 constexpr int KV_BM = 128;       // keys per block (TMEM lanes)
 constexpr int KV_BN = 128;       // queries per step
 constexpr int kKvThreads = 320;  // 8 compute warps, 1 TMA warp, 1 MMA warp
@@ -169,8 +172,11 @@ template <int D>
 struct KvSmem {
   static constexpr int kSlab = 128 * 128;
   static constexpr int kTile = kSlab * (D / 64);
-  static constexpr int kStats = 2 * 2 * KV_BN * 4;  // [stage][lse2 | delta][128] fp32
-  static constexpr int kBytes = 6 * kTile + kStats + 1024 + 256;
+  static constexpr int kStages = D == 64 ? 4 : 2;              // of Q, dO, LSE and Delta
+  static constexpr int kSBufs = D == 64 ? 2 : 1;               // buffers of S^T / P^T in tensor memory
+  static constexpr int kOffStats = (2 + 2 * kStages) * kTile;  // [stage][lse2 | delta][128] fp32
+  static constexpr int kOffBars = kOffStats + kStages * 2 * KV_BN * 4;
+  static constexpr int kBytes = kOffBars + 256 + 1024;
 };
 
 template <int D>
@@ -183,27 +189,40 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
                            const __grid_constant__ CUtensorMap tm_v_raw, const __grid_constant__ CUtensorMap tm_v_gist,
                            Geom g, int Hq, int Hkv, float scale, const float* __restrict__ lse,
                            const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk,
-                           __nv_bfloat16* __restrict__ dv, int n_sink_kt, int n_gist_kt) {
+                           __nv_bfloat16* __restrict__ dv, int n_sink_kt, int n_gist_kt, int n_raw_kt, int pairs,
+                           FastDiv heavy_div, FastDiv raw_div, FastDiv hkv_div) {
   using SM = KvSmem<D>;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
   const uint32_t sK = base, sV = base + SM::kTile;
-  const uint32_t sQ[2] = {base + 2 * SM::kTile, base + 4 * SM::kTile};
-  const uint32_t sDO[2] = {base + 3 * SM::kTile, base + 5 * SM::kTile};
-  float* stats = reinterpret_cast<float*>(gen + 6 * SM::kTile);  // [stage][2][128]
-  const uint32_t bars = base + 6 * SM::kTile + SM::kStats;
-  const uint32_t bar_kv = bars, bar_full[2] = {bars + 8, bars + 16}, bar_empty[2] = {bars + 24, bars + 32},
-                 bar_S = bars + 40, bar_dP = bars + 48, bar_P = bars + 56, bar_dS = bars + 64, bar_final = bars + 72,
-                 tmem_slot = bars + 80;
-  volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen + 6 * SM::kTile + SM::kStats + 80);
+  constexpr int kSt = SM::kStages;
+  const uint32_t sQ0 = base + 2 * SM::kTile, sDO0 = sQ0 + kSt * SM::kTile;  // stage st at + st * kTile
+  float* stats = reinterpret_cast<float*>(gen + SM::kOffStats);             // [stage][2][128]
+  const uint32_t bars = base + SM::kOffBars;
+  // (two barriers per S buffer: a buffer's next phase cannot complete before everyone has seen the one before)
+  const uint32_t bar_kv = bars, bar_S = bars + 8 /* + 8 * buffer */, bar_dP = bars + 24,
+                 bar_P = bars + 32 /* + 8 * buffer */, bar_dS = bars + 48, bar_final = bars + 56, tmem_slot = bars + 64;
+  const uint32_t bar_full = bars + 72, bar_empty = bars + 72 + 8 * kSt;  // + 8 * stage
+  volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen + SM::kOffBars + 64);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int hk = blockIdx.y, b = blockIdx.z, G = Hq / Hkv;
-  // sink and gist key tiles are seen by every later query: heaviest, scheduled first
-  const int rank = blockIdx.x;
-  const int kseg = rank < n_sink_kt ? kSegSink : (rank < n_sink_kt + n_gist_kt ? kSegGist : kSegRaw);
-  const int kt = rank - (kseg == kSegSink ? 0 : (kseg == kSegGist ? n_sink_kt : n_sink_kt + n_gist_kt));
+  const int G = Hq / Hkv;
+  // Sink and gist key tiles are seen by every later query: heaviest, and first over ALL heads and batch indices (a
+  // long walk that starts late is the kernel's tail); the tiles of one KV head are neighbours and share its Q and dO.
+  const int n_heavy = n_sink_kt + n_gist_kt;
+  int pair, rank;  // pair = batch index * Hkv + KV head
+  if ((int)blockIdx.x < n_heavy * pairs) {
+    pair = fdiv(heavy_div, blockIdx.x);
+    rank = blockIdx.x - pair * n_heavy;
+  } else {
+    const int y = blockIdx.x - n_heavy * pairs;
+    pair = fdiv(raw_div, y);
+    rank = n_heavy + (y - pair * n_raw_kt);
+  }
+  const int b = fdiv(hkv_div, pair), hk = pair - b * Hkv;
+  const int kseg = rank < n_sink_kt ? kSegSink : (rank < n_heavy ? kSegGist : kSegRaw);
+  const int kt = rank - (kseg == kSegSink ? 0 : (kseg == kSegGist ? n_sink_kt : n_heavy));
   const int key_seg_len = seg_len(g, kseg);
   const int key_seg_base = seg_base(g, kseg);
   const int key_a = kt * KV_BM, key_b = min(key_a + KV_BM - 1, key_seg_len - 1);
@@ -225,13 +244,15 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 
   if (threadIdx.x == 0) {
     mbar_init(bar_kv, 1);
-    mbar_init(bar_full[0], 1);
-    mbar_init(bar_full[1], 1);
-    mbar_init(bar_empty[0], 1);
-    mbar_init(bar_empty[1], 1);
+    for (int i = 0; i < kSt; ++i) {
+      mbar_init(bar_full + 8 * i, 1);
+      mbar_init(bar_empty + 8 * i, 1);
+    }
     mbar_init(bar_S, 1);
+    mbar_init(bar_S + 8, 1);
     mbar_init(bar_dP, 1);
     mbar_init(bar_P, 8);
+    mbar_init(bar_P + 8, 8);
     mbar_init(bar_dS, 8);
     mbar_init(bar_final, 1);
     mbar_fence_init();
@@ -241,12 +262,20 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
-  const uint32_t t_dK = tmem, t_dV = tmem + 128, t_A = tmem + 256, t_B = tmem + 384;
+  const uint32_t t_dK = tmem, t_dV = tmem + D, t_A0 = tmem + 2 * D /* + 128 * S buffer */, t_B = t_A0 + 128 * SM::kSBufs;
+  static_assert(2 * D + 128 * (SM::kSBufs + 1) <= 512, "tensor memory");
   bool ok = true;
 
-  auto tile_of = [&](int it, int& qseg, int& qt, int& head) {
-    const int t = it / G;
-    head = hk * G + (it - t * G);
+  // steps: query tiles (raw, gist, sink) from the first one up, the G heads of a tile back to back
+  struct StepIter {
+    int t, hd;
+  };
+  auto advance = [&](StepIter& x) {
+    if (++x.hd == G) x.hd = 0, ++x.t;
+  };
+  auto tile_of = [&](const StepIter& x, int& qseg, int& qt, int& head) {
+    const int t = x.t;
+    head = hk * G + x.hd;
     if (t < n_raw_q) {
       qseg = kSegRaw;
       qt = rq_lo + t;
@@ -271,35 +300,50 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
         tma_load_4d(sV + sl * SM::kSlab, mv, bar_kv, sl * 64, hk, key_a, b);
       }
     }
-    for (int it = 0; it < n_iter; ++it) {
-      const int st = it & 1;
+    // LSE (in log2 units) and Delta of a step's 128 query rows, 4 rows per lane, fetched one step ahead
+    float st_l[KV_BN / 32], st_d[KV_BN / 32];
+    auto fetch_stats = [&](const StepIter& at) {
       int qseg, qt, head;
-      tile_of(it, qseg, qt, head);
-      if (it >= 2) ok = mbar_wait_warp(bar_empty[st], ((it >> 1) - 1) & 1);
-      if (!ok) break;
-      const int q_seg_len = seg_len(g, qseg), q_seg_base = seg_base(g, qseg);
-      float* ls = stats + st * 2 * KV_BN;
-      const long long row_base = ((long long)b * Hq + head) * g.N + q_seg_base;
+      tile_of(at, qseg, qt, head);
+      const int q_seg_len = seg_len(g, qseg);
+      const long long row_base = ((long long)b * Hq + head) * g.N + seg_base(g, qseg);
 #pragma unroll
       for (int i = 0; i < KV_BN / 32; ++i) {
-        const int c = lane + 32 * i, row = qt * KV_BN + c;
+        const int row = qt * KV_BN + lane + 32 * i;
         const bool valid = row < q_seg_len;
         // rows past the segment get LSE = +inf, so their P is exactly zero
-        ls[c] = valid ? lse[row_base + row] * kLog2e : INFINITY;
-        ls[KV_BN + c] = valid ? delta[row_base + row] : 0.f;
+        st_l[i] = valid ? lse[row_base + row] * kLog2e : INFINITY;
+        st_d[i] = valid ? delta[row_base + row] : 0.f;
+      }
+    };
+    StepIter cur{0, 0}, ahead{0, 0};
+    if (n_iter > 0) fetch_stats(ahead);
+    for (int it = 0; it < n_iter; ++it, advance(cur)) {
+      const int st = it % kSt;
+      int qseg, qt, head;
+      tile_of(cur, qseg, qt, head);
+      if (it >= kSt) ok = mbar_wait_warp(bar_empty + 8 * st, (it / kSt - 1) & 1);
+      if (!ok) break;
+      float* ls = stats + st * 2 * KV_BN;
+#pragma unroll
+      for (int i = 0; i < KV_BN / 32; ++i) {
+        ls[lane + 32 * i] = st_l[i];
+        ls[KV_BN + lane + 32 * i] = st_d[i];
       }
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive_expect_tx(bar_full[st], 2 * SM::kTile);
+        mbar_arrive_expect_tx(bar_full + 8 * st, 2 * SM::kTile);
         const CUtensorMap* mq = qseg == kSegRaw ? &tm_q_raw : (qseg == kSegGist ? &tm_q_gist : &tm_q_sink);
         const CUtensorMap* md = qseg == kSegRaw ? &tm_do_raw : (qseg == kSegGist ? &tm_do_gist : &tm_do_sink);
 #pragma unroll
         for (int sl = 0; sl < D / 64; ++sl) {
-          tma_load_4d(sQ[st] + sl * SM::kSlab, mq, bar_full[st], sl * 64, head, qt * KV_BN, b);
-          tma_load_4d(sDO[st] + sl * SM::kSlab, md, bar_full[st], sl * 64, head, qt * KV_BN, b);
+          tma_load_4d(sQ0 + st * SM::kTile + sl * SM::kSlab, mq, bar_full + 8 * st, sl * 64, head, qt * KV_BN, b);
+          tma_load_4d(sDO0 + st * SM::kTile + sl * SM::kSlab, md, bar_full + 8 * st, sl * 64, head, qt * KV_BN, b);
         }
       }
       __syncwarp();
+      advance(ahead);
+      if (it + 1 < n_iter) fetch_stats(ahead);
     }
     if (!ok) atomicExch(&g_bwd_timeout, 1u);
   } else if (warp == 9) {
@@ -311,55 +355,56 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       // A operand of the accumulating MMAs: bf16 pairs in TMEM; query columns [0,64) are packed at
       // columns [0,32) of the buffer, query columns [64,128) at columns [64,96)
       auto a_col = [](int kk) { return (kk / 4) * 64 + (kk % 4) * 8; };
-      ok = mbar_wait_warp(bar_kv, 0);
-      for (int it = 0; it < n_iter && ok; ++it) {
-        const int st = it & 1;
-        ok = mbar_wait_warp(bar_full[st], (it >> 1) & 1);
-        if (!ok) break;
+      auto issue_S = [&](int it) {  // S^T of step it, once its Q (and dO) have arrived
+        const int st = it % kSt, sb = it % SM::kSBufs;
+        if (!mbar_wait_warp(bar_full + 8 * st, (it / kSt) & 1)) return false;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t off = (kk / 4) * SM::kSlab + (kk % 4) * 32;
-          umma_ss(leader, t_A, make_smem_desc(sK + off, 16, 1024), make_smem_desc(sQ[st] + off, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_A0 + 128 * sb, make_smem_desc(sK + off, 16, 1024),
+                  make_smem_desc(sQ0 + st * SM::kTile + off, 16, 1024), idesc_s, kk > 0);
         }
-        umma_commit(leader, bar_S);
-        if (it > 0) {
-          const int ps = (it - 1) & 1;
-          ok = mbar_wait_warp(bar_dS, (it - 1) & 1);
-          if (!ok) break;
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < KV_BN / 16; ++kk)
-            umma_ts(leader, t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
-                    (it > 1 || kk > 0) ? 1u : 0u);
-          umma_commit(leader, bar_empty[ps]);
-        }
+        umma_commit(leader, bar_S + 8 * sb);
+        return true;
+      };
+      auto issue_dP = [&](int it) {
+        const int st = it % kSt;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t off = (kk / 4) * SM::kSlab + (kk % 4) * 32;
-          umma_ss(leader, t_B, make_smem_desc(sV + off, 16, 1024), make_smem_desc(sDO[st] + off, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_B, make_smem_desc(sV + off, 16, 1024), make_smem_desc(sDO0 + st * SM::kTile + off, 16, 1024),
+                  idesc_s, kk > 0);
         }
         umma_commit(leader, bar_dP);
-        ok = mbar_wait_warp(bar_P, it & 1);
+      };
+      ok = mbar_wait_warp(bar_kv, 0);
+      if (ok && n_iter > 0) ok = issue_S(0);
+      if (ok && n_iter > 0) issue_dP(0);
+      for (int it = 0; it < n_iter && ok; ++it) {
+        const int st = it % kSt, sb = it % SM::kSBufs;
+        // With two S buffers the next scores do not wait for this step's P^T: the exponentials of step it + 1 follow
+        // dS of step it at once, and dP(it + 1) runs under them.
+        if (SM::kSBufs == 2 && it + 1 < n_iter) ok = issue_S(it + 1);
+        ok = ok && mbar_wait_warp(bar_P + 8 * sb, (it / SM::kSBufs) & 1);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < KV_BN / 16; ++kk)
-          umma_ts(leader, t_dV, t_A + a_col(kk), make_smem_desc(sDO[st] + kk * 2048, SM::kSlab, 1024), idesc_acc,
-                  (it > 0 || kk > 0) ? 1u : 0u);
-      }
-      if (ok && n_iter > 0) {
-        const int ps = (n_iter - 1) & 1;
-        ok = mbar_wait_warp(bar_dS, (n_iter - 1) & 1);
-        if (ok) {
-          tc_fence_after();
+          umma_ts(leader, t_dV, t_A0 + 128 * sb + a_col(kk), make_smem_desc(sDO0 + st * SM::kTile + kk * 2048, SM::kSlab, 1024),
+                  idesc_acc, (it > 0 || kk > 0) ? 1u : 0u);
+        if (SM::kSBufs == 1 && it + 1 < n_iter) ok = issue_S(it + 1);
+        ok = ok && mbar_wait_warp(bar_dS, it & 1);
+        if (!ok) break;
+        tc_fence_after();
 #pragma unroll
-          for (int kk = 0; kk < KV_BN / 16; ++kk)
-            umma_ts(leader, t_dK, t_B + a_col(kk), make_smem_desc(sQ[ps] + kk * 2048, SM::kSlab, 1024), idesc_acc,
-                    (n_iter > 1 || kk > 0) ? 1u : 0u);
-          umma_commit(leader, bar_final);
-        }
+        for (int kk = 0; kk < KV_BN / 16; ++kk)
+          umma_ts(leader, t_dK, t_B + a_col(kk), make_smem_desc(sQ0 + st * SM::kTile + kk * 2048, SM::kSlab, 1024), idesc_acc,
+                  (it > 0 || kk > 0) ? 1u : 0u);
+        umma_commit(leader, bar_empty + 8 * st);
+        if (it + 1 < n_iter) issue_dP(it + 1);
       }
+      if (ok && n_iter > 0) umma_commit(leader, bar_final);
       if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
     }
   } else {
@@ -374,10 +419,12 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
     key_q_interval3(g, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
 
-    for (int it = 0; it < n_iter && ok; ++it) {
-      const int st = it & 1;
+    StepIter cur{0, 0};
+    for (int it = 0; it < n_iter && ok; ++it, advance(cur)) {
+      const int st = it % kSt, sb = it % SM::kSBufs;
+      const uint32_t t_A = t_A0 + 128 * sb;
       int qseg, qt, head;
-      tile_of(it, qseg, qt, head);
+      tile_of(cur, qseg, qt, head);
       const int q0 = qt * KV_BN, q_seg_len = seg_len(g, qseg);
       const int qb = min(q0 + KV_BN - 1, q_seg_len - 1);
       // full: every (query, key) pair of the tile is visible -> no mask arithmetic
@@ -388,7 +435,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       const int hi = (qseg == kSegRaw ? my_hi_r : (qseg == kSegGist ? my_hi_g : my_hi_s)) - q0 - 64 * hf;
       const float* ls = stats + st * 2 * KV_BN + 64 * hf;
       const float* dl = ls + KV_BN;
-      ok = mbar_wait_warp(bar_full[st], (it >> 1) & 1) && mbar_wait_warp(bar_S, it & 1);
+      ok = mbar_wait_warp(bar_full + 8 * st, (it / kSt) & 1) && mbar_wait_warp(bar_S + 8 * sb, (it / SM::kSBufs) & 1);
       if (!ok) break;
       tc_fence_after();
       float p[64];
@@ -418,7 +465,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive_warp(bar_P);
+      mbar_arrive_warp(bar_P + 8 * sb);
       ok = mbar_wait_warp(bar_dP, it & 1);
       if (!ok) break;
       tc_fence_after();
@@ -493,7 +540,8 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 }
 
 // ------------------------------------------------------------------------------------------------
-// dQ kernel
+// dQ kernel.  Two blocks per SM cover each other's softmax; with head_dim 64 a ring of four K / V stages and a second S
+// buffer leave only dP and dS on the chain of a step (the problem above: 0.38 ms -> 0.285).
 constexpr int DQ_BM = 128;  // query rows per block
 constexpr int DQ_BN = 64;   // keys per step
 constexpr int kDqThreads = 192;
@@ -502,7 +550,12 @@ template <int D>
 struct DqSmem {
   static constexpr int kQSlab = DQ_BM * 128, kQTile = kQSlab * (D / 64);
   static constexpr int kKSlab = DQ_BN * 128, kKTile = kKSlab * (D / 64);
-  static constexpr int kBytes = 2 * kQTile + 2 * kKTile + 1024 + 128;
+  // Two blocks share an SM (its shared memory, and 256 tensor-memory columns each); with head_dim 64 that leaves room
+  // for a ring of K / V tiles and a second S buffer.
+  static constexpr int kStages = D == 64 ? 4 : 1;
+  static constexpr int kSBufs = D == 64 ? 2 : 1;
+  static constexpr int kOffBars = 2 * kQTile + 2 * kStages * kKTile;
+  static constexpr int kBytes = kOffBars + 256 + 1024;
 };
 
 template <int D>
@@ -519,12 +572,12 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
-  const uint32_t sQ = base, sDO = base + SM::kQTile, sK = base + 2 * SM::kQTile, sV = sK + SM::kKTile;
-  const uint32_t bars = sV + SM::kKTile;
-  const uint32_t bar_q = bars, bar_k = bars + 8, bar_v = bars + 16, bar_s = bars + 24, bar_p = bars + 32,
-                 bar_pv = bars + 40, tmem_slot = bars + 48;
-  volatile uint32_t* tmem_slot_ptr =
-      reinterpret_cast<volatile uint32_t*>(gen + 2 * SM::kQTile + 2 * SM::kKTile + 48);
+  constexpr int kSt = SM::kStages;
+  const uint32_t sQ = base, sDO = base + SM::kQTile, sK0 = base + 2 * SM::kQTile /* + stage * kKTile */, sV0 = sK0 + kSt * SM::kKTile;
+  const uint32_t bars = base + SM::kOffBars;
+  const uint32_t bar_q = bars, bar_s = bars + 8, bar_p = bars + 16, bar_fin = bars + 24, tmem_slot = bars + 32;
+  const uint32_t full_k = bars + 40, full_v = full_k + 8 * kSt, empty_k = full_v + 8 * kSt, empty_v = empty_k + 8 * kSt;
+  volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen + SM::kOffBars + 32);
 
   const int warp = threadIdx.x >> 5;
   const int h = blockIdx.y, b = blockIdx.z, hk = h / (Hq / Hkv);
@@ -557,11 +610,10 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
 
   if (threadIdx.x == 0) {
     mbar_init(bar_q, 1);
-    mbar_init(bar_k, 1);
-    mbar_init(bar_v, 1);
+    for (int i = 0; i < 4 * kSt; ++i) mbar_init(full_k + 8 * i, 1);
     mbar_init(bar_s, 1);
     mbar_init(bar_p, 4);
-    mbar_init(bar_pv, 1);
+    mbar_init(bar_fin, 1);
     mbar_fence_init();
   }
   if (warp == 5) tmem_alloc(tmem_slot, 256);
@@ -569,7 +621,8 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
-  const uint32_t t_S = tmem, t_dP = tmem + 64, t_dQ = tmem + 128;
+  const uint32_t t_S0 = tmem /* + 64 * S buffer */, t_dP = tmem + 64 * SM::kSBufs, t_dQ = t_dP + 64;
+  static_assert(64 * (SM::kSBufs + 1) + D <= 256, "tensor memory of a block");
   bool ok = true;
 
   if (warp == 4) {
@@ -587,16 +640,19 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
         key_tile(j, sg, idx);
         const CUtensorMap* mk = sg == kSegRaw ? &tm_k_raw : (sg == kSegGist ? &tm_k_gist : &tm_k_sink);
         const CUtensorMap* mv = sg == kSegRaw ? &tm_v_raw : (sg == kSegGist ? &tm_v_gist : &tm_v_sink);
-        if (j > 0) ok = mbar_wait(bar_s, (j - 1) & 1);  // dP(j-1) done: V buffer free
+        const int st = j % kSt, ph = (j / kSt - 1) & 1;
+        if (j >= kSt) ok = mbar_wait(empty_v + 8 * st, ph);  // dP of step j - kSt done
         if (!ok) break;
-        mbar_arrive_expect_tx(bar_v, SM::kKTile);
+        mbar_arrive_expect_tx(full_v + 8 * st, SM::kKTile);
 #pragma unroll
-        for (int sl = 0; sl < D / 64; ++sl) tma_load_4d(sV + sl * SM::kKSlab, mv, bar_v, sl * 64, hk, idx * DQ_BN, b);
-        if (j > 0) ok = mbar_wait(bar_pv, (j - 1) & 1);  // dQ MMA (j-1) done: K buffer free
+        for (int sl = 0; sl < D / 64; ++sl)
+          tma_load_4d(sV0 + st * SM::kKTile + sl * SM::kKSlab, mv, full_v + 8 * st, sl * 64, hk, idx * DQ_BN, b);
+        if (j >= kSt) ok = mbar_wait(empty_k + 8 * st, ph);  // dQ of step j - kSt done
         if (!ok) break;
-        mbar_arrive_expect_tx(bar_k, SM::kKTile);
+        mbar_arrive_expect_tx(full_k + 8 * st, SM::kKTile);
 #pragma unroll
-        for (int sl = 0; sl < D / 64; ++sl) tma_load_4d(sK + sl * SM::kKSlab, mk, bar_k, sl * 64, hk, idx * DQ_BN, b);
+        for (int sl = 0; sl < D / 64; ++sl)
+          tma_load_4d(sK0 + st * SM::kKTile + sl * SM::kKSlab, mk, full_k + 8 * st, sl * 64, hk, idx * DQ_BN, b);
       }
       if (!ok) atomicExch(&g_bwd_timeout, 1u);
     }
@@ -605,31 +661,54 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       const uint32_t leader = elect_one();
       constexpr uint32_t idesc_s = make_idesc_bf16(DQ_BM, DQ_BN, false, false);
       constexpr uint32_t idesc_dq = make_idesc_bf16(DQ_BM, D, false, true);
-      ok = mbar_wait_warp(bar_q, 0);
-      for (int j = 0; j < nt && ok; ++j) {
-        ok = mbar_wait_warp(bar_k, j & 1) && mbar_wait_warp(bar_v, j & 1);
-        if (!ok) break;
+      auto issue_S = [&](int j) {
+        const int st = j % kSt;
+        if (!mbar_wait_warp(full_k + 8 * st, (j / kSt) & 1)) return false;
         tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t qoff = (kk / 4) * SM::kQSlab + (kk % 4) * 32, koff = (kk / 4) * SM::kKSlab + (kk % 4) * 32;
-          umma_ss(leader, t_S, make_smem_desc(sQ + qoff, 16, 1024), make_smem_desc(sK + koff, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_S0 + 64 * (j % SM::kSBufs), make_smem_desc(sQ + qoff, 16, 1024),
+                  make_smem_desc(sK0 + st * SM::kKTile + koff, 16, 1024), idesc_s, kk > 0);
         }
+        return true;
+      };
+      auto issue_dP = [&](int j) {  // completes the step's inputs: its S went before
+        const int st = j % kSt;
+        if (!mbar_wait_warp(full_v + 8 * st, (j / kSt) & 1)) return false;
+        tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint32_t qoff = (kk / 4) * SM::kQSlab + (kk % 4) * 32, koff = (kk / 4) * SM::kKSlab + (kk % 4) * 32;
-          umma_ss(leader, t_dP, make_smem_desc(sDO + qoff, 16, 1024), make_smem_desc(sV + koff, 16, 1024), idesc_s, kk > 0);
+          umma_ss(leader, t_dP, make_smem_desc(sDO + qoff, 16, 1024), make_smem_desc(sV0 + st * SM::kKTile + koff, 16, 1024),
+                  idesc_s, kk > 0);
         }
         umma_commit(leader, bar_s);
-        ok = mbar_wait_warp(bar_p, j & 1);
+        umma_commit(leader, empty_v + 8 * st);
+        return true;
+      };
+      ok = mbar_wait_warp(bar_q, 0) && issue_S(0);  // (every query row sees a key: nt > 0)
+      ok = ok && issue_dP(0);
+      for (int j = 0; j < nt && ok; ++j) {
+        const int st = j % kSt;
+        const bool has_next = j + 1 < nt;
+        if (SM::kSBufs == 2 && has_next) ok = issue_S(j + 1);  // runs under the softmax of step j
+        ok = ok && mbar_wait_warp(bar_p, j & 1);
         if (!ok) break;
         tc_fence_after();
+        if (SM::kSBufs == 2 && has_next) ok = issue_dP(j + 1);  // what the softmax waits for goes before dQ
+        if (!ok) break;
 #pragma unroll
         for (int kk = 0; kk < DQ_BN / 16; ++kk)
-          umma_ts(leader, t_dQ, t_S + kk * 8, make_smem_desc(sK + kk * 2048, SM::kKSlab, 1024), idesc_dq,
-                  (j > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(leader, bar_pv);
+          umma_ts(leader, t_dQ, t_S0 + 64 * (j % SM::kSBufs) + kk * 8,
+                  make_smem_desc(sK0 + st * SM::kKTile + kk * 2048, SM::kKSlab, 1024), idesc_dq, (j > 0 || kk > 0) ? 1u : 0u);
+        umma_commit(leader, empty_k + 8 * st);
+        if (SM::kSBufs == 1 && has_next) {
+          ok = issue_S(j + 1);
+          ok = ok && issue_dP(j + 1);
+        }
       }
+      if (ok) umma_commit(leader, bar_fin);
       if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
     }
   } else {
@@ -663,6 +742,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       ok = mbar_wait_warp(bar_s, j & 1);
       if (!ok) break;
       tc_fence_after();
+      const uint32_t t_S = t_S0 + 64 * (j % SM::kSBufs);
 #pragma unroll
       for (int c = 0; c < DQ_BN / 32; ++c) {
         uint32_t sv[32], dv_[32];
@@ -689,7 +769,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       tc_fence_before();
       mbar_arrive_warp(bar_p);
     }
-    if (ok) ok = mbar_wait_warp(bar_pv, (nt - 1) & 1);
+    if (ok) ok = mbar_wait_warp(bar_fin, 0);
     if (ok) {
       tc_fence_after();
       const long long tok = (long long)b * g.N + q_base + row_a + r_in_tile;
@@ -1565,9 +1645,11 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
   if (e != cudaSuccess) return fail(UNIGIST_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   {
     KernelScope ks("attn_bwd_dkdv_sm100_kernel", st);
-    attn_bwd_dkdv_sm100_kernel<D><<<dim3(n_tiles, Hkv, B), kKvThreads, KvSmem<D>::kBytes, st>>>(
+    const int pairs = B * Hkv, n_heavy = n_sink_t + n_gist_t;
+    attn_bwd_dkdv_sm100_kernel<D><<<n_tiles * pairs, kKvThreads, KvSmem<D>::kBytes, st>>>(
         mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
-        (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t);
+        (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, make_fastdiv(n_heavy),
+        make_fastdiv(n_raw_t), make_fastdiv(Hkv));
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {
