@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256)
 bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, int D, long long tokens,
                 const void* __restrict__ d_o, const __nv_bfloat16* __restrict__ o,
                 __nv_bfloat16* __restrict__ d_o_bf16, float* __restrict__ dq32) {
+  pdl_begin();
   constexpr int kHeads = 4;  // rows in flight
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -258,6 +259,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     mbar_fence_init();
   }
   if (warp == 9) tmem_alloc(tmem_slot, 512);
+  pdl_begin();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -617,6 +619,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     mbar_fence_init();
   }
   if (warp == 5) tmem_alloc(tmem_slot, 256);
+  pdl_begin();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1012,6 +1015,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
     mbar_fence_init();
   }
   if (warp == kFuMmaWarp) tmem_alloc(tmem_slot, 512);
+  pdl_begin();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1421,6 +1425,7 @@ __global__ void __launch_bounds__(128)
 dkdv_reduce_kernel(Geom g, int interleaved, int Hkv, int n_sink_kt, int n_gist_kt, int n_chunks, int chunk_tiles,
                    const float* __restrict__ partial, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
                    float scale) {
+  pdl_begin();
   const int rank = blockIdx.x >> 3, row0 = (blockIdx.x & 7) * 16, hk = blockIdx.y, b = blockIdx.z;
   const int n_heavy_kt = n_sink_kt + n_gist_kt;
   const int kseg = rank < n_sink_kt ? kSegSink : kSegGist;
@@ -1453,6 +1458,7 @@ template <int kRuns>
 __global__ void __launch_bounds__(256)
 dq_convert_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, long long tokens,
                   const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, float scale) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -1512,12 +1518,8 @@ int32_t launch_prep(const TokRuns<kRuns>& T, const unigist_problem& p, long long
   const int blocks = (int)((tokens + 7) / 8 < sm_count() * 16 ? (tokens + 7) / 8 : sm_count() * 16);
   {
     KernelScope ks("bwd_prep_kernel", st);
-    if (f32)
-      bwd_prep_kernel<true, kRuns><<<blocks, 256, 0, st>>>(T, il, p.num_q_heads, p.head_dim, tokens, d_o,
-                                                           (const __nv_bfloat16*)o, sc.do_bf16, sc.dq32);
-    else
-      bwd_prep_kernel<false, kRuns><<<blocks, 256, 0, st>>>(T, il, p.num_q_heads, p.head_dim, tokens, d_o,
-                                                            (const __nv_bfloat16*)o, nullptr, sc.dq32);
+    launch_chained(f32 ? bwd_prep_kernel<true, kRuns> : bwd_prep_kernel<false, kRuns>, dim3(blocks), 256, 0, st, 1, T, il,
+                   p.num_q_heads, p.head_dim, tokens, d_o, (const __nv_bfloat16*)o, sc.do_bf16, sc.dq32);
   }
   return check_launch("backward prep kernel");
 }
@@ -1528,7 +1530,7 @@ int32_t launch_convert(const TokRuns<kRuns>& T, const unigist_problem& p, long l
   const int blocks = (int)((tokens + 7) / 8 < sm_count() * 16 ? (tokens + 7) / 8 : sm_count() * 16);
   {
     KernelScope ks("dq_convert_kernel", st);
-    dq_convert_kernel<kRuns><<<blocks, 256, 0, st>>>(T, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_q_heads, tokens,
+    launch_chained(dq_convert_kernel<kRuns>, dim3(blocks), 256, 0, st, 1, T, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_q_heads, tokens,
                                                      sc.dq32, (__nv_bfloat16*)dq, scale);
   }
   return check_launch("dQ convert kernel");
@@ -1599,8 +1601,7 @@ int32_t launch_fused(const BwdRuns<kRuns>& P, dim3 grid, const unigist_problem& 
   if (e != cudaSuccess) return fail(UNIGIST_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   {
     KernelScope ks("attn_bwd_fused_sm100_kernel", st);
-    attn_bwd_fused_sm100_kernel<kRuns><<<grid, kFuThreads, FuSmem::kBytes, st>>>(
-        P, p.num_q_heads, p.num_kv_heads, scale, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, make_fastdiv(p.ratio));
+    launch_chained(attn_bwd_fused_sm100_kernel<kRuns>, grid, kFuThreads, FuSmem::kBytes, st, 1, P, p.num_q_heads, p.num_kv_heads, scale, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, make_fastdiv(p.ratio));
   }
   return check_launch("tcgen05 fused backward kernel");
 }
@@ -1610,8 +1611,7 @@ int32_t launch_dkdv_reduce(const BwdRun& R, int batch, const unigist_problem& p,
   if (R.n_chunks <= 1) return UNIGIST_OK;
   {
     KernelScope ks("dkdv_reduce_kernel", st);
-    dkdv_reduce_kernel<<<dim3((R.n_sink_kt + R.n_gist_kt) * 8, p.num_kv_heads, batch), 128, 0, st>>>(
-        R.g, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_kv_heads, R.n_sink_kt, R.n_gist_kt, R.n_chunks,
+    launch_chained(dkdv_reduce_kernel, dim3((R.n_sink_kt + R.n_gist_kt) * 8, p.num_kv_heads, batch), 128, 0, st, 1, R.g, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_kv_heads, R.n_sink_kt, R.n_gist_kt, R.n_chunks,
         R.chunk_tiles, R.partial, R.dk, R.dv, scale);
   }
   return check_launch("dK/dV reduce kernel");
@@ -1646,16 +1646,14 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
   {
     KernelScope ks("attn_bwd_dkdv_sm100_kernel", st);
     const int pairs = B * Hkv, n_heavy = n_sink_t + n_gist_t;
-    attn_bwd_dkdv_sm100_kernel<D><<<n_tiles * pairs, kKvThreads, KvSmem<D>::kBytes, st>>>(
-        mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
+    launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(n_tiles * pairs), kKvThreads, KvSmem<D>::kBytes, st, 1, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
         (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, make_fastdiv(n_heavy),
         make_fastdiv(n_raw_t), make_fastdiv(Hkv));
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {
     KernelScope ks("attn_bwd_dq_sm100_kernel", st);
-    attn_bwd_dq_sm100_kernel<D><<<dim3(n_tiles, Hq, B), kDqThreads, DqSmem<D>::kBytes, st>>>(
-        mq[0], mq[1], mq[2], md[0], md[1], md[2], mk64[0], mk64[1], mk64[2], mv64[0], mv64[1], mv64[2], g, Hq, Hkv, scale,
+    launch_chained(attn_bwd_dq_sm100_kernel<D>, dim3(n_tiles, Hq, B), kDqThreads, DqSmem<D>::kBytes, st, 1, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk64[0], mk64[1], mk64[2], mv64[0], mv64[1], mv64[2], g, Hq, Hkv, scale,
         lse, delta, (__nv_bfloat16*)dq, n_sink_t, n_raw_t);
   }
   return check_launch("tcgen05 dQ kernel");

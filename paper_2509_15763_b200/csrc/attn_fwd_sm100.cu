@@ -334,6 +334,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
     mbar_fence_init();
   }
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  pdl_begin();  // nothing above touches global memory
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -770,8 +771,8 @@ int32_t go_fwd(Kern kern, size_t smem, dim3 grid, const Params& P, const unigist
   if (e != cudaSuccess) return fail(UNIGIST_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   {
     KernelScope ks("attn_fwd_sm100_kernel", st);
-    kern<<<grid, kThreads, smem, st>>>(P, Hq, make_fastdiv(p.ratio), make_fastdiv(pair ? (Hq / Hkv) / 2 : Hq / Hkv),
-                                       scale * 1.4426950408889634f, pair, il ? 1 : 0);
+    launch_chained(kern, grid, kThreads, smem, st, 1, P, Hq, make_fastdiv(p.ratio),
+                   make_fastdiv(pair ? (Hq / Hkv) / 2 : Hq / Hkv), scale * 1.4426950408889634f, pair, il ? 1 : 0);
   }
   return check_launch("tcgen05 forward kernel");
 }

@@ -20,6 +20,7 @@ compact_gather_kernel(Geom g, int B, int Hkv, int vecs, int L, const uint4* __re
                       const uint4* __restrict__ v, uint4* __restrict__ kc, uint4* __restrict__ vc,
                       int num_blocks, const int32_t* __restrict__ table, int max_blocks,
                       int32_t* __restrict__ seq_lens, int32_t* __restrict__ kept_idx, int interleaved) {
+  pdl_begin();
   const long long per_tok = (long long)Hkv * vecs;
   const long long total = (long long)B * L * per_tok;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -46,6 +47,7 @@ compact_gather_kernel(Geom g, int B, int Hkv, int vecs, int L, const uint4* __re
 // In place, aligned segments: only the block table changes.
 __global__ void compact_edit_table_kernel(Geom g, int L, int32_t* __restrict__ table, int max_blocks,
                                           int32_t* __restrict__ seq_lens, int32_t* __restrict__ kept_idx) {
+  pdl_begin();
   extern __shared__ int32_t old_row[];
   const int b = blockIdx.x;
   const int nbN = g.N / PG, nbL = L / PG;
@@ -74,6 +76,7 @@ compact_stage_kernel(Geom g, int B, int Hkv, int vecs, int L, uint4* __restrict_
                      uint4* __restrict__ vc, int num_blocks, const int32_t* __restrict__ table,
                      int max_blocks, uint4* __restrict__ stage, int32_t* __restrict__ seq_lens,
                      int32_t* __restrict__ kept_idx) {
+  pdl_begin();
   const long long per_tok = (long long)Hkv * vecs;
   const long long total = (long long)B * L * per_tok;
   uint4* stage_v = stage + total;
@@ -117,8 +120,7 @@ int32_t launch_compact_gather(const Geom& g, const unigist_problem& p, const voi
   const long long total = (long long)p.batch * L * p.num_kv_heads * vecs;
   {
     KernelScope ks("compact_gather_kernel", st);
-    compact_gather_kernel<<<grid_for(total), 256, 0, st>>>(
-        g, p.batch, p.num_kv_heads, vecs, L, (const uint4*)k, (const uint4*)v, (uint4*)kc, (uint4*)vc,
+    launch_chained(compact_gather_kernel, dim3(grid_for(total)), 256, 0, st, 1, g, p.batch, p.num_kv_heads, vecs, L, (const uint4*)k, (const uint4*)v, (uint4*)kc, (uint4*)vc,
         num_blocks, table, max_blocks, seq_lens, kept_idx, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0);
   }
   return check_launch("compaction gather kernel");
@@ -138,22 +140,20 @@ int32_t launch_compact_inplace(const Geom& g, const unigist_problem& p, void* kc
     }
     {
       KernelScope ks("compact_edit_table_kernel", st);
-      compact_edit_table_kernel<<<p.batch, 256, smem, st>>>(g, L, table, max_blocks, seq_lens, kept_idx);
+      launch_chained(compact_edit_table_kernel, dim3(p.batch), 256, smem, st, 1, g, L, table, max_blocks, seq_lens, kept_idx);
     }
     return check_launch("compaction table edit kernel");
   }
   const long long total = (long long)p.batch * L * p.num_kv_heads * vecs;
   {
     KernelScope ks("compact_stage_kernel", st);
-    compact_stage_kernel<false><<<grid_for(total), 256, 0, st>>>(
-        g, p.batch, p.num_kv_heads, vecs, L, (uint4*)kc, (uint4*)vc, num_blocks, table, max_blocks,
+    launch_chained(compact_stage_kernel<false>, dim3(grid_for(total)), 256, 0, st, 1, g, p.batch, p.num_kv_heads, vecs, L, (uint4*)kc, (uint4*)vc, num_blocks, table, max_blocks,
         (uint4*)ws, seq_lens, kept_idx);
   }
   if (int32_t rc = check_launch("compaction staging kernel")) return rc;
   {
     KernelScope ks("compact_writeback_kernel", st);
-    compact_stage_kernel<true><<<grid_for(total), 256, 0, st>>>(
-        g, p.batch, p.num_kv_heads, vecs, L, (uint4*)kc, (uint4*)vc, num_blocks, table, max_blocks,
+    launch_chained(compact_stage_kernel<true>, dim3(grid_for(total)), 256, 0, st, 1, g, p.batch, p.num_kv_heads, vecs, L, (uint4*)kc, (uint4*)vc, num_blocks, table, max_blocks,
         (uint4*)ws, seq_lens, kept_idx);
   }
   return check_launch("compaction write-back kernel");

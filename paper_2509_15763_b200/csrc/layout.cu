@@ -6,6 +6,7 @@ namespace ug {
 
 __global__ void layout_kernel(Geom g, int32_t* __restrict__ sp, int32_t* __restrict__ up,
                               int32_t* __restrict__ pos) {
+  pdl_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += gridDim.x * blockDim.x) {
     if (sp) sp[i] = shift_perm(g, i);
     const int sig = unshift_perm(g, i);
@@ -20,7 +21,7 @@ int32_t launch_layout(const Geom& g, int32_t* sp, int32_t* up, int32_t* pos, cud
   if (blocks > sm_count() * 8) blocks = sm_count() * 8;
   {
     KernelScope ks("layout_kernel", st);
-    layout_kernel<<<blocks, threads, 0, st>>>(g, sp, up, pos);
+    launch_chained(layout_kernel, dim3(blocks), threads, 0, st, 1, g, sp, up, pos);
   }
   return check_launch("layout kernel");
 }
@@ -32,6 +33,7 @@ template <bool kInverse>
 __global__ void __launch_bounds__(256)
 shift_rows_kernel(Geom g, const uint4* __restrict__ src, uint4* __restrict__ dst, int vecs,
                   long long rows) {
+  pdl_begin();
   constexpr int kRows = 4, kVec = 4;  // up to kRows * kVec loads in flight per lane
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -73,10 +75,8 @@ int32_t launch_shift(const Geom& g, int B, const void* src, void* dst, size_t ro
   const int blocks = (int)(want < cap ? (want > 0 ? want : 1) : cap);
   {
     KernelScope ks(inverse ? "unshift_rows_kernel" : "shift_rows_kernel", st);
-    if (inverse)
-      shift_rows_kernel<true><<<blocks, 256, 0, st>>>(g, (const uint4*)src, (uint4*)dst, vecs, rows);
-    else
-      shift_rows_kernel<false><<<blocks, 256, 0, st>>>(g, (const uint4*)src, (uint4*)dst, vecs, rows);
+    launch_chained(inverse ? shift_rows_kernel<true> : shift_rows_kernel<false>, dim3(blocks), 256, 0, st, 1, g,
+                   (const uint4*)src, (uint4*)dst, vecs, rows);
   }
   return check_launch("gist shift kernel");
 }

@@ -21,6 +21,7 @@ prefill_gather_kernel(int B, int Hkv, int vecs, int s, int u0, int w0, int c_raw
                       const uint4* __restrict__ kc, const uint4* __restrict__ vc, int num_blocks,
                       const int32_t* __restrict__ table, int max_blocks, const uint4* __restrict__ k_chunk,
                       const uint4* __restrict__ v_chunk, uint4* __restrict__ k_ctx, uint4* __restrict__ v_ctx) {
+  pdl_begin();
   const int Tc = w0 + c_raw, n_ctx = s + Tc + u0 + c_gists;
   const int sq = u0 == 0 ? s : 0, n_chunk = sq + c_raw + c_gists;
   const long long per_tok = (long long)Hkv * vecs;
@@ -84,7 +85,7 @@ int32_t launch_prefill_chunk(const unigist_problem& p, const Geom& g_full, float
     const long long cap = (long long)sm_count() * 16;
     const int blocks = (int)(want < cap ? want : cap);
     KernelScope ks("prefill_gather_kernel", st);
-    prefill_gather_kernel<<<blocks, 256, 0, st>>>(B, Hkv, vecs, s, u0, w0, c_raw, c, (const uint4*)kc, (const uint4*)vc,
+    launch_chained(prefill_gather_kernel, dim3(blocks), 256, 0, st, 1, B, Hkv, vecs, s, u0, w0, c_raw, c, (const uint4*)kc, (const uint4*)vc,
                                                   num_blocks, table, max_blocks, (const uint4*)k, (const uint4*)v, k_ctx,
                                                   v_ctx);
   }

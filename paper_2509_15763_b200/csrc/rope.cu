@@ -31,6 +31,7 @@ rope_kernel(Geom g, long long tokens, int heads, double log2_theta, int to_shift
   double inv_freq[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) inv_freq[e] = exp2(-2.0 * (j0 + e) / D * log2_theta);
+  pdl_begin();
   for (long long tk = warp; tk < tokens; tk += nwarps) {  // tk = b * N + t, t interleaved
     const long long b = tk / g.N;
     const int t = (int)(tk - b * g.N);
@@ -98,12 +99,8 @@ int32_t launch_rope(const Geom& g, int B, int heads, int D, float theta_base, bo
   const double log2_theta = log2((double)theta_base);
   {
     KernelScope ks("rope_kernel", st);
-    if (D == 128)
-      rope_kernel<128><<<blocks, 256, 0, st>>>(g, tokens, heads, log2_theta, to_shifted ? 1 : 0, from_shifted ? 1 : 0, inverse ? 1 : 0,
-                                                 (const __nv_bfloat16*)src, (__nv_bfloat16*)dst);
-    else
-      rope_kernel<64><<<blocks, 256, 0, st>>>(g, tokens, heads, log2_theta, to_shifted ? 1 : 0, from_shifted ? 1 : 0, inverse ? 1 : 0,
-                                                (const __nv_bfloat16*)src, (__nv_bfloat16*)dst);
+    launch_chained(D == 128 ? rope_kernel<128> : rope_kernel<64>, dim3(blocks), 256, 0, st, 1, g, tokens, heads, log2_theta,
+                   to_shifted ? 1 : 0, from_shifted ? 1 : 0, inverse ? 1 : 0, (const __nv_bfloat16*)src, (__nv_bfloat16*)dst);
   }
   return check_launch("rope kernel");
 }
