@@ -32,9 +32,13 @@ __device__ unsigned int g_bwd_timeout = 0;
 // and a warp finds its token's run by scanning the (at most twelve) first-token indices.
 struct TokRun {
   Geom g;
+  FastDiv n_div, unit_div, r_div;  // by N, r + 1, r
   long long tok_begin;
   float* delta;
 };
+TokRun make_tok_run(const Geom& g, long long tok_begin, float* delta) {
+  return {g, make_fastdiv(g.N), make_fastdiv(g.r + 1), make_fastdiv(g.r), tok_begin, delta};
+}
 template <int kRuns>
 struct TokRuns {
   TokRun run[kRuns];
@@ -42,74 +46,71 @@ struct TokRuns {
 };
 
 
-// Delta and dO conversion: one warp per token.  The token's batch index and shifted position are worked out
-// once (the divisions cost more than a row's loads), then its Hq rows go by four at a time, all loads of the
-// four issued before the first use; 4 elements per lane and pass.
-template <bool kF32, int kRuns>
+// Delta and dO conversion: one warp per token.  Bound by HBM: reads dO and O, writes zeros for the dQ accumulator, which
+// is 8 bytes an element in all.  The token's batch index and shifted position are worked out once, by multiplication;
+// its Hq rows then go by in 16-byte pieces, D / 8 lanes to a row, kSteps rows (times the rows a warp covers at once) of dO
+// and O in flight before the first use.
+template <bool kF32, int kRuns, int D>
 __global__ void __launch_bounds__(256)
-bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, int D, long long tokens,
-                const void* __restrict__ d_o, const __nv_bfloat16* __restrict__ o,
-                __nv_bfloat16* __restrict__ d_o_bf16, float* __restrict__ dq32) {
+bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, int tokens, const void* __restrict__ d_o,
+                const __nv_bfloat16* __restrict__ o, __nv_bfloat16* __restrict__ d_o_bf16, float* __restrict__ dq32) {
   pdl_begin();
-  constexpr int kHeads = 4;  // rows in flight
-  const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  constexpr int kLanes = D / 8, kRows = 32 / kLanes, kSteps = 4;  // lanes of a row, rows of a warp access
+  const int lane = threadIdx.x & 31, sub = lane / kLanes, col = (lane % kLanes) * 8;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
   for (long long tk = warp; tk < tokens; tk += nwarps) {  // tk = packed token index (run's first token + b * N + t)
     int ri = 0;
     if constexpr (kRuns > 1)
       while (ri + 1 < P.n && tk >= P.run[ri + 1].tok_begin) ++ri;
-    const Geom g = P.run[ri].g;
-    const long long local = tk - P.run[ri].tok_begin;
-    const long long b = local / g.N;
-    const int t = (int)(local - b * g.N);
-    // Delta is kept in shifted order, whatever the order of dO and O
-    float* delta_tok = P.run[ri].delta + b * Hq * g.N + (interleaved ? unshift_perm(g, t) : t);
+    const TokRun& R = P.run[ri];
+    const int N = R.g.N, local = (int)(tk - R.tok_begin);
+    const int b = fdiv(R.n_div, local), t = local - b * N;
+    int pos = t;  // Delta is kept in shifted order, whatever the order of dO and O
+    if (interleaved && t >= R.g.s) {
+      const int q = t - R.g.s, u = fdiv(R.unit_div, q), in_unit = q - u * (R.g.r + 1);
+      pos = in_unit == R.g.r ? R.g.s + R.g.T + u : R.g.s + u * R.g.r + in_unit;
+    }
+    float* delta_tok = R.delta + (long long)b * Hq * N + pos;
     const long long row0 = tk * Hq;
-    for (int h0 = 0; h0 < Hq; h0 += kHeads) {
-      float acc[kHeads];
+    for (int h0 = 0; h0 < Hq; h0 += kRows * kSteps) {
+      uint4 db[kSteps], ob[kSteps];  // 8 bf16 of dO and of O
 #pragma unroll
-      for (int u = 0; u < kHeads; ++u) acc[u] = 0.f;
-      for (int d = lane * 4; d < D; d += 128) {
-        uint2 dbits[kHeads], obits[kHeads];  // 4 bf16 of dO and of O
-#pragma unroll
-        for (int u = 0; u < kHeads; ++u) {
-          if (h0 + u >= Hq) continue;
-          const long long at = (row0 + h0 + u) * D + d;
-          if (kF32) {
-            const float4 x = __ldcs(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(d_o) + at));
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x, x.y), hi = __floats2bfloat162_rn(x.z, x.w);
-            dbits[u].x = *reinterpret_cast<const uint32_t*>(&lo);
-            dbits[u].y = *reinterpret_cast<const uint32_t*>(&hi);
-          } else {
-            dbits[u] = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(d_o) + at);
-          }
-          obits[u] = *reinterpret_cast<const uint2*>(o + at);
+      for (int u = 0; u < kSteps; ++u) {
+        const int h = h0 + u * kRows + sub;
+        if (h >= Hq) continue;
+        const long long at = (row0 + h) * D + col;
+        if (kF32) {
+          const float4 x = __ldcs(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(d_o) + at));
+          const float4 y = __ldcs(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(d_o) + at) + 1);
+          db[u] = make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
+        } else {
+          db[u] = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(d_o) + at);
         }
+        ob[u] = *reinterpret_cast<const uint4*>(o + at);
+      }
+      // the fused backward accumulates dQ into this fp32 buffer: start it at zero
+      if (dq32) {
+        const int n4 = min(kRows * kSteps, Hq - h0) * (D / 4);
+        float4* z = reinterpret_cast<float4*>(dq32 + (row0 + h0) * D);
 #pragma unroll
-        for (int u = 0; u < kHeads; ++u) {
-          if (h0 + u >= Hq) continue;
-          const long long at = (row0 + h0 + u) * D + d;
-          // the fused backward accumulates dQ into this fp32 buffer: start it at zero
-          if (dq32) __stcs(reinterpret_cast<float4*>(dq32 + at), make_float4(0.f, 0.f, 0.f, 0.f));
-          if (kF32) *reinterpret_cast<uint2*>(d_o_bf16 + at) = dbits[u];
-          // a bf16 is the high half of an fp32
-          acc[u] += __uint_as_float(dbits[u].x << 16) * __uint_as_float(obits[u].x << 16) +
-                    __uint_as_float(dbits[u].x & 0xffff0000u) * __uint_as_float(obits[u].x & 0xffff0000u) +
-                    __uint_as_float(dbits[u].y << 16) * __uint_as_float(obits[u].y << 16) +
-                    __uint_as_float(dbits[u].y & 0xffff0000u) * __uint_as_float(obits[u].y & 0xffff0000u);
-        }
+        for (int i = 0; i < kRows * kSteps * (D / 4) / 32; ++i)
+          if (i * 32 + lane < n4) __stcs(z + i * 32 + lane, make_float4(0.f, 0.f, 0.f, 0.f));
       }
 #pragma unroll
-      for (int u = 0; u < kHeads; ++u) {
+      for (int u = 0; u < kSteps; ++u) {
+        const int h = h0 + u * kRows + sub;
+        float acc = 0.f;
+        if (h < Hq) {
+          if (kF32) *reinterpret_cast<uint4*>(d_o_bf16 + (row0 + h) * D + col) = db[u];
+          const uint32_t x[4] = {db[u].x, db[u].y, db[u].z, db[u].w}, y[4] = {ob[u].x, ob[u].y, ob[u].z, ob[u].w};
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], off);
-      }
-      if (lane < kHeads && h0 + lane < Hq) {
-        float mine = acc[0];
+          for (int e = 0; e < 4; ++e)  // a bf16 is the high half of an fp32
+            acc += __uint_as_float(x[e] << 16) * __uint_as_float(y[e] << 16) +
+                   __uint_as_float(x[e] & 0xffff0000u) * __uint_as_float(y[e] & 0xffff0000u);
+        }
 #pragma unroll
-        for (int u = 1; u < kHeads; ++u) mine = lane == u ? acc[u] : mine;
-        delta_tok[(long long)(h0 + lane) * g.N] = mine;
+        for (int off = kLanes / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (h < Hq && lane % kLanes == 0) delta_tok[(long long)h * N] = acc;
       }
     }
   }
@@ -1466,11 +1467,15 @@ dq_convert_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int
     int ri = 0;
     if constexpr (kRuns > 1)
       while (ri + 1 < P.n && tk >= P.run[ri + 1].tok_begin) ++ri;
-    const Geom g = P.run[ri].g;
-    const long long local = tk - P.run[ri].tok_begin;
-    const long long b = local / g.N;
-    const int sigma = (int)(local - b * g.N);
-    const long long out_tk = P.run[ri].tok_begin + b * g.N + (interleaved ? shift_perm(g, sigma) : sigma);
+    const TokRun& R = P.run[ri];
+    const Geom& g = R.g;
+    const int local = (int)(tk - R.tok_begin), b = fdiv(R.n_div, local), sigma = local - b * g.N;
+    int row = sigma;
+    if (interleaved && sigma >= g.s) {
+      const int i = sigma - g.s;
+      row = i < g.T ? sigma + fdiv(R.r_div, i) : g.s + (i - g.T) * (g.r + 1) + g.r;
+    }
+    const long long out_tk = R.tok_begin + (long long)b * g.N + row;
     const float4* s4 = reinterpret_cast<const float4*>(src + tk * Hq * 128) + lane;
     uint2* d2 = reinterpret_cast<uint2*>(dst + out_tk * Hq * 128) + lane;
     for (int h0 = 0; h0 < Hq; h0 += 4) {
@@ -1518,8 +1523,10 @@ int32_t launch_prep(const TokRuns<kRuns>& T, const unigist_problem& p, long long
   const int blocks = (int)((tokens + 7) / 8 < sm_count() * 16 ? (tokens + 7) / 8 : sm_count() * 16);
   {
     KernelScope ks("bwd_prep_kernel", st);
-    launch_chained(f32 ? bwd_prep_kernel<true, kRuns> : bwd_prep_kernel<false, kRuns>, dim3(blocks), 256, 0, st, 1, T, il,
-                   p.num_q_heads, p.head_dim, tokens, d_o, (const __nv_bfloat16*)o, sc.do_bf16, sc.dq32);
+    const auto kern = p.head_dim == 128 ? (f32 ? bwd_prep_kernel<true, kRuns, 128> : bwd_prep_kernel<false, kRuns, 128>)
+                                        : (f32 ? bwd_prep_kernel<true, kRuns, 64> : bwd_prep_kernel<false, kRuns, 64>);
+    launch_chained(kern, dim3(blocks), 256, 0, st, 1, T, il, p.num_q_heads, (int)tokens, d_o, (const __nv_bfloat16*)o,
+                   sc.do_bf16, sc.dq32);
   }
   return check_launch("backward prep kernel");
 }
@@ -1691,9 +1698,7 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   const void* do_src = f32 ? static_cast<const void*>(sc.do_bf16) : d_o;
   TokRuns<1> T;
   T.n = 1;
-  T.run[0].g = g;
-  T.run[0].tok_begin = 0;
-  T.run[0].delta = delta;
+  T.run[0] = make_tok_run(g, 0, delta);
   if (int32_t rc = launch_prep(T, p, tokens, d_o, o, sc, st)) return rc;
 
   if (!fused)
@@ -1745,9 +1750,7 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
     long long ctas = 0;
     for (int i = 0; i < n; ++i) {
       const SeqRun& t = runs[first + i];
-      T.run[i].g = t.g;
-      T.run[i].tok_begin = t.first_row - tok_lo;
-      T.run[i].delta = sc.delta + t.first_row * Hq;
+      T.run[i] = make_tok_run(t.g, t.first_row - tok_lo, sc.delta + t.first_row * Hq);
       const SeqRun& r = runs[first + order[i]];
       if (int32_t rc = fill_bwd_run(&P.run[i], r.g, p, r.batch, (const char*)q + r.first_row * rq,
                                     (const char*)do_src + r.first_row * rq, (const char*)k + r.first_row * rk,
