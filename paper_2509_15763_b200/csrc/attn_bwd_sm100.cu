@@ -161,6 +161,25 @@ __device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key
   key_q_interval(g, kseg == kSegRaw, key, true, qseg == kSegRaw, lo, hi);
 }
 
+// One 32-query chunk of P^T for one key: p = 2^(s * c - lse2[q]); kMasked: bit e of `bits` says query e sees the key.
+template <bool kMasked>
+__device__ __forceinline__ void p_chunk(const uint32_t (&v)[32], const float* __restrict__ ls, float scale_log2,
+                                              uint32_t bits, float* __restrict__ p, uint32_t (&pk)[16]) {
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    const float4 l4 = *reinterpret_cast<const float4*>(ls + i);
+    const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      float x = fmaf(__uint_as_float(v[i + e]), scale_log2, -lv[e]);
+      if (kMasked) x = (bits >> (i + e)) & 1u ? x : -INFINITY;
+      p[i + e] = ex2(x);
+    }
+    pk[i / 2] = pack_bf16(p[i], p[i + 1]);
+    pk[i / 2 + 1] = pack_bf16(p[i + 2], p[i + 3]);
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
 // dK / dV kernel.  Bound by the chain scores -> P -> dP -> dS of one step, not by the tensor pipe: with head_dim 64
 // tensor memory has room for a second S buffer and shared memory for four Q / dO stages, which take the scores and the
@@ -168,7 +187,9 @@ __device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key
 // heads) took 0.70 ms before and 0.45 now.
 constexpr int KV_BM = 128;       // keys per block (TMEM lanes)
 constexpr int KV_BN = 128;       // queries per step
-constexpr int kKvThreads = 320;  // 8 compute warps, 1 TMA warp, 1 MMA warp
+// 16 compute warps (four per TMEM lane quarter, 32 query columns each: half the columns per thread shorten the chain of a
+// step), 1 TMA warp, 1 MMA warp
+constexpr int kKvCompute = 16, kKvThreads = (kKvCompute + 2) * 32;
 
 template <int D>
 struct KvSmem {
@@ -210,17 +231,22 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = Hq / Hkv;
-  // Sink and gist key tiles are seen by every later query: heaviest, and first over ALL heads and batch indices (a
-  // long walk that starts late is the kernel's tail); the tiles of one KV head are neighbours and share its Q and dO.
-  const int n_heavy = n_sink_kt + n_gist_kt;
+  // Blocks come in clusters of two.  Sink and gist key tiles are seen by every later query: heaviest, and first over ALL
+  // heads and batch indices (a long walk that starts late is the kernel's tail); the two blocks of a cluster share ONE
+  // such key tile, each walks half of its queries, and they add their dK and dV through distributed shared memory (the
+  // longest walk was 1.3 times an SM's share of all steps on the problem above).  Of the raw key tiles either block of a
+  // cluster takes one of its own.  The tiles of one KV head are neighbours and share its Q and dO.
+  const int n_heavy = n_sink_kt + n_gist_kt, crank = blockIdx.x & 1, cluster = blockIdx.x >> 1;
+  const bool split = cluster < n_heavy * pairs;
   int pair, rank;  // pair = batch index * Hkv + KV head
-  if ((int)blockIdx.x < n_heavy * pairs) {
-    pair = fdiv(heavy_div, blockIdx.x);
-    rank = blockIdx.x - pair * n_heavy;
+  if (split) {
+    pair = fdiv(heavy_div, cluster);
+    rank = cluster - pair * n_heavy;
   } else {
-    const int y = blockIdx.x - n_heavy * pairs;
+    const int y = cluster - n_heavy * pairs;
     pair = fdiv(raw_div, y);
-    rank = n_heavy + (y - pair * n_raw_kt);
+    rank = n_heavy + 2 * (y - pair * ((n_raw_kt + 1) / 2)) + crank;
+    if (rank >= n_heavy + n_raw_kt) return;  // an odd number of raw key tiles (its cluster never meets)
   }
   const int b = fdiv(hkv_div, pair), hk = pair - b * Hkv;
   const int kseg = rank < n_sink_kt ? kSegSink : (rank < n_heavy ? kSegGist : kSegRaw);
@@ -242,7 +268,10 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
   key_q_interval3(g, kseg, key_a, true, kSegSink, lo_a, hi_a);
   key_q_interval3(g, kseg, key_b, true, kSegSink, lo_b, hi_b);
   const int n_sink_q = hi_b >= lo_a ? hi_b / KV_BN - lo_a / KV_BN + 1 : 0, sq_lo = lo_a / KV_BN, sink_t_lo = lo_b, sink_t_hi = hi_a;
-  const int n_iter = (n_raw_q + n_gist_q + n_sink_q) * G;
+  // this block's part of the walk: query tiles [t_begin, t_end) in the order of the steps below
+  const int n_tiles = n_raw_q + n_gist_q + n_sink_q, t_half = (n_tiles + 1) / 2;
+  const int t_begin = split && crank ? t_half : 0, t_end = split && !crank ? t_half : n_tiles;
+  const int n_iter = (t_end - t_begin) * G;
 
   if (threadIdx.x == 0) {
     mbar_init(bar_kv, 1);
@@ -253,13 +282,13 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     mbar_init(bar_S, 1);
     mbar_init(bar_S + 8, 1);
     mbar_init(bar_dP, 1);
-    mbar_init(bar_P, 8);
-    mbar_init(bar_P + 8, 8);
-    mbar_init(bar_dS, 8);
+    mbar_init(bar_P, kKvCompute);
+    mbar_init(bar_P + 8, kKvCompute);
+    mbar_init(bar_dS, kKvCompute);
     mbar_init(bar_final, 1);
     mbar_fence_init();
   }
-  if (warp == 9) tmem_alloc(tmem_slot, 512);
+  if (warp == kKvCompute + 1) tmem_alloc(tmem_slot, 512);
   pdl_begin();
   tc_fence_before();
   __syncthreads();
@@ -291,7 +320,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     }
   };
 
-  if (warp == 8) {
+  if (warp == kKvCompute) {
     // ------------------------------------------------------------ producer: K, V once; Q, dO, LSE, Delta per step
     if (lane == 0) {
       mbar_arrive_expect_tx(bar_kv, 2 * SM::kTile);
@@ -319,7 +348,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
         st_d[i] = valid ? delta[row_base + row] : 0.f;
       }
     };
-    StepIter cur{0, 0}, ahead{0, 0};
+    StepIter cur{t_begin, 0}, ahead{t_begin, 0};
     if (n_iter > 0) fetch_stats(ahead);
     for (int it = 0; it < n_iter; ++it, advance(cur)) {
       const int st = it % kSt;
@@ -349,15 +378,15 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       if (it + 1 < n_iter) fetch_stats(ahead);
     }
     if (!ok) atomicExch(&g_bwd_timeout, 1u);
-  } else if (warp == 9) {
+  } else if (warp == kKvCompute + 1) {
     // ------------------------------------------------------------ MMA issuer
     {
       const uint32_t leader = elect_one();
       constexpr uint32_t idesc_s = make_idesc_bf16(KV_BM, KV_BN, false, false);
       constexpr uint32_t idesc_acc = make_idesc_bf16(KV_BM, D, false, true);
-      // A operand of the accumulating MMAs: bf16 pairs in TMEM; query columns [0,64) are packed at
-      // columns [0,32) of the buffer, query columns [64,128) at columns [64,96)
-      auto a_col = [](int kk) { return (kk / 4) * 64 + (kk % 4) * 8; };
+      // A operand of the accumulating MMAs: bf16 pairs in TMEM; query columns [32 h, 32 h + 32) are packed at
+      // columns [32 h, 32 h + 16) of the buffer
+      auto a_col = [](int kk) { return (kk / 2) * 32 + (kk % 2) * 8; };
       auto issue_S = [&](int it) {  // S^T of step it, once its Q (and dO) have arrived
         const int st = it % kSt, sb = it % SM::kSBufs;
         if (!mbar_wait_warp(bar_full + 8 * st, (it / kSt) & 1)) return false;
@@ -411,7 +440,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       if (!ok && leader) atomicExch(&g_bwd_timeout, 1u);
     }
   } else {
-    // ------------------------------------------------------------ compute: thread = key (TMEM lane), 64 query columns
+    // ------------------------------------------------------------ compute: thread = key (TMEM lane), 32 query columns
     const int qd = warp & 3, hf = warp >> 2;
     const int key = key_a + qd * 32 + lane;
     const bool key_valid = key <= key_b;
@@ -422,7 +451,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
     key_q_interval3(g, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
 
-    StepIter cur{0, 0};
+    StepIter cur{t_begin, 0};
     for (int it = 0; it < n_iter && ok; ++it, advance(cur)) {
       const int st = it % kSt, sb = it % SM::kSBufs;
       const uint32_t t_A = t_A0 + 128 * sb;
@@ -434,37 +463,30 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       const int t_lo = qseg == kSegRaw ? raw_t_lo : (qseg == kSegGist ? gist_t_lo : sink_t_lo);
       const int t_hi = qseg == kSegRaw ? raw_t_hi : (qseg == kSegGist ? gist_t_hi : sink_t_hi);
       const bool full = key_tile_whole && q0 >= t_lo && qb <= t_hi;
-      const int lo = (qseg == kSegRaw ? my_lo_r : (qseg == kSegGist ? my_lo_g : my_lo_s)) - q0 - 64 * hf;
-      const int hi = (qseg == kSegRaw ? my_hi_r : (qseg == kSegGist ? my_hi_g : my_hi_s)) - q0 - 64 * hf;
-      const float* ls = stats + st * 2 * KV_BN + 64 * hf;
+      const int lo = (qseg == kSegRaw ? my_lo_r : (qseg == kSegGist ? my_lo_g : my_lo_s)) - q0 - 32 * hf;
+      const int hi = (qseg == kSegRaw ? my_hi_r : (qseg == kSegGist ? my_hi_g : my_hi_s)) - q0 - 32 * hf;
+      const float* ls = stats + st * 2 * KV_BN + 32 * hf;
       const float* dl = ls + KV_BN;
       ok = mbar_wait_warp(bar_full + 8 * st, (it / kSt) & 1) && mbar_wait_warp(bar_S + 8 * sb, (it / SM::kSBufs) & 1);
       if (!ok) break;
       tc_fence_after();
-      float p[64];
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
+      float p[32];
+      {
         uint32_t v[32];
-        tmem_ld(t_A + lane_base + 64 * hf + 32 * c, v);
+        tmem_ld(t_A + lane_base + 32 * hf, v);
         tmem_wait_ld();
         uint32_t pk[16];
-#pragma unroll
-        for (int i = 0; i < 32; i += 4) {
-          const float4 l4 = *reinterpret_cast<const float4*>(ls + 32 * c + i);
-          const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float x = fmaf(__uint_as_float(v[i + e]), scale_log2, -lv[e]);
-            if (!full) {
-              const int col = 32 * c + i + e;
-              x = (col >= lo && col <= hi) ? x : -INFINITY;
-            }
-            p[32 * c + i + e] = ex2(x);
-          }
-          pk[i / 2] = pack_bf16(p[32 * c + i], p[32 * c + i + 1]);
-          pk[i / 2 + 1] = pack_bf16(p[32 * c + i + 2], p[32 * c + i + 3]);
+        // a partly visible tile: most of its 32 x 32 pieces are wholly visible all the same
+        uint32_t bits = 0xffffffffu;
+        if (!full) {
+          const int qa = max(lo, 0), qz = min(hi, 31);
+          bits = qa > qz ? 0u : ((0xffffffffu >> (31 - qz)) & (0xffffffffu << qa));
         }
-        tmem_st(t_A + lane_base + 64 * hf + 16 * c, pk);
+        if (full || __all_sync(0xffffffffu, bits == 0xffffffffu))
+          p_chunk<false>(v, ls, scale_log2, 0u, p, pk);
+        else
+          p_chunk<true>(v, ls, scale_log2, bits, p, pk);
+        tmem_st(t_A + lane_base + 32 * hf, pk);
       }
       tmem_wait_st();
       tc_fence_before();
@@ -472,71 +494,101 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       ok = mbar_wait_warp(bar_dP, it & 1);
       if (!ok) break;
       tc_fence_after();
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
+      {
         uint32_t v[32];
-        tmem_ld(t_B + lane_base + 64 * hf + 32 * c, v);
+        tmem_ld(t_B + lane_base + 32 * hf, v);
         tmem_wait_ld();
         uint32_t pk[16];
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
-          const float4 d4 = *reinterpret_cast<const float4*>(dl + 32 * c + i);
+          const float4 d4 = *reinterpret_cast<const float4*>(dl + i);
           const float dv4[4] = {d4.x, d4.y, d4.z, d4.w};
           float ds[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) ds[e] = p[32 * c + i + e] * (__uint_as_float(v[i + e]) - dv4[e]);
+          for (int e = 0; e < 4; ++e) ds[e] = p[i + e] * (__uint_as_float(v[i + e]) - dv4[e]);
           pk[i / 2] = pack_bf16(ds[0], ds[1]);
           pk[i / 2 + 1] = pack_bf16(ds[2], ds[3]);
         }
-        tmem_st(t_B + lane_base + 64 * hf + 16 * c, pk);
+        tmem_st(t_B + lane_base + 32 * hf, pk);
       }
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive_warp(bar_dS);
     }
     if (ok && n_iter > 0) ok = mbar_wait_warp(bar_final, 0);
-    if (ok) {
-      tc_fence_after();
-      const long long tok = (long long)b * g.N + key_seg_base + key;
-      // D = 128: this warp stores columns [64 hf, 64 hf + 64) of dK and of dV; D = 64: hf picks dK or dV
-      constexpr int kChunks = 2;
+    if (!ok) atomicExch(&g_bwd_timeout, 1u);
+  }
+
+  // dK and dV leave: a compute warp has its 32 keys and 32 columns of one of them (D = 64) or of both (D = 128).  Where
+  // two blocks share the key tile, block 0 finishes dK and block 1 dV: each puts its part of the other one into its
+  // (consumed) Q ring, rows of D floats with the 16-byte pieces permuted by row.
+  const int hf = warp >> 2, krow = (warp & 3) * 32 + lane;
+  const bool compute = warp < kKvCompute;
+  constexpr int kWhich = D == 128 ? 2 : 1;
+  auto is_dk_of = [&](int which) { return D == 128 ? which == 0 : hf < 2; };
+  const int col0 = D == 128 ? 32 * hf : 32 * (hf & 1);
+  auto load = [&](bool is_dk, uint32_t (&v)[32]) {
+    if (n_iter > 0) {
+      tmem_ld((is_dk ? t_dK : t_dV) + (static_cast<uint32_t>((warp & 3) * 32) << 16) + col0, v);
+      tmem_wait_ld();
+    } else {
 #pragma unroll
-      for (int which = 0; which < (D == 128 ? 2 : 1); ++which) {
-        const bool is_dk = D == 128 ? which == 0 : hf == 0;
-        const int col0 = D == 128 ? 64 * hf : 0;
-        const uint32_t tsrc = (is_dk ? t_dK : t_dV) + lane_base + col0;
-        __nv_bfloat16* dst = (is_dk ? dk : dv) + (tok * Hkv + hk) * D + col0;
-        const float mul = is_dk ? scale : 1.f;
+      for (int i = 0; i < 32; ++i) v[i] = 0u;
+    }
+  };
+  auto piece = [&](int i) { return sQ0 + krow * D * 4 + ((((col0 + i) / 4) ^ (krow & 7)) << 4); };
+  if (compute) tc_fence_after();
+  if (split) {
+    if (compute && ok) {
 #pragma unroll
-        for (int c = 0; c < kChunks; ++c) {
-          uint32_t v[32];
-          if (n_iter > 0) {
-            tmem_ld(tsrc + 32 * c, v);
-            tmem_wait_ld();
-          } else {
+      for (int which = 0; which < kWhich; ++which) {
+        if (is_dk_of(which) == (crank == 0)) continue;
+        uint32_t v[32];
+        load(is_dk_of(which), v);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = 0u;
-          }
-          if (key_valid) {
+        for (int i = 0; i < 32; i += 4) st_shared_v4(piece(i), make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]));
+      }
+    }
+    cluster_sync();
+  }
+  if (compute && ok) {
+    const int key = key_a + krow;
+    const long long tok = (long long)b * g.N + key_seg_base + key;
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint4 pk;
-              pk.x = pack_bf16(__uint_as_float(v[i]) * mul, __uint_as_float(v[i + 1]) * mul);
-              pk.y = pack_bf16(__uint_as_float(v[i + 2]) * mul, __uint_as_float(v[i + 3]) * mul);
-              pk.z = pack_bf16(__uint_as_float(v[i + 4]) * mul, __uint_as_float(v[i + 5]) * mul);
-              pk.w = pack_bf16(__uint_as_float(v[i + 6]) * mul, __uint_as_float(v[i + 7]) * mul);
-              *reinterpret_cast<uint4*>(dst + 32 * c + i) = pk;
-            }
-          }
+    for (int which = 0; which < kWhich; ++which) {
+      const bool is_dk = is_dk_of(which);
+      if (split && is_dk != (crank == 0)) continue;
+      uint32_t v[32];
+      load(is_dk, v);
+      if (split) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const float4 x = ld_cluster_v4(piece(i), crank ^ 1);
+          v[i] = __float_as_uint(__uint_as_float(v[i]) + x.x);
+          v[i + 1] = __float_as_uint(__uint_as_float(v[i + 1]) + x.y);
+          v[i + 2] = __float_as_uint(__uint_as_float(v[i + 2]) + x.z);
+          v[i + 3] = __float_as_uint(__uint_as_float(v[i + 3]) + x.w);
         }
       }
-    } else {
-      atomicExch(&g_bwd_timeout, 1u);
+      __nv_bfloat16* dst = (is_dk ? dk : dv) + (tok * Hkv + hk) * D + col0;
+      const float mul = is_dk ? scale : 1.f;
+      if (key <= key_b) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 8) {
+          uint4 pk;
+          pk.x = pack_bf16(__uint_as_float(v[i]) * mul, __uint_as_float(v[i + 1]) * mul);
+          pk.y = pack_bf16(__uint_as_float(v[i + 2]) * mul, __uint_as_float(v[i + 3]) * mul);
+          pk.z = pack_bf16(__uint_as_float(v[i + 4]) * mul, __uint_as_float(v[i + 5]) * mul);
+          pk.w = pack_bf16(__uint_as_float(v[i + 6]) * mul, __uint_as_float(v[i + 7]) * mul);
+          *reinterpret_cast<uint4*>(dst + i) = pk;
+        }
+      }
     }
   }
+  if (split) cluster_sync();  // the other block has read this one's shared memory
   tc_fence_before();
   __syncthreads();
-  if (warp == 9) {
+  if (warp == kKvCompute + 1) {
     __syncwarp();
     tmem_dealloc(tmem, 512);
   }
@@ -832,25 +884,6 @@ static_assert(kFuThreads * kFuRegsLaunch <= 65536 && kFuThreads * (kFuRegsLaunch
               "launch register count is stale");
 static_assert(2 * kFuRegsCompute + 2 * kFuRegsReadout + kFuRegsOther <= 5 * kFuRegsLaunch,
               "register split exceeds the block's allocation");
-
-// One 32-query chunk of P^T for one key: p = 2^(s * c - lse2[q]); kMasked: bit e of `bits` says query e sees the key.
-template <bool kMasked>
-__device__ __forceinline__ void fused_p_chunk(const uint32_t (&v)[32], const float* __restrict__ ls, float scale_log2,
-                                              uint32_t bits, float* __restrict__ p, uint32_t (&pk)[16]) {
-#pragma unroll
-  for (int i = 0; i < 32; i += 4) {
-    const float4 l4 = *reinterpret_cast<const float4*>(ls + i);
-    const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float x = fmaf(__uint_as_float(v[i + e]), scale_log2, -lv[e]);
-      if (kMasked) x = (bits >> (i + e)) & 1u ? x : -INFINITY;
-      p[i + e] = ex2(x);
-    }
-    pk[i / 2] = pack_bf16(p[i], p[i + 1]);
-    pk[i / 2 + 1] = pack_bf16(p[i + 2], p[i + 3]);
-  }
-}
 
 struct FuSmem {
   static constexpr int kSlab = 128 * 128;    // [128 rows x 64 bf16]
@@ -1312,11 +1345,11 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         tmem_wait_ld();
         uint32_t pk[16];
         if (full) {
-          fused_p_chunk<false>(v, ls + 32 * c, scale_log2, 0u, p + 32 * c, pk);
+          p_chunk<false>(v, ls + 32 * c, scale_log2, 0u, p + 32 * c, pk);
         } else {
           const int a = max(lo - 32 * c, 0), bb = min(hi - 32 * c, 31);
           const uint32_t bits = a > bb ? 0u : ((0xffffffffu >> (31 - bb)) & (0xffffffffu << a));
-          fused_p_chunk<true>(v, ls + 32 * c, scale_log2, bits, p + 32 * c, pk);
+          p_chunk<true>(v, ls + 32 * c, scale_log2, bits, p + 32 * c, pk);
         }
         tmem_st(t_S + lane_base + 64 * hf + 16 * c, pk);
       }
@@ -1653,9 +1686,11 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
   {
     KernelScope ks("attn_bwd_dkdv_sm100_kernel", st);
     const int pairs = B * Hkv, n_heavy = n_sink_t + n_gist_t;
-    launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(n_tiles * pairs), kKvThreads, KvSmem<D>::kBytes, st, 1, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
+    const int raw_clusters = (n_raw_t + 1) / 2;
+    launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(2 * (n_heavy + raw_clusters) * pairs), kKvThreads, KvSmem<D>::kBytes,
+                   st, 2, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
         (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, make_fastdiv(n_heavy),
-        make_fastdiv(n_raw_t), make_fastdiv(Hkv));
+        make_fastdiv(raw_clusters), make_fastdiv(Hkv));
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {

@@ -258,6 +258,14 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr, int rank) {
   return v;
 }
 
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr, int rank) {
+  uint32_t at;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+  return v;
+}
+
 // Barrier among `count` threads (a multiple of 32) of the block; id 0 is __syncthreads' own.
 __device__ __forceinline__ void named_barrier_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
