@@ -32,12 +32,12 @@ __device__ unsigned int g_bwd_timeout = 0;
 // and a warp finds its token's run by scanning the (at most twelve) first-token indices.
 struct TokRun {
   Geom g;
-  FastDiv n_div, unit_div, r_div;  // by N, r + 1, r
+  GeomDiv div;
   long long tok_begin;
   float* delta;
 };
 TokRun make_tok_run(const Geom& g, long long tok_begin, float* delta) {
-  return {g, make_fastdiv(g.N), make_fastdiv(g.r + 1), make_fastdiv(g.r), tok_begin, delta};
+  return {g, make_geom_div(g), tok_begin, delta};
 }
 template <int kRuns>
 struct TokRuns {
@@ -64,13 +64,9 @@ bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int H
       while (ri + 1 < P.n && tk >= P.run[ri + 1].tok_begin) ++ri;
     const TokRun& R = P.run[ri];
     const int N = R.g.N, local = (int)(tk - R.tok_begin);
-    const int b = fdiv(R.n_div, local), t = local - b * N;
-    int pos = t;  // Delta is kept in shifted order, whatever the order of dO and O
-    if (interleaved && t >= R.g.s) {
-      const int q = t - R.g.s, u = fdiv(R.unit_div, q), in_unit = q - u * (R.g.r + 1);
-      pos = in_unit == R.g.r ? R.g.s + R.g.T + u : R.g.s + u * R.g.r + in_unit;
-    }
-    float* delta_tok = R.delta + (long long)b * Hq * N + pos;
+    const int b = fdiv(R.div.n, local), t = local - b * N;
+    // Delta is kept in shifted order, whatever the order of dO and O
+    float* delta_tok = R.delta + (long long)b * Hq * N + (interleaved ? unshift_perm(R.g, R.div, t) : t);
     const long long row0 = tk * Hq;
     for (int h0 = 0; h0 < Hq; h0 += kRows * kSteps) {
       uint4 db[kSteps], ob[kSteps];  // 8 bf16 of dO and of O
@@ -1502,13 +1498,8 @@ dq_convert_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int
       while (ri + 1 < P.n && tk >= P.run[ri + 1].tok_begin) ++ri;
     const TokRun& R = P.run[ri];
     const Geom& g = R.g;
-    const int local = (int)(tk - R.tok_begin), b = fdiv(R.n_div, local), sigma = local - b * g.N;
-    int row = sigma;
-    if (interleaved && sigma >= g.s) {
-      const int i = sigma - g.s;
-      row = i < g.T ? sigma + fdiv(R.r_div, i) : g.s + (i - g.T) * (g.r + 1) + g.r;
-    }
-    const long long out_tk = R.tok_begin + (long long)b * g.N + row;
+    const int local = (int)(tk - R.tok_begin), b = fdiv(R.div.n, local), sigma = local - b * g.N;
+    const long long out_tk = R.tok_begin + (long long)b * g.N + (interleaved ? shift_perm(g, R.div, sigma) : sigma);
     const float4* s4 = reinterpret_cast<const float4*>(src + tk * Hq * 128) + lane;
     uint2* d2 = reinterpret_cast<uint2*>(dst + out_tk * Hq * 128) + lane;
     for (int h0 = 0; h0 < Hq; h0 += 4) {

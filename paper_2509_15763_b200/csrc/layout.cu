@@ -31,24 +31,22 @@ int32_t launch_layout(const Geom& g, int32_t* sp, int32_t* up, int32_t* pos, cud
 // (the permutation is evaluated once per row), kRows rows in flight per warp.
 template <bool kInverse>
 __global__ void __launch_bounds__(256)
-shift_rows_kernel(Geom g, const uint4* __restrict__ src, uint4* __restrict__ dst, int vecs,
-                  long long rows) {
+shift_rows_kernel(Geom g, GeomDiv div, const uint4* __restrict__ src, uint4* __restrict__ dst, int vecs,
+                  int rows) {
   pdl_begin();
   constexpr int kRows = 4, kVec = 4;  // up to kRows * kVec loads in flight per lane
   const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
   for (long long r0 = warp * kRows; r0 < rows; r0 += nwarps * kRows) {
     const uint4* sp[kRows];
     uint4* dp[kRows];
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
-      const long long row = r0 + u < rows ? r0 + u : rows - 1;  // the tail repeats the last row (same bytes)
-      const int b = (int)(row / g.N);
-      const int i = (int)(row - (long long)b * g.N);
-      const int j = kInverse ? unshift_perm(g, i) : shift_perm(g, i);
+      const int row = r0 + u < rows ? (int)r0 + u : rows - 1;  // the tail repeats the last row (same bytes)
+      const int b = fdiv(div.n, row), i = row - b * g.N;
+      const int j = kInverse ? unshift_perm(g, div, i) : shift_perm(g, div, i);
       sp[u] = src + ((long long)b * g.N + j) * vecs;
-      dp[u] = dst + row * vecs;
+      dp[u] = dst + (long long)row * vecs;
     }
     for (int v0 = lane; v0 < vecs; v0 += 32 * kVec) {
       uint4 val[kRows][kVec];
@@ -76,7 +74,7 @@ int32_t launch_shift(const Geom& g, int B, const void* src, void* dst, size_t ro
   {
     KernelScope ks(inverse ? "unshift_rows_kernel" : "shift_rows_kernel", st);
     launch_chained(inverse ? shift_rows_kernel<true> : shift_rows_kernel<false>, dim3(blocks), 256, 0, st, 1, g,
-                   (const uint4*)src, (uint4*)dst, vecs, rows);
+                   make_geom_div(g), (const uint4*)src, (uint4*)dst, vecs, (int)rows);
   }
   return check_launch("gist shift kernel");
 }

@@ -103,6 +103,22 @@ __host__ __device__ inline int unshift_perm(const Geom& g, int t) {
   return p == g.r ? g.s + g.T + u : g.s + u * g.r + p;
 }
 
+// Both for code that does this for every token: the divisions by N, r and r + 1 as multiplications.
+struct GeomDiv {
+  FastDiv n, r, unit;
+};
+inline GeomDiv make_geom_div(const Geom& g) { return {make_fastdiv(g.N), make_fastdiv(g.r), make_fastdiv(g.r + 1)}; }
+__host__ __device__ inline int shift_perm(const Geom& g, const GeomDiv& dv, int sigma) {
+  if (sigma < g.s) return sigma;
+  const int i = sigma - g.s;
+  return i < g.T ? sigma + fdiv(dv.r, i) : g.s + (i - g.T) * (g.r + 1) + g.r;
+}
+__host__ __device__ inline int unshift_perm(const Geom& g, const GeomDiv& dv, int t) {
+  if (t < g.s) return t;
+  const int q = t - g.s, u = fdiv(dv.unit, q), p = q - u * (g.r + 1);
+  return p == g.r ? g.s + g.T + u : g.s + u * g.r + p;
+}
+
 // Row of a [B, N, H, D] tensor that holds row `row` of a segment: in shifted order, or in
 // interleaved order (Eq. 2) when the caller's tensors were never shifted.
 // The three segments of the shifted order.
