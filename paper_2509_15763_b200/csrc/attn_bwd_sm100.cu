@@ -54,7 +54,7 @@ template <bool kF32, int kRuns, int D>
 __global__ void __launch_bounds__(256)
 bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, int tokens, const void* __restrict__ d_o,
                 const __nv_bfloat16* __restrict__ o, __nv_bfloat16* __restrict__ d_o_bf16, float* __restrict__ dq32) {
-  pdl_begin();
+  pdl_wait();
   constexpr int kLanes = D / 8, kRows = 32 / kLanes, kSteps = 4;  // lanes of a row, rows of a warp access
   const int lane = threadIdx.x & 31, sub = lane / kLanes, col = (lane % kLanes) * 8;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -285,7 +285,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     mbar_fence_init();
   }
   if (warp == kKvCompute + 1) tmem_alloc(tmem_slot, 512);
-  pdl_begin();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -668,7 +668,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     mbar_fence_init();
   }
   if (warp == 5) tmem_alloc(tmem_slot, 256);
-  pdl_begin();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1045,7 +1045,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
     mbar_fence_init();
   }
   if (warp == kFuMmaWarp) tmem_alloc(tmem_slot, 512);
-  pdl_begin();
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1455,7 +1455,7 @@ __global__ void __launch_bounds__(128)
 dkdv_reduce_kernel(Geom g, int interleaved, int Hkv, int n_sink_kt, int n_gist_kt, int n_chunks, int chunk_tiles,
                    const float* __restrict__ partial, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
                    float scale) {
-  pdl_begin();
+  pdl_wait();
   const int rank = blockIdx.x >> 3, row0 = (blockIdx.x & 7) * 16, hk = blockIdx.y, b = blockIdx.z;
   const int n_heavy_kt = n_sink_kt + n_gist_kt;
   const int kseg = rank < n_sink_kt ? kSegSink : kSegGist;
@@ -1488,7 +1488,7 @@ template <int kRuns>
 __global__ void __launch_bounds__(256)
 dq_convert_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int Hq, long long tokens,
                   const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, float scale) {
-  pdl_begin();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;

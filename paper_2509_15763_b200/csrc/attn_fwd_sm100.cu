@@ -334,7 +334,7 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
     mbar_fence_init();
   }
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-  pdl_begin();  // nothing above touches global memory
+  pdl_wait();  // nothing above touches global memory
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

@@ -18,7 +18,7 @@ __host__ __device__ inline int state_ints(int r, int k) { return kHdr + (k + 1) 
 
 // After a prefix of `units_done` whole units in the cache order of compaction [sinks | gists | window raw].
 __global__ void cache_state_init_kernel(int B, int s, int r, int k, int units_done, int32_t* __restrict__ state) {
-  pdl_begin();
+  pdl_wait();
   const int b = blockIdx.x;
   int32_t* st = state + (long long)b * state_ints(r, k);
   const int w_units = units_done < k ? units_done : k;
@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(128)
 cache_append_kernel(int Hkv, int vecs, int r, int k, int is_gist, const uint4* __restrict__ k_new,
                     const uint4* __restrict__ v_new, uint4* __restrict__ kc, uint4* __restrict__ vc, int num_blocks,
                     const int32_t* __restrict__ table, int max_blocks, int32_t* seq_lens, int32_t* state) {
-  pdl_begin();
+  pdl_wait();
   const int b = blockIdx.x, rows = Hkv * vecs;
   int32_t* st = state + (long long)b * state_ints(r, k);
   int32_t* ring = st + kHdr;

@@ -20,7 +20,7 @@ compact_gather_kernel(Geom g, int B, int Hkv, int vecs, int L, const uint4* __re
                       const uint4* __restrict__ v, uint4* __restrict__ kc, uint4* __restrict__ vc,
                       int num_blocks, const int32_t* __restrict__ table, int max_blocks,
                       int32_t* __restrict__ seq_lens, int32_t* __restrict__ kept_idx, int interleaved) {
-  pdl_begin();
+  pdl_wait();
   const long long per_tok = (long long)Hkv * vecs;
   const long long total = (long long)B * L * per_tok;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -47,7 +47,7 @@ compact_gather_kernel(Geom g, int B, int Hkv, int vecs, int L, const uint4* __re
 // In place, aligned segments: only the block table changes.
 __global__ void compact_edit_table_kernel(Geom g, int L, int32_t* __restrict__ table, int max_blocks,
                                           int32_t* __restrict__ seq_lens, int32_t* __restrict__ kept_idx) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ int32_t old_row[];
   const int b = blockIdx.x;
   const int nbN = g.N / PG, nbL = L / PG;
@@ -76,7 +76,7 @@ compact_stage_kernel(Geom g, int B, int Hkv, int vecs, int L, uint4* __restrict_
                      uint4* __restrict__ vc, int num_blocks, const int32_t* __restrict__ table,
                      int max_blocks, uint4* __restrict__ stage, int32_t* __restrict__ seq_lens,
                      int32_t* __restrict__ kept_idx) {
-  pdl_begin();
+  pdl_wait();
   const long long per_tok = (long long)Hkv * vecs;
   const long long total = (long long)B * L * per_tok;
   uint4* stage_v = stage + total;

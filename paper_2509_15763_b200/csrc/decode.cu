@@ -180,7 +180,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     }
     mbar_fence_init();
   }
-  pdl_begin();  // nothing above touches global memory
+  pdl_wait();  // nothing above touches global memory
   Walk<kFlat> start;
   if constexpr (kFlat) {
     page_prefix(P, prefix, reinterpret_cast<int*>(merge));
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(THREADS)
 decode_combine_kernel(const __grid_constant__ DecParams P, int max_shares) {
   __shared__ int first[kMaxFlatSeqs + 1];
   __shared__ int tmp[THREADS / 32];
-  pdl_begin();
+  pdl_wait();
   page_prefix(P, first, tmp);
   const int seq = blockIdx.x, hk = blockIdx.y, total = first[P.S], warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int a = first[seq], b = first[seq + 1], n = flat_shares(total, max_shares);

@@ -6,7 +6,7 @@ namespace ug {
 
 __global__ void layout_kernel(Geom g, int32_t* __restrict__ sp, int32_t* __restrict__ up,
                               int32_t* __restrict__ pos) {
-  pdl_begin();
+  pdl_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += gridDim.x * blockDim.x) {
     if (sp) sp[i] = shift_perm(g, i);
     const int sig = unshift_perm(g, i);
@@ -33,7 +33,7 @@ template <bool kInverse>
 __global__ void __launch_bounds__(256)
 shift_rows_kernel(Geom g, GeomDiv div, const uint4* __restrict__ src, uint4* __restrict__ dst, int vecs,
                   int rows) {
-  pdl_begin();
+  pdl_wait();
   constexpr int kRows = 4, kVec = 4;  // up to kRows * kVec loads in flight per lane
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;

@@ -21,7 +21,7 @@ prefill_gather_kernel(int B, int Hkv, int vecs, int s, int u0, int w0, int c_raw
                       const uint4* __restrict__ kc, const uint4* __restrict__ vc, int num_blocks,
                       const int32_t* __restrict__ table, int max_blocks, const uint4* __restrict__ k_chunk,
                       const uint4* __restrict__ v_chunk, uint4* __restrict__ k_ctx, uint4* __restrict__ v_ctx) {
-  pdl_begin();
+  pdl_wait();
   const int Tc = w0 + c_raw, n_ctx = s + Tc + u0 + c_gists;
   const int sq = u0 == 0 ? s : 0, n_chunk = sq + c_raw + c_gists;
   const long long per_tok = (long long)Hkv * vecs;

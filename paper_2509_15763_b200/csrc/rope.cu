@@ -23,7 +23,7 @@ rope_kernel(Geom g, GeomDiv div, int tokens, int heads, double log2_theta, int t
   double inv_freq[kMine];  // of frequencies lane, lane + 32
 #pragma unroll
   for (int e = 0; e < kMine; ++e) inv_freq[e] = exp2(-2.0 * (lane + 32 * e) / D * log2_theta);
-  pdl_begin();
+  pdl_wait();
   for (long long tk = warp; tk < tokens; tk += nwarps) {  // tk = b * N + t, t interleaved
     const int b = fdiv(div.n, (int)tk), t = (int)tk - b * g.N;
     const int sigma = unshift_perm(g, div, t);  // the token's shifted position

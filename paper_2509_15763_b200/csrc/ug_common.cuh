@@ -132,16 +132,11 @@ __host__ __device__ inline int seg_row_to_token(const Geom& g, bool interleaved,
   return seg == kSegRaw ? g.s + row + row / g.r : g.s + row * (g.r + 1) + g.r;
 }
 
-// Programmatic dependent launch: the next kernel on the stream may become resident once every block has said so;
-// its pdl_wait() returns when this kernel has completed and its writes are visible.  Both do nothing in a kernel
-// that was launched without the attribute.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Programmatic dependent launch: returns when the kernel before this one on the stream has completed and its writes are
+// visible; every thread calls it before its first access to global memory (in a kernel launched without the attribute it
+// does nothing).  No kernel lets its successor start before its own blocks end (griddepcontrol.launch_dependents): with
+// blocks of the next kernel already sitting on the SMs a training pass took 2 - 4 % longer.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Both, where a kernel's prologue ends: before its first access to global memory.
-__device__ __forceinline__ void pdl_begin() {
-  pdl_launch_dependents();
-  pdl_wait();
-}
 
 // Host side helpers (api.cu).
 int32_t fail(int32_t code, const char* fmt, ...);
@@ -162,9 +157,9 @@ struct KernelScope {
   int slot;
   cudaStream_t st;
 };
-// Launches a kernel whose first access to global memory comes after pdl_wait() (every thread calls it): the kernel may
-// become resident while the one before it on the stream is still running, so that launch latency and prologue are
-// hidden.  cluster > 1: blocks along x in clusters of that many.  An error is picked up by check_launch.
+// Launches a kernel whose first access to global memory comes after pdl_wait(): it may become resident as the one before
+// it on the stream drains, so that launch latency and prologue are hidden.  cluster > 1: blocks along x in clusters of
+// that many.  An error is picked up by check_launch.
 template <typename T>
 struct AsIs {
   using type = T;
