@@ -157,23 +157,39 @@ __device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key
   key_q_interval(g, kseg == kSegRaw, key, true, qseg == kSegRaw, lo, hi);
 }
 
-// One 32-query chunk of P^T for one key: p = 2^(s * c - lse2[q]); kMasked: bit e of `bits` says query e sees the key.
+// One 32-query chunk of P^T for one key: p = 2^(s * c + nl[q]), nl = -LSE in log2 units; kMasked: bit e of `bits` says
+// query e sees the key.  Two queries at a time (packed fp32).
 template <bool kMasked>
-__device__ __forceinline__ void p_chunk(const uint32_t (&v)[32], const float* __restrict__ ls, float scale_log2,
-                                              uint32_t bits, float* __restrict__ p, uint32_t (&pk)[16]) {
+__device__ __forceinline__ void p_chunk(const uint32_t (&v)[32], const float* __restrict__ nl, uint64_t scale2, uint32_t bits,
+                                        float* __restrict__ p, uint32_t (&pk)[16]) {
 #pragma unroll
   for (int i = 0; i < 32; i += 4) {
-    const float4 l4 = *reinterpret_cast<const float4*>(ls + i);
-    const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
+    const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(nl + i);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float x = fmaf(__uint_as_float(v[i + e]), scale_log2, -lv[e]);
-      if (kMasked) x = (bits >> (i + e)) & 1u ? x : -INFINITY;
-      p[i + e] = ex2(x);
+    for (int h = 0; h < 2; ++h) {
+      const int e = i + 2 * h;
+      float x0, x1;
+      f32x2_split(fma2(f32x2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), scale2, h ? l4.y : l4.x), x0, x1);
+      if (kMasked) {
+        x0 = (bits >> e) & 1u ? x0 : -INFINITY;
+        x1 = (bits >> (e + 1)) & 1u ? x1 : -INFINITY;
+      }
+      p[e] = ex2(x0);
+      p[e + 1] = ex2(x1);
+      pk[e / 2] = pack_bf16(p[e], p[e + 1]);
     }
-    pk[i / 2] = pack_bf16(p[i], p[i + 1]);
-    pk[i / 2 + 1] = pack_bf16(p[i + 2], p[i + 3]);
   }
+}
+// dS = p (dP - Delta) of two neighbours, rounded to bf16; nd = -Delta of both.
+__device__ __forceinline__ uint32_t ds_pair(float p0, float p1, uint32_t dp0, uint32_t dp1, uint64_t nd) {
+  float x0, x1;
+  f32x2_split(mul2(f32x2(p0, p1), add2(f32x2(__uint_as_float(dp0), __uint_as_float(dp1)), nd)), x0, x1);
+  return pack_bf16(x0, x1);
+}
+// Bit e: column e of 32 lies inside [lo, hi].
+__device__ __forceinline__ uint32_t piece_bits(int lo, int hi) {
+  const int a = max(lo, 0), b = min(hi, 31);
+  return a > b ? 0u : ((0xffffffffu >> (31 - b)) & (0xffffffffu << a));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -339,9 +355,9 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
       for (int i = 0; i < KV_BN / 32; ++i) {
         const int row = qt * KV_BN + lane + 32 * i;
         const bool valid = row < q_seg_len;
-        // rows past the segment get LSE = +inf, so their P is exactly zero
-        st_l[i] = valid ? lse[row_base + row] * kLog2e : INFINITY;
-        st_d[i] = valid ? delta[row_base + row] : 0.f;
+        // both negated, so that they are added; rows past the segment get LSE = +inf, so their P is exactly zero
+        st_l[i] = valid ? -(lse[row_base + row] * kLog2e) : -INFINITY;
+        st_d[i] = valid ? -delta[row_base + row] : 0.f;
       }
     };
     StepIter cur{t_begin, 0}, ahead{t_begin, 0};
@@ -441,7 +457,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     const int key = key_a + qd * 32 + lane;
     const bool key_valid = key <= key_b;
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
-    const float scale_log2 = scale * kLog2e;
+    const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     int my_lo_r, my_hi_r, my_lo_g, my_hi_g, my_lo_s, my_hi_s;  // queries that see this key, per query segment
     key_q_interval3(g, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
     key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
@@ -474,14 +490,11 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
         uint32_t pk[16];
         // a partly visible tile: most of its 32 x 32 pieces are wholly visible all the same
         uint32_t bits = 0xffffffffu;
-        if (!full) {
-          const int qa = max(lo, 0), qz = min(hi, 31);
-          bits = qa > qz ? 0u : ((0xffffffffu >> (31 - qz)) & (0xffffffffu << qa));
-        }
+        if (!full) bits = piece_bits(lo, hi);
         if (full || __all_sync(0xffffffffu, bits == 0xffffffffu))
-          p_chunk<false>(v, ls, scale_log2, 0u, p, pk);
+          p_chunk<false>(v, ls, scale2, 0u, p, pk);
         else
-          p_chunk<true>(v, ls, scale_log2, bits, p, pk);
+          p_chunk<true>(v, ls, scale2, bits, p, pk);
         tmem_st(t_A + lane_base + 32 * hf, pk);
       }
       tmem_wait_st();
@@ -497,13 +510,9 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
         uint32_t pk[16];
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
-          const float4 d4 = *reinterpret_cast<const float4*>(dl + i);
-          const float dv4[4] = {d4.x, d4.y, d4.z, d4.w};
-          float ds[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ds[e] = p[i + e] * (__uint_as_float(v[i + e]) - dv4[e]);
-          pk[i / 2] = pack_bf16(ds[0], ds[1]);
-          pk[i / 2 + 1] = pack_bf16(ds[2], ds[3]);
+          const ulonglong2 d4 = *reinterpret_cast<const ulonglong2*>(dl + i);
+          pk[i / 2] = ds_pair(p[i], p[i + 1], v[i], v[i + 1], d4.x);
+          pk[i / 2 + 1] = ds_pair(p[i + 2], p[i + 3], v[i + 2], v[i + 3], d4.y);
         }
         tmem_st(t_B + lane_base + 32 * hf, pk);
       }
@@ -769,9 +778,10 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     const bool valid = row_a + r_in_tile <= row_b;
     const RowIv my = row_intervals(g, q_base + row);
     const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
-    const float scale_log2 = scale * kLog2e;
+    const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     const long long stat_idx = ((long long)b * Hq + h) * g.N + q_base + row;
-    const float lse2 = lse[stat_idx] * kLog2e, dl = delta[stat_idx];
+    const float nl = -(lse[stat_idx] * kLog2e), nd = -delta[stat_idx];
+    const uint64_t nl2 = f32x2(nl, nl), nd2 = f32x2(nd, nd);
     for (int j = 0; j < nt && ok; ++j) {
       int sg, idx;
       key_tile(j, sg, idx);
@@ -795,26 +805,33 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       if (!ok) break;
       tc_fence_after();
       const uint32_t t_S = t_S0 + 64 * (j % SM::kSBufs);
+      // both operands of the whole row in one go (a block's 192 threads leave 168 registers each)
+      uint32_t sv[DQ_BN], dv_[DQ_BN];
 #pragma unroll
       for (int c = 0; c < DQ_BN / 32; ++c) {
-        uint32_t sv[32], dv_[32];
-        tmem_ld(t_S + lane_base + 32 * c, sv);
-        tmem_ld(t_dP + lane_base + 32 * c, dv_);
-        tmem_wait_ld();
-        uint32_t pk[16];
+        tmem_ld32(t_S + lane_base + 32 * c, sv + 32 * c);
+        tmem_ld32(t_dP + lane_base + 32 * c, dv_ + 32 * c);
+      }
+      tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-          float x0 = fmaf(__uint_as_float(sv[i]), scale_log2, -lse2);
-          float x1 = fmaf(__uint_as_float(sv[i + 1]), scale_log2, -lse2);
-          if (!full) {
-            const int col = 32 * c + i;
-            x0 = (col >= lo && col <= hi) ? x0 : -INFINITY;
-            x1 = (col + 1 >= lo && col + 1 <= hi) ? x1 : -INFINITY;
+      for (int c = 0; c < DQ_BN / 32; ++c) {
+        uint32_t pk[16];
+        uint32_t bits = 0xffffffffu;
+        if (!full) bits = piece_bits(lo - 32 * c, hi - 32 * c);
+        auto piece = [&](bool masked) {
+#pragma unroll
+          for (int i = 0; i < 32; i += 2) {
+            const int e = 32 * c + i;
+            float x0, x1;
+            f32x2_split(fma2(f32x2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), scale2, nl2), x0, x1);
+            if (masked) {
+              x0 = (bits >> i) & 1u ? x0 : -INFINITY;
+              x1 = (bits >> (i + 1)) & 1u ? x1 : -INFINITY;
+            }
+            pk[i / 2] = ds_pair(ex2(x0), ex2(x1), dv_[e], dv_[e + 1], nd2);
           }
-          const float ds0 = ex2(x0) * (__uint_as_float(dv_[i]) - dl);
-          const float ds1 = ex2(x1) * (__uint_as_float(dv_[i + 1]) - dl);
-          pk[i / 2] = pack_bf16(ds0, ds1);
-        }
+        };
+        if (full || __all_sync(0xffffffffu, bits == 0xffffffffu)) piece(false); else piece(true);
         tmem_st(t_S + lane_base + 16 * c, pk);
       }
       tmem_wait_st();
@@ -1112,9 +1129,9 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         for (int i = 0; i < 4; ++i) {
           const int row = qt * 128 + lane + 32 * i;
           const bool valid = row < q_seg_len;
-          // rows past the segment get LSE = +inf, so their P is exactly zero
-          st_l[i] = valid ? lse[row_base + row] * kLog2e : INFINITY;
-          st_d[i] = valid ? delta[row_base + row] : 0.f;
+          // both negated, so that they are added; rows past the segment get LSE = +inf, so their P is exactly zero
+          st_l[i] = valid ? -(lse[row_base + row] * kLog2e) : -INFINITY;
+          st_d[i] = valid ? -delta[row_base + row] : 0.f;
         }
       };
       StepIter cur{t_begin, 0}, ahead{t_begin, 0};
@@ -1306,7 +1323,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
     const int key = key_a + krow;
     const bool key_valid = key <= key_b;
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
-    const float scale_log2 = scale * kLog2e;
+    const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     int my_lo_r, my_hi_r, my_lo_g, my_hi_g, my_lo_s, my_hi_s;  // queries that see this key, per query segment
     key_q_interval3(g, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
     key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
@@ -1341,11 +1358,9 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         tmem_wait_ld();
         uint32_t pk[16];
         if (full) {
-          p_chunk<false>(v, ls + 32 * c, scale_log2, 0u, p + 32 * c, pk);
+          p_chunk<false>(v, ls + 32 * c, scale2, 0u, p + 32 * c, pk);
         } else {
-          const int a = max(lo - 32 * c, 0), bb = min(hi - 32 * c, 31);
-          const uint32_t bits = a > bb ? 0u : ((0xffffffffu >> (31 - bb)) & (0xffffffffu << a));
-          p_chunk<true>(v, ls + 32 * c, scale_log2, bits, p + 32 * c, pk);
+          p_chunk<true>(v, ls + 32 * c, scale2, piece_bits(lo - 32 * c, hi - 32 * c), p + 32 * c, pk);
         }
         tmem_st(t_S + lane_base + 64 * hf + 16 * c, pk);
       }
@@ -1363,14 +1378,14 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
         tmem_wait_ld();
 #pragma unroll
         for (int i = 0; i < 32; i += 8) {  // 8 queries = one 16-byte chunk of this key's dS^T row
-          const float4 d0 = *reinterpret_cast<const float4*>(dl + 32 * c + i);
-          const float4 d1 = *reinterpret_cast<const float4*>(dl + 32 * c + i + 4);
+          const ulonglong2 d0 = *reinterpret_cast<const ulonglong2*>(dl + 32 * c + i);
+          const ulonglong2 d1 = *reinterpret_cast<const ulonglong2*>(dl + 32 * c + i + 4);
           const float* pp = p + 32 * c + i;
           uint4 w;
-          w.x = pack_bf16(pp[0] * (__uint_as_float(v[i]) - d0.x), pp[1] * (__uint_as_float(v[i + 1]) - d0.y));
-          w.y = pack_bf16(pp[2] * (__uint_as_float(v[i + 2]) - d0.z), pp[3] * (__uint_as_float(v[i + 3]) - d0.w));
-          w.z = pack_bf16(pp[4] * (__uint_as_float(v[i + 4]) - d1.x), pp[5] * (__uint_as_float(v[i + 5]) - d1.y));
-          w.w = pack_bf16(pp[6] * (__uint_as_float(v[i + 6]) - d1.z), pp[7] * (__uint_as_float(v[i + 7]) - d1.w));
+          w.x = ds_pair(pp[0], pp[1], v[i], v[i + 1], d0.x);
+          w.y = ds_pair(pp[2], pp[3], v[i + 2], v[i + 3], d0.y);
+          w.z = ds_pair(pp[4], pp[5], v[i + 4], v[i + 5], d1.x);
+          w.w = ds_pair(pp[6], pp[7], v[i + 6], v[i + 7], d1.y);
           const int chunk = 4 * c + i / 8;
           *reinterpret_cast<uint4*>(ds_row + ((chunk ^ swz) << 4)) = w;
         }
