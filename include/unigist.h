@@ -169,7 +169,7 @@ int32_t unigist_attn_fwd(const unigist_problem* p, const void* q, const void* k,
  * UNIGIST_FLAG_DOUT_FP32); dq [B,N,Hq,D], dk, dv [B,N,Hkv,D] device bf16, all shifted.
  * dK/dV are accumulated without atomics: a key tile is owned by one thread block, or, where very many queries see
  * it (sink and gist keys of a long sequence), by one block per chunk of those queries whose fp32 partial sums a
- * small kernel adds in chunk order; either way they are the same bit for bit from run to run.  For head_dim 128
+ * small kernel, or the two blocks of a cluster, add in a fixed order; either way they are the same bit for bit from run to run.  For head_dim 128
  * dQ is the sum, over the key tiles that see a query tile, of fp32 partial tiles reduced into the workspace in
  * whatever order the blocks arrive: its last bit may differ between runs (UNIGIST_FLAG_DETERMINISTIC_DQ trades
  * speed for a fixed order).  workspace:
@@ -284,7 +284,8 @@ int32_t unigist_decode_step(const unigist_problem* p, const void* q, const void*
                             const int32_t* seq_lens, const int32_t* state, void* o, float* lse, void* workspace,
                             size_t ws_bytes, void* stream);
 
-/* Scratch for unigist_decode (split-KV partial results). */
+/* Scratch for unigist_decode (partial results of sequences that several thread blocks share).  This much gives the best
+ * schedule; a smaller workspace is accepted as long as the message of UNIGIST_ERR_WORKSPACE does not ask for more. */
 size_t unigist_decode_workspace_bytes(int32_t num_seqs, int32_t num_q_heads, int32_t num_kv_heads,
                                       int32_t head_dim, int32_t max_blocks_per_seq);
 

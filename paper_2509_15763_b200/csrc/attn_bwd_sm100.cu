@@ -4,7 +4,8 @@
 //                              dQ accumulator of the fused kernel.
 // head_dim 128: attn_bwd_fused_sm100_kernel (described where it is defined) and dq_convert_kernel.
 // head_dim 64: two kernels (a 64-row dQ^T accumulator would halve the fused kernel's tensor throughput):
-//   attn_bwd_dkdv_sm100_kernel one thread block owns a 128-key tile of one KV head and walks every
+//   attn_bwd_dkdv_sm100_kernel one thread block owns a 128-key tile of one KV head (two blocks of a cluster share a
+//                              sink or gist key tile) and walks every
 //                              128-query tile of every query head of the group that can see it:
 //                              S^T = K Q^T and dP^T = V dO^T (TMEM), P^T = exp2(S^T c - LSE),
 //                              dS^T = P^T o (dP^T - Delta), dV += P^T dO, dK += dS^T Q.  dK and dV
@@ -195,8 +196,8 @@ __device__ __forceinline__ uint32_t piece_bits(int lo, int hi) {
 // ------------------------------------------------------------------------------------------------
 // dK / dV kernel.  Bound by the chain scores -> P -> dP -> dS of one step, not by the tensor pipe: with head_dim 64
 // tensor memory has room for a second S buffer and shared memory for four Q / dO stages, which take the scores and the
-// loads off that chain; with heavy tiles first over all heads, two sequences of 8190 raw tokens (ratio 7, 16 / 4
-// heads) took 0.70 ms before and 0.45 now.
+// loads off that chain (two sequences of 8190 raw tokens, ratio 7, 16 / 4 heads: 0.70 -> 0.45 ms, heavy tiles first over
+// all heads included); shared heavy tiles, 16 compute warps and packed arithmetic brought it to 0.32.
 constexpr int KV_BM = 128;       // keys per block (TMEM lanes)
 constexpr int KV_BN = 128;       // queries per step
 // 16 compute warps (four per TMEM lane quarter, 32 query columns each: half the columns per thread shorten the chain of a
@@ -601,7 +602,8 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 
 // ------------------------------------------------------------------------------------------------
 // dQ kernel.  Two blocks per SM cover each other's softmax; with head_dim 64 a ring of four K / V stages and a second S
-// buffer leave only dP and dS on the chain of a step (the problem above: 0.38 ms -> 0.285).
+// buffer leave only dP and dS on the chain of a step (the problem above: 0.38 ms -> 0.285; 0.27 with a row's operands loaded in
+// one go and packed arithmetic; eight compute warps of 32 keys were slower, 0.31).
 constexpr int DQ_BM = 128;  // query rows per block
 constexpr int DQ_BN = 64;   // keys per step
 constexpr int kDqThreads = 192;
