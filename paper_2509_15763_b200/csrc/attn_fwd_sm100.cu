@@ -636,6 +636,15 @@ int32_t get_encode_fn(EncodeFn* out) {
   *out = encode;
   return UNIGIST_OK;
 }
+// Encodes a map.  The driver call wants a current context, and a thread whose first CUDA call this is has none yet:
+// setting the device that the runtime would use anyway makes its context current (no work, allowed while capturing).
+template <typename... Args>
+CUresult encode_bound(EncodeFn encode, Args... args) {
+  CUresult r = encode(args...);
+  int dev = 0;
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode(args...);
+  return r;
+}
 int32_t encode_map(CUtensorMap* map, const void* base, int D, int H, long long N, int B, long long seg_first_row,
                    long long seg_rows, int box_cols, int box_rows, int elem_bytes) {
   EncodeFn encode;
@@ -647,7 +656,7 @@ int32_t encode_map(CUtensorMap* map, const void* base, int D, int H, long long N
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   void* addr = const_cast<char*>(static_cast<const char*>(base)) + seg_first_row * H * D * elem_bytes;
   const bool bf16 = elem_bytes == 2;
-  CUresult r = encode(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, addr, dims,
+  CUresult r = encode_bound(encode, map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, addr, dims,
                       strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                       bf16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -701,7 +710,7 @@ int32_t encode_tile_map(CUtensorMap* map, const void* base, int D, int H, int B,
   const cuuint32_t box[5] = {64, 1, (cuuint32_t)unit_rows, (cuuint32_t)(128 / unit_rows), 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   void* addr = const_cast<char*>(static_cast<const char*>(base)) + first_row * row_bytes;
-  CUresult rc = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, addr, dims, strides, box, estr,
+  CUresult rc = encode_bound(encode, map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, addr, dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (rc != CUDA_SUCCESS) return fail(UNIGIST_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)rc);
@@ -715,7 +724,7 @@ int32_t encode_map_2d_bf16(CUtensorMap* map, const void* base, long long rows, i
   const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
   const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+  CUresult r = encode_bound(encode, map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(UNIGIST_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
