@@ -1,4 +1,8 @@
 """What the binding's marshalling refuses before any C call (no GPU needed)."""
+import subprocess
+import sys
+from pathlib import Path
+
 import pytest
 import torch
 
@@ -43,3 +47,53 @@ def test_wrong_kinds_of_arguments_are_refused():
         ug.unigist_attn_fwd_docs(P, ["x"], *[t()] * 5)
     with pytest.raises(TypeError):
         ug.unigist_attn_fwd_docs(P, 16, *[t()] * 5)
+
+
+# One call of every enqueueing function with a fake CUDA tensor `x` as one of its tensors: inside a transform x has no storage,
+# so its address cannot be taken.
+NO_STORAGE = """
+import sys, types
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+import paper_2509_15763_b200 as ug
+
+P, st = ug.Problem(1, 16, 4, 4, 1, 1, 64), types.SimpleNamespace(cuda_stream=0)
+calls = [
+    lambda x, t: ug.unigist_gist_shift(P, x, t, stream=st),
+    lambda x, t: ug.unigist_gist_unshift(P, t, x, stream=st),
+    lambda x, t: ug.unigist_rope(P, t, x, 1e4, stream=st),
+    lambda x, t: ug.unigist_attn_fwd(P, t, t, x, t, t, stream=st),
+    lambda x, t: ug.unigist_attn_bwd(P, *[t] * 9, x, stream=st),
+    lambda x, t: ug.unigist_attn_fwd_docs(P, [16], x, t, t, t, t, stream=st),
+    lambda x, t: ug.unigist_attn_bwd_docs(P, [16], *[t] * 5, x, t, t, t, t, stream=st),
+    lambda x, t: ug.unigist_kv_compact(P, t, x, t, t, t, t, stream=st),
+    lambda x, t: ug.unigist_prefill_chunk(P, 0, 1, *[t] * 9, x, stream=st),
+    lambda x, t: ug.unigist_cache_state_init(P, 0, x, stream=st),
+    lambda x, t: ug.unigist_cache_append(P, x, t, False, *[t] * 5, stream=st),
+    lambda x, t: ug.unigist_decode_step(P, x, *[t] * 8, stream=st),
+    lambda x, t: ug.unigist_decode(x[0], *[t] * 7, stream=st),
+    lambda x, t: ug.unigist_decode_static(x[0], *[t] * 6, stream=st),
+]
+before = ug.unigist_launch_count()
+with FakeTensorMode():
+    t = torch.zeros(1, 20, 1, 64, dtype=torch.bfloat16, device="cuda")
+    for call in calls:
+        def f(x):
+            call(x, t)
+            return x.float().sum()
+        for run in (lambda: torch.func.vmap(f)(torch.stack([t, t])), lambda: torch.func.grad(f)(t),
+                    lambda: torch.func.jvp(f, (t,), (t,))):
+            try:
+                run()
+            except RuntimeError as e:
+                assert "Cannot access data pointer" in str(e), e
+            else:
+                raise AssertionError("accepted")
+assert ug.unigist_launch_count() == before
+print("refused", 3 * len(calls))
+"""
+
+
+def test_tensors_without_storage_are_refused():
+    run = subprocess.run([sys.executable, "-c", NO_STORAGE], cwd=Path(__file__).resolve().parent.parent, capture_output=True, text=True)
+    assert run.returncode == 0 and "refused 42" in run.stdout, run.stderr[-2000:]
