@@ -71,12 +71,11 @@ struct Args {
     auto field = [&](const char* name) {
       PyObject* v = PyObject_GetAttrString(o, name);
       if (!v) throw python_error();
-      if (!PyLong_Check(v)) {
-        Py_DECREF(v);
-        raise(PyExc_TypeError, "the fields of a problem are integers (softmax_scale: a number)");
-      }
-      const unsigned long long x = PyLong_AsUnsignedLongLongMask(v);
+      PyObject* i = PyNumber_Index(v);  // whatever counts as an integer (numpy's too), as ctypes takes it; no float
       Py_DECREF(v);
+      if (!i) throw python_error();
+      const unsigned long long x = PyLong_AsUnsignedLongLongMask(i);
+      Py_DECREF(i);
       if (PyErr_Occurred()) throw python_error();
       return x;
     };

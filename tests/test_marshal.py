@@ -3,6 +3,7 @@ import subprocess
 import sys
 from pathlib import Path
 
+import numpy as np
 import pytest
 import torch
 
@@ -47,6 +48,16 @@ def test_wrong_kinds_of_arguments_are_refused():
         ug.unigist_attn_fwd_docs(P, ["x"], *[t()] * 5)
     with pytest.raises(TypeError):
         ug.unigist_attn_fwd_docs(P, 16, *[t()] * 5)
+
+
+def test_a_problem_of_numpy_integers_is_a_problem():
+    fields = [np.int64(1), np.int32(16), np.int16(4), np.uint8(4), np.int64(1), np.int64(1), np.int64(64)]
+    p = ug.Problem(*fields, num_sinks=np.int64(0), flags=np.uint32(0))
+    assert ug.unigist_total_len(p) == 20  # the size queries take it
+    with pytest.raises(ValueError, match="contiguous CUDA tensors"):  # ... and so do the calls: on to their tensors
+        ug.unigist_gist_shift(p, t(), t())
+    with pytest.raises(TypeError):
+        ug.unigist_gist_shift(ug.Problem(np.float32(1), *fields[1:]), t(), t())
 
 
 # One call of every enqueueing function with a fake CUDA tensor `x` as one of its tensors: inside a transform x has no storage,
