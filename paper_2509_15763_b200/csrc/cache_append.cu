@@ -95,6 +95,7 @@ cache_append_kernel(int Hkv, int vecs, int r, int k, int is_gist, const uint4* _
       st[3] = 0;
     }
   }
+  if (slot < 0) return;  // (a sequence length below zero)
   const int blk = table[(long long)b * max_blocks + slot / PG];
   if (blk < 0 || blk >= num_blocks) return;  // never write outside the cache
   for (int e = threadIdx.x; e < rows; e += blockDim.x) {

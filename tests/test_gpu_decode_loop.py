@@ -127,3 +127,22 @@ def test_append_flags_misuse_and_leaves_the_cache_alone():
     ug.unigist_cache_append(p, x, x, True, kc, vc, table, lens, state)   # a gist with no raw token before it
     torch.cuda.synchronize()
     assert state[4].item() == 2 and lens.item() == 0 and kc.abs().sum().item() == 0
+
+
+def test_append_to_a_length_below_zero_writes_no_row():
+    r, D, Hkv = 4, 128, 2
+    p = ug.Problem(2, 8, r, 4, Hkv, Hkv, D)
+    kc = torch.zeros(4, Hkv, PG, D, dtype=torch.bfloat16, device=DEV)
+    vc = torch.zeros_like(kc)
+    table = torch.tensor([[1, 2], [3, 0]], dtype=torch.int32, device=DEV)  # (the rows before page 1 are inside the tensor)
+    lens = torch.tensor([-1, 5], dtype=torch.int32, device=DEV)
+    state = torch.zeros(ug.unigist_cache_state_bytes(p) // 4, dtype=torch.int32, device=DEV)
+    ug.unigist_cache_state_init(p, 0, state)
+    x = torch.ones(2, Hkv, D, dtype=torch.bfloat16, device=DEV)
+    ug.unigist_cache_append(p, x, x, False, kc, vc, table, lens, state)
+    torch.cuda.synchronize()
+    assert lens.tolist() == [0, 6]
+    for cache in (kc, vc):
+        assert (cache[3, :, 5] == 1).all()
+        cache[3, :, 5] = 0
+        assert (cache == 0).all()
