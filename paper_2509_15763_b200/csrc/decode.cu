@@ -57,6 +57,13 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// x, or the largest finite number for an infinity or NaN (min of the magnitudes; the operand that is a number wins).
+__device__ __forceinline__ float to_finite(float x) {
+  float y;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(y) : "f"(x), "f"(3.402823466e38f));
+  return y;
+}
+
 // Shared memory of a block: the ring, the barriers, the warps' results and, for the flat walk, the sequences'
 // running page counts.  Two blocks share an SM (233,472 bytes with 1 KB of the system's own per block).
 constexpr int kMaxFlatSeqs = 768;
@@ -313,7 +320,9 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         m_run = m_new;
         float ps = 0.f;
         // P as bf16 pairs, pa[nt] = tokens 8 nt + 2 qc + {0, 1} of row g, and what the rounding left over: it goes into
-        // the padding rows 8 .. 15 of the same products, so that O sees P to 16 bits at no cost
+        // the padding rows 8 .. 15 of the same products, so that O sees P to 16 bits at no cost.  (Times an infinite V
+        // a rest of zero gives NaN and one below zero the opposite infinity; the product with P alone is what counts there,
+        // and it stays what it is when something finite is added.)
         uint32_t pa[8], pb[8];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
@@ -339,10 +348,10 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
             mma_bf16(c0, pa[2 * ks], pb[2 * ks], pa[2 * ks + 1], pb[2 * ks + 1], v0, v1);
             mma_bf16(c1, pa[2 * ks], pb[2 * ks], pa[2 * ks + 1], pb[2 * ks + 1], v2, v3);
           }
-          o[2 * np][0] = fmaf(o[2 * np][0], f, c0[0] + c0[2]);
-          o[2 * np][1] = fmaf(o[2 * np][1], f, c0[1] + c0[3]);
-          o[2 * np + 1][0] = fmaf(o[2 * np + 1][0], f, c1[0] + c1[2]);
-          o[2 * np + 1][1] = fmaf(o[2 * np + 1][1], f, c1[1] + c1[3]);
+          o[2 * np][0] = fmaf(o[2 * np][0], f, c0[0] + to_finite(c0[2]));
+          o[2 * np][1] = fmaf(o[2 * np][1], f, c0[1] + to_finite(c0[3]));
+          o[2 * np + 1][0] = fmaf(o[2 * np + 1][0], f, c1[0] + to_finite(c1[2]));
+          o[2 * np + 1][1] = fmaf(o[2 * np + 1][1], f, c1[1] + to_finite(c1[3]));
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bars + 8 * (STAGES + st));  // the stage may be refilled

@@ -68,3 +68,34 @@ def test_decode_cuts(Hq, Hkv, lens, width, least):
         oo, ll = oracle.decode(D ** -0.5, f64(q[i:i + 1]), [kl], [vl])
         check_close(f"O of sequence {i}", f64(o[i:i + 1]), oo, TOL_O_MAX, TOL_O_MEAN)
         check_close(f"LSE of sequence {i}", f64(lse[i:i + 1]), ll, TOL_LSE)
+
+
+@pytest.mark.parametrize("width", [3, 9, 700])  # one block, a cluster, the flat walk
+@pytest.mark.parametrize("n", [1, 130])
+def test_infinities_in_v(width, n):
+    """A visible infinity in V comes out as that infinity (both signs in one column: NaN), whatever the rounding of its
+    weight; the other columns are as exact as ever."""
+    Hq, Hkv, D = 8, 2, 128
+    g = torch.Generator().manual_seed(n + width)
+    pages = -(-n // PG)
+    kc, vc = (torch.randn(pages, Hkv, PG, D, generator=g).to(torch.bfloat16) for _ in range(2))
+    inf = float("inf")
+    for i, column in enumerate((0, 9, 77)):  # the token that holds an infinity: the first one, and where there are more, others
+        t = (0, n // 2, n - 1)[i]
+        vc[t // PG, :, t % PG, column] = inf if i % 2 == 0 else -inf
+    if n > 1:
+        vc[0, :, 0, 127], vc[0, :, 1, 127] = inf, -inf
+    q = (0.5 * torch.randn(1, Hq, D, generator=g)).to(torch.bfloat16)  # (every weight stays above zero)
+    table = torch.zeros(1, width, dtype=torch.int32)
+    table[0, :pages] = torch.arange(pages)
+    ws = torch.empty(ug.unigist_decode_workspace_bytes(1, Hq, Hkv, D, width), dtype=torch.uint8, device=DEV)
+    o = torch.zeros(1, Hq, D, dtype=torch.bfloat16, device=DEV)
+    ug.unigist_decode(*(x.to(DEV) for x in (q, kc, vc, table, torch.tensor([n], dtype=torch.int32))), o, None, ws)
+    torch.cuda.synchronize()
+    got = f64(o[0])
+    assert (got[:, 0] == inf).all() and (got[:, 9] == -inf).all() and (got[:, 77] == inf).all()
+    assert n == 1 or np.isnan(got[:, 127]).all()
+    rest = [c for c in range(D) if c not in (0, 9, 77, 127)]
+    kl, vl = (f64(c.permute(0, 2, 1, 3).reshape(-1, Hkv, D)[:n]) for c in (kc, vc))
+    want = oracle.decode(D ** -0.5, f64(q), [kl], [np.where(np.isfinite(vl), vl, 0.0)])[0][0]
+    check_close("the other columns", got[:, rest], want[:, rest], TOL_O_MAX, TOL_O_MEAN)
