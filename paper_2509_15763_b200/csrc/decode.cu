@@ -1,9 +1,10 @@
 // Decode attention over the compacted, paged KV cache (Section 4.3): one query per sequence,
 // every cache entry visible.  Split over keys: each thread block streams contiguous ranges of 64-token
 // pages through a ring in shared memory.  A short walk is shared by a cluster of blocks that merge through
-// distributed shared memory; otherwise the pages of all sequences are dealt out evenly and a second kernel adds
-// up the sequences that were cut.  HBM-bound: K and V are read exactly once (64 sequences of 9216 tokens, 2.4 GB:
-// 6.9 TB/s, the copy rate of the chip being 6.5; one of 1337 tokens: 5.7 us in a graph, 8.5 with two kernels).
+// distributed shared memory, or by more blocks whose results a second kernel adds up; otherwise the pages of all
+// sequences are dealt out evenly, and the second kernel adds up the sequences that were cut (decode_plan).  HBM-bound:
+// K and V are read exactly once (64 sequences of 9216 tokens, 2.4 GB: 6.9 TB/s, the copy rate of the chip being 6.5;
+// one of 1337 tokens: 5.7 us in a graph, 8.5 with two kernels).
 //   producer warp:  per page one K and one V tile (64 tokens x 128 dims, 16 KB each) by TMA, 128-byte
 //                   swizzle, into a 3-stage ring guarded by full / empty mbarriers; two thread blocks
 //                   per SM keep about 128 KB of loads in flight.
@@ -64,14 +65,14 @@ __device__ __forceinline__ float to_finite(float x) {
   return y;
 }
 
-// Shared memory of a block: the ring, the barriers, the warps' results and, for the flat walk, the sequences'
-// running page counts.  Two blocks share an SM (233,472 bytes with 1 KB of the system's own per block).
-constexpr int kMaxFlatSeqs = 768;
+// Shared memory of a block: the ring, the barriers, the warps' results and, for the flat walk, the running page
+// counts.  Two blocks share an SM (233,472 bytes with 1 KB of the system's own per block).
+constexpr int kRow = DD + 4;  // a head's result: 128 sums, maximum, sum of the weights (rows of whole 16-byte pieces)
 struct DecSmem {
   static constexpr int kOffBars = STAGES * STAGE_BYTES;
-  static constexpr int kOffMerge = kOffBars + 64;                              // [warps][8 heads][128 + 2] fp32
-  static constexpr int kOffFirst = kOffMerge + kConsumers * 8 * (DD + 2) * 4;  // [S + 1] int
-  static constexpr int kBytes = kOffFirst + (kMaxFlatSeqs + 1) * 4 + 1024 /*align*/;
+  static constexpr int kOffMerge = kOffBars + 64;                              // [warps][8 heads][kRow] fp32
+  static constexpr int kOffFirst = kOffMerge + kConsumers * 8 * kRow * 4;  // [THREADS + 1] 64-bit
+  static constexpr int kBytes = kOffFirst + (THREADS + 1) * 8 + 1024 /*align*/;
 };
 static_assert(2 * (DecSmem::kBytes + 1024) <= 233472, "two blocks per SM");
 
@@ -82,16 +83,23 @@ struct DecParams {
   const int32_t* holes;  // per sequence: [2] number of freed slots, [holes_off ..] the slots; or null
   __nv_bfloat16* o;
   float* lse;
-  float* part_o;    // flat walk: [slots][Hq][128] unnormalised partial outputs
-  float2* part_ml;  // [slots][Hq] (maximum in log2 units, sum)
+  long long* pages_before;  // flat walk: [S + 1] pages of the sequences before each, left by the first kernel for the second
+  int splits;               // even split: blocks per (sequence, KV head) whose partial results the second kernel adds, or 0
+  float* part_o;            // [slots][Hq][128] unnormalised partial outputs
+  float2* part_ml;          // [slots][Hq] (maximum in log2 units, sum)
   int S, Hq, Hkv, G, num_blocks, max_blocks, holes_stride, holes_off;
   float scale_log2;
 };
 
-// One element of O, and with it (d = 0) the row's LSE.  A sequence with nothing to attend to (length 0, or every
+__device__ __forceinline__ void add_weighted(float4& acc, float& L, float weight, float4 x, float l) {
+  acc.x += weight * x.x, acc.y += weight * x.y, acc.z += weight * x.z, acc.w += weight * x.w;
+  L += weight * l;
+}
+// Four elements of O, and with them (d = 0) the row's LSE.  A sequence with nothing to attend to (length 0, or every
 // slot freed) has O = 0 and LSE = -inf, not 0 / 0.
-__device__ __forceinline__ void write_row(const DecParams& P, long long row, int d, float acc, float M, float L) {
-  P.o[row * DD + d] = __float2bfloat16_rn(L > 0.f ? acc / L : 0.f);
+__device__ __forceinline__ void write_row(const DecParams& P, long long row, int d, float4 acc, float M, float L) {
+  *reinterpret_cast<uint2*>(P.o + row * DD + d) =
+      L > 0.f ? make_uint2(pack_bf16(acc.x / L, acc.y / L), pack_bf16(acc.z / L, acc.w / L)) : make_uint2(0u, 0u);
   if (P.lse && d == 0) P.lse[row] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
 }
 
@@ -100,44 +108,69 @@ __device__ __forceinline__ int pages_of(int len, int max_blocks) {
   return len > 0 ? min((len - 1) / PG + 1, max_blocks) : 0;
 }
 
-// first[i] = pages of the sequences before i (first[S] = all): every block works it out for itself, each thread
-// adding up a run of neighbouring sequences.  `tmp`: 4 ints of shared memory.  Ends with a barrier.
-__device__ __forceinline__ void page_prefix(const DecParams& P, int* first, int* tmp) {
-  constexpr int kPer = kMaxFlatSeqs / THREADS;
-  const int per = (P.S + THREADS - 1) / THREADS, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int n[kPer], sum = 0;
+// The sequences are taken in groups of `per` neighbours, one group a thread: first[t] = pages of the groups before t
+// (first[THREADS] = all).  Every block works it out for itself.  `tmp`: one number per warp.  Ends with a barrier.
+__device__ __forceinline__ void page_prefix(const DecParams& P, int per, long long* first, long long* tmp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int s0 = min((int)threadIdx.x * per, P.S), s1 = min(s0 + per, P.S);
+  long long sum = 0;
+  for (int i = s0; i < s1; i += 8) {
+    int n[8];
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int s = threadIdx.x * per + i;
-    n[i] = i < per && s < P.S ? pages_of(P.seq_lens[s], P.max_blocks) : 0;
+    for (int u = 0; u < 8; ++u) n[u] = i + u < s1 ? pages_of(P.seq_lens[i + u], P.max_blocks) : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sum += n[u];
   }
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) sum += n[i];
-  int incl = sum;
+  long long incl = sum;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
-    const int x = __shfl_up_sync(0xffffffffu, incl, off);
+    const long long x = __shfl_up_sync(0xffffffffu, incl, off);
     if (lane >= off) incl += x;
   }
   if (lane == 31) tmp[warp] = incl;
   __syncthreads();
-  int at = incl - sum;
+  long long at = incl - sum;
   for (int w = 0; w < warp; ++w) at += tmp[w];
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int s = threadIdx.x * per + i;
-    if (i < per && s <= P.S) first[s] = at;
-    at += n[i];
-  }
-  // (where the runs end exactly at S, the last entry belongs to no thread's run)
-  if (threadIdx.x == THREADS - 1 && THREADS * per == P.S) first[P.S] = at;
+  first[threadIdx.x] = at;
+  if (threadIdx.x == THREADS - 1) first[THREADS] = at + sum;
   __syncthreads();
 }
 
+// P.pages_before from the groups' counts: a warp of every block of the first KV head takes some of the groups.
+__device__ __forceinline__ void leave_pages_before(const DecParams& P, int per, const long long* first) {
+  const int lane = threadIdx.x & 31;
+  for (int t = blockIdx.x; t < THREADS; t += gridDim.x) {
+    const int s1 = min((t + 1) * per, P.S);
+    long long at = first[t];
+    for (int s = t * per + lane; s - lane < s1; s += 32) {
+      const int n = s < s1 ? pages_of(P.seq_lens[s], P.max_blocks) : 0;
+      long long incl = n;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const long long x = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += x;
+      }
+      if (s < s1) P.pages_before[s] = at + incl - n;
+      at += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  if (blockIdx.x == 0 && lane == 0) P.pages_before[P.S] = first[THREADS];
+}
+
 // First page of share c when `total` pages are cut into n equal shares.
-__device__ __forceinline__ int share_begin(int total, int n, int c) { return (int)((long long)total * c / n); }
-// Shares of the flat walk: none may be empty, or a cut sequence would count a slot that nobody writes.
-__device__ __forceinline__ int flat_shares(int total, int n) { return min(total, n); }
+__device__ __forceinline__ long long share_begin(long long total, int n, int c) { return total * c / n; }
+// Shares of the flat walk: a page for each of a block's warps where there are enough (and none may be empty, or a cut
+// sequence would count a slot that nobody writes).
+__device__ __forceinline__ int flat_shares(long long total, int n) {
+  return (int)min((total + kConsumers - 1) / kConsumers, (long long)n);
+}
+// Slots for the partial results of S sequences cut into n shares, and the slot of a share's part of a sequence.  Along the
+// walk sequence and share never fall and one of them rises from one part to the next, so their sum tells the parts apart;
+// and a share holds at most two parts, the end of a sequence and the beginning of one.  Whichever takes less room.
+__host__ __device__ __forceinline__ int flat_slots(int S, int n) { return n + (S - 1 < n ? S - 1 : n); }
+__device__ __forceinline__ long long flat_slot(int S, int n, int seq, int share, bool begins) {
+  return S - 1 < n ? seq + share : 2 * share + (begins ? 1 : 0);
+}
 
 // What a block walks: runs of consecutive pages of one sequence.  Split by rank: one run, the rank's share of
 // sequence blockIdx.z.  Flat: the block's share of all sequences' pages laid end to end, cut at the sequences' ends.
@@ -145,15 +178,22 @@ template <bool kFlat>
 struct Walk {
   int seq, len, first, count;  // the current run: pages [first, first + count) of sequence seq
   bool whole;                  // ... which is all of the sequence
-  int page, end;               // flat: position in the end-to-end order
-  __device__ __forceinline__ bool next(const DecParams& P, const int* prefix) {
+  long long page, end;         // flat: position in the end-to-end order
+  long long before;            // flat: pages before sequence seq
+  __device__ __forceinline__ bool next(const DecParams& P) {
     if (page >= end) return false;
     if constexpr (kFlat) {
-      while (prefix[seq + 1] <= page) ++seq;
-      first = page - prefix[seq];
-      count = min(prefix[seq + 1], end) - page;
-      whole = first == 0 && page + count == prefix[seq + 1];
-      len = P.seq_lens[seq];
+      int n;
+      for (;; ++seq) {
+        if (seq >= P.S) return false;
+        len = P.seq_lens[seq];
+        n = pages_of(len, P.max_blocks);
+        if (before + n > page) break;
+        before += n;
+      }
+      first = (int)(page - before);
+      count = (int)(min(before + n, end) - page);
+      whole = count == n;
       page += count;
     } else {
       page = end;
@@ -162,11 +202,11 @@ struct Walk {
   }
 };
 
-// kFlat = false: grid (c, Hkv, S) in clusters of c blocks; the c blocks of a (sequence, KV head) share its pages
-// evenly, merge through distributed shared memory and write O.  No scratch, one launch.
+// kFlat = false: grid (c, Hkv, S); the c blocks of a (sequence, KV head) share its pages evenly.  They are a cluster, merge
+// through distributed shared memory and write O (no scratch, one launch), or (P.splits = c) leave partial results.
 // kFlat = true: grid (n, Hkv); block x takes the x-th of n equal shares of all sequences' pages laid end to end, so
 // that sequences of any lengths keep every block equally busy; a sequence that lies inside one share is finished
-// there, one that is cut leaves a partial result per share in slot seq + share, for decode_combine_kernel.
+// there, one that is cut leaves a partial result per share in its flat_slot, for decode_combine_kernel.
 template <bool kFlat>
 __global__ void __launch_bounds__(THREADS, 2)
 decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -176,7 +216,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
   const uint32_t bars = base + DecSmem::kOffBars;  // full[s] at + 8 s, empty[s] at + 8 (STAGES + s)
   float* merge = reinterpret_cast<float*>(gen + DecSmem::kOffMerge);
-  int* prefix = reinterpret_cast<int*>(gen + DecSmem::kOffFirst);
+  long long* first = reinterpret_cast<long long*>(gen + DecSmem::kOffFirst);
   const int hk = blockIdx.y, G = P.G;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -189,24 +229,27 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   }
   pdl_wait();  // nothing above touches global memory
   Walk<kFlat> start;
+  const int per = (P.S + THREADS - 1) / THREADS;  // flat: sequences per group of the page counts
   if constexpr (kFlat) {
-    page_prefix(P, prefix, reinterpret_cast<int*>(merge));
-    const int total = prefix[P.S], n = flat_shares(total, gridDim.x);
+    page_prefix(P, per, first, reinterpret_cast<long long*>(merge));
+    const long long total = first[THREADS];
+    const int n = flat_shares(total, gridDim.x);
     const bool busy = (int)blockIdx.x < n;
     start.page = busy ? share_begin(total, n, blockIdx.x) : 0;
     start.end = busy ? share_begin(total, n, blockIdx.x + 1) : 0;
-    int lo = 0, hi = P.S - 1;  // the sequence that holds the first page
+    int lo = 0, hi = THREADS - 1;  // the group that holds the first page
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (prefix[mid] <= start.page) lo = mid; else hi = mid - 1;
+      if (first[mid] <= start.page) lo = mid; else hi = mid - 1;
     }
-    start.seq = lo;
+    start.seq = lo * per;
+    start.before = first[lo];
   } else {
     start.seq = blockIdx.z;
     start.len = P.seq_lens[start.seq];
     const int n = pages_of(start.len, P.max_blocks);
-    start.first = share_begin(n, gridDim.x, blockIdx.x);
-    start.count = share_begin(n, gridDim.x, blockIdx.x + 1) - start.first;
+    start.first = (uint32_t)n * blockIdx.x / gridDim.x;  // (at most 2^25 pages, 32 blocks)
+    start.count = (uint32_t)n * (blockIdx.x + 1) / gridDim.x - start.first;
     start.whole = gridDim.x == 1;
     start.page = 0;
     start.end = 1;
@@ -218,7 +261,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     // ------------------------------------------------------------ producer
     Walk<kFlat> w = start;
     int i = 0;  // pages loaded so far
-    while (ok && w.next(P, prefix)) {
+    while (ok && w.next(P)) {
       const int32_t* row = P.table + (long long)w.seq * P.max_blocks;
       int32_t phys_mine = 0;
       for (int j = 0; j < w.count; ++j, ++i) {
@@ -243,13 +286,14 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       }
     }
     if (!ok && lane == 0) atomicExch(&g_decode_timeout, 1u);
+    if (kFlat && blockIdx.y == 0) leave_pages_before(P, per, first);  // (under the last pages' products)
   } else {
     // ------------------------------------------------------------ consumer: pages warp, warp + 3, ...
     const int g = lane >> 2, qc = lane & 3;   // query head (row of the padded 16 x 128 Q), column pair
     const int lr = lane & 7, lj = lane >> 3;  // ldmatrix: this lane supplies row lr of matrix lj
     Walk<kFlat> w = start;
     int i0 = 0;  // ring position of the run's first page
-    while (w.next(P, prefix)) {
+    while (w.next(P)) {
       // A fragments of Q for the 8 k-steps of 16 dims: rows 8..15 are padding (zero)
       uint32_t qa0[8], qa2[8];
       {
@@ -359,7 +403,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       i0 += w.count;
       // the warps' results for this run meet in shared memory
       if (g < G) {
-        float* mrow = merge + (warp * 8 + g) * (DD + 2);
+        float* mrow = merge + (warp * 8 + g) * kRow;
 #pragma unroll
         for (int nt = 0; nt < 16; ++nt) {
           mrow[8 * nt + 2 * qc] = o[nt][0];
@@ -374,30 +418,31 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       const bool alone = kFlat ? w.whole : gridDim.x == 1;
       // split by rank: this block's result goes over the (consumed) first stage of the ring, for its peers to read
       float* mine = reinterpret_cast<float*>(gen);
-      for (int idx = threadIdx.x; idx < G * DD; idx += kConsumers * 32) {
-        const int h = idx / DD, d = idx % DD;
+      const long long part = kFlat ? flat_slot(P.S, gridDim.x, w.seq, blockIdx.x, w.first == 0)
+                                   : (long long)w.seq * P.splits + blockIdx.x;
+      for (int idx = threadIdx.x; idx < G * (DD / 4); idx += kConsumers * 32) {
+        const int h = idx / (DD / 4), d = idx % (DD / 4) * 4;
         float M = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < kConsumers; ++u) M = fmaxf(M, merge[(u * 8 + h) * (DD + 2) + DD]);
-        float acc = 0.f, L = 0.f;
+        for (int u = 0; u < kConsumers; ++u) M = fmaxf(M, merge[(u * 8 + h) * kRow + DD]);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float L = 0.f;
 #pragma unroll
         for (int u = 0; u < kConsumers; ++u) {
-          const float* mrow = merge + (u * 8 + h) * (DD + 2);
-          const float wgt = mrow[DD] == -INFINITY ? 0.f : ex2(mrow[DD] - M);
-          acc += wgt * mrow[d];
-          L += wgt * mrow[DD + 1];
+          const float* mrow = merge + (u * 8 + h) * kRow;
+          add_weighted(acc, L, mrow[DD] == -INFINITY ? 0.f : ex2(mrow[DD] - M), *reinterpret_cast<const float4*>(mrow + d), mrow[DD + 1]);
         }
         if (alone) {
           write_row(P, (long long)w.seq * P.Hq + hk * G + h, d, acc, M, L);
-        } else if (kFlat) {
-          const long long slot = ((long long)w.seq + blockIdx.x) * P.Hq + hk * G + h;
-          P.part_o[slot * DD + d] = acc;
+        } else if (kFlat || P.splits) {
+          const long long slot = part * P.Hq + hk * G + h;
+          *reinterpret_cast<float4*>(P.part_o + slot * DD + d) = acc;
           if (d == 0) P.part_ml[slot] = make_float2(M, L);
         } else {
-          mine[h * (DD + 2) + d] = acc;
+          *reinterpret_cast<float4*>(mine + h * kRow + d) = acc;
           if (d == 0) {
-            mine[h * (DD + 2) + DD] = M;
-            mine[h * (DD + 2) + DD + 1] = L;
+            mine[h * kRow + DD] = M;
+            mine[h * kRow + DD + 1] = L;
           }
         }
       }
@@ -406,24 +451,23 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     if (!ok && lane == 0) atomicExch(&g_decode_timeout, 1u);
   }
   if constexpr (!kFlat) {
-    if (gridDim.x == 1) return;
+    if (gridDim.x == 1 || P.splits) return;
     // each block of the cluster merges its share of the G * 128 outputs over all the blocks' results
     cluster_sync();
-    const int c = gridDim.x, per = (G * DD + c - 1) / c;
-    const int lo = blockIdx.x * per, hi = min(lo + per, G * DD);
+    const int c = gridDim.x, per = (G * (DD / 4) + c - 1) / c;
+    const int lo = blockIdx.x * per, hi = min(lo + per, G * (DD / 4));
     for (int idx = lo + threadIdx.x; idx < hi; idx += THREADS) {
-      const int h = idx / DD, d = idx % DD;
-      const uint32_t ml_at = base + (h * (DD + 2) + DD) * 4, o_at = base + (h * (DD + 2) + d) * 4;
+      const int h = idx / (DD / 4), d = idx % (DD / 4) * 4;
+      const uint32_t ml_at = base + (h * kRow + DD) * 4, o_at = base + (h * kRow + d) * 4;
       float M = -INFINITY;
 #pragma unroll 8
       for (int r = 0; r < c; ++r) M = fmaxf(M, ld_cluster_f32(ml_at, r));
-      float acc = 0.f, L = 0.f;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float L = 0.f;
 #pragma unroll 8
       for (int r = 0; r < c; ++r) {
         const float m = ld_cluster_f32(ml_at, r);
-        const float wgt = m == -INFINITY ? 0.f : ex2(m - M);
-        acc += wgt * ld_cluster_f32(o_at, r);
-        L += wgt * ld_cluster_f32(ml_at + 4, r);
+        add_weighted(acc, L, m == -INFINITY ? 0.f : ex2(m - M), ld_cluster_v4(o_at, r), ld_cluster_f32(ml_at + 4, r));
       }
       write_row(P, (long long)blockIdx.z * P.Hq + hk * G + h, d, acc, M, L);
     }
@@ -431,49 +475,73 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   }
 }
 
-// Flat walk: one block per (sequence, KV head) adds up the partial results of a sequence that was cut; a warp
-// takes a query head, a lane four dims.  A sequence inside one share is finished already; an empty one has O = 0.
+// Adds up the partial results of sequences that were cut.  kWide: a block per (sequence, query head), whose warps share the
+// parts; otherwise a block per (sequence, KV head), a warp per query head.  A lane takes four dims.  In the flat walk a
+// sequence inside one share is finished already; an empty one has O = 0.
+template <bool kWide>
 __global__ void __launch_bounds__(THREADS)
 decode_combine_kernel(const __grid_constant__ DecParams P, int max_shares) {
-  __shared__ int first[kMaxFlatSeqs + 1];
-  __shared__ int tmp[THREADS / 32];
+  constexpr int kWarps = THREADS / 32, kStep = kWide ? kWarps : 1, kLoads = 8;  // parts in flight per warp
+  __shared__ float4 sums[kWide ? kWarps : 1][32];
+  __shared__ float2 stats[kWide ? kWarps : 1];
   pdl_wait();
-  page_prefix(P, first, tmp);
-  const int seq = blockIdx.x, hk = blockIdx.y, total = first[P.S], warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int a = first[seq], b = first[seq + 1], n = flat_shares(total, max_shares);
-  // the shares that hold the sequence's first and last page
-  const int c0 = b > a ? (int)((((long long)a + 1) * n - 1) / total) : 0;
-  const int c1 = b > a ? (int)(((long long)b * n - 1) / total) : 0;
-  if (b > a && c0 == c1) return;
-  for (int h = warp; h < P.G; h += THREADS / 32) {
-    const long long row = (long long)seq * P.Hq + hk * P.G + h;
+  const int seq = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int c0 = 0, cnt = P.splits;  // the shares that hold the sequence: the first, and how many
+  if (!P.splits) {
+    const long long a = P.pages_before[seq], b = P.pages_before[seq + 1], total = P.pages_before[P.S];
+    const int n = flat_shares(total, max_shares);
+    if (b > a) {
+      c0 = (int)(((a + 1) * n - 1) / total);
+      cnt = (int)((b * n - 1) / total) - c0 + 1;
+      if (cnt == 1) return;
+    }
+  }
+  const int h_begin = kWide ? blockIdx.y : blockIdx.y * P.G + warp, h_end = kWide ? h_begin + 1 : (blockIdx.y + 1) * P.G;
+  for (int h = h_begin; h < h_end; h += kWarps) {
+    auto slot_of = [&](int i) {
+      return (P.splits ? (long long)seq * P.splits + i : flat_slot(P.S, max_shares, seq, c0 + i, i == 0)) * P.Hq + h;
+    };
     float M = -INFINITY, L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (b > a) {
-      const long long slot0 = ((long long)seq + c0) * P.Hq + hk * P.G + h;
-      const int cnt = c1 - c0 + 1;
-      for (int i = lane; i < cnt; i += 32) M = fmaxf(M, P.part_ml[slot0 + (long long)i * P.Hq].x);
+    for (int i0 = kWide ? warp : 0; i0 < cnt; i0 += kLoads * kStep) {
+      float2 ml[kLoads];
+      float4 x[kLoads];
 #pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-#pragma unroll 8
-      for (int i = 0; i < cnt; ++i) {
-        const long long slot = slot0 + (long long)i * P.Hq;
-        const float2 ml = P.part_ml[slot];
-        const float4 x = reinterpret_cast<const float4*>(P.part_o + slot * DD)[lane];
-        const float wgt = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
-        acc.x += wgt * x.x, acc.y += wgt * x.y, acc.z += wgt * x.z, acc.w += wgt * x.w;
-        L += wgt * ml.y;
+      for (int u = 0; u < kLoads; ++u) {
+        const int i = i0 + u * kStep;
+        const long long slot = slot_of(min(i, cnt - 1));
+        ml[u] = P.part_ml[slot];
+        x[u] = reinterpret_cast<const float4*>(P.part_o + slot * DD)[lane];
+        if (i >= cnt) ml[u].x = -INFINITY;
       }
+      const float before = M;
+#pragma unroll
+      for (int u = 0; u < kLoads; ++u) M = fmaxf(M, ml[u].x);
+      const float f = before == -INFINITY ? 0.f : ex2(before - M);
+      acc.x *= f, acc.y *= f, acc.z *= f, acc.w *= f, L *= f;
+#pragma unroll
+      for (int u = 0; u < kLoads; ++u)
+        if (ml[u].x != -INFINITY) add_weighted(acc, L, ex2(ml[u].x - M), x[u], ml[u].y);
     }
-    reinterpret_cast<uint2*>(P.o + row * DD)[lane] =
-        L > 0.f ? make_uint2(pack_bf16(acc.x / L, acc.y / L), pack_bf16(acc.z / L, acc.w / L)) : make_uint2(0u, 0u);
-    if (P.lse && lane == 0) P.lse[row] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
+    if constexpr (kWide) {
+      sums[warp][lane] = acc;
+      if (lane == 0) stats[warp] = make_float2(M, L);
+      __syncthreads();
+      if (warp > 0) return;
+      M = -INFINITY, L = 0.f, acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) M = fmaxf(M, stats[w].x);
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w)
+        if (stats[w].x != -INFINITY) add_weighted(acc, L, ex2(stats[w].x - M), sums[w][lane], stats[w].y);
+    }
+    write_row(P, (long long)seq * P.Hq + h, lane * 4, acc, M, L);
   }
 }
 
 }  // namespace
 
-// Splits per sequence of the smallest scratch a call accepts: whole waves of 2 blocks per SM.
+// Blocks per (sequence, KV head) of the even split: whole waves of 2 blocks per SM.
 static int decode_num_splits(int S, int Hkv, int max_blocks) {
   constexpr int kMaxSplits = 32;
   const long long slots = (long long)sm_count() * 2;
@@ -495,32 +563,37 @@ static int decode_num_splits(int S, int Hkv, int max_blocks) {
 }
 
 namespace {
-constexpr size_t kSlotBytes = (DD + 2) * sizeof(float);  // per query head
+// Workspace of the flat walk: the sequences' page counts, then n shares' slots.
+size_t flat_counts_bytes(int S) { return ((size_t)S + 1) * sizeof(long long) / 16 * 16 + 16; }
+size_t flat_slot_bytes(int Hq) { return (size_t)Hq * (DD + 2) * sizeof(float); }
+size_t flat_bytes(int S, int Hq, int n) { return flat_counts_bytes(S) + (size_t)flat_slots(S, n) * flat_slot_bytes(Hq); }
 
-// How a decode call is cut.  flat = 0: clusters of `c` blocks per (sequence, KV head).  flat > 0: that many shares.
+// How a decode call is cut: into `flat` shares of all pages, or (flat = 0) every (sequence, KV head) into `c` blocks, a
+// cluster or (split) with partial results.  By sizes alone: the lengths are on the device.
 struct DecPlan {
   int c, flat;
+  bool split;
 };
-DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks) {
-  const long long slots = (long long)sm_count() * 2, pairs = (long long)S * Hkv;
+DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks, size_t ws_bytes) {
+  const long long slots = (long long)sm_count() * 2, pairs = (long long)S * Hkv, n = slots / Hkv;
+  // rounds of three pages (one for each consumer warp) that a block takes for `pages`, and for its share of one sequence
+  auto rounds_of = [](long long pages) { return (pages + kConsumers - 1) / kConsumers; };
+  auto rounds = [&](int c) { return rounds_of((max_blocks + c - 1) / c); };
   // few (sequence, KV head) pairs: enough blocks per pair to fill the chip, no more than shorten the walk of the
-  // longest possible sequence (a block's three consumer warps take three pages at a time)
-  auto rounds = [&](int c) { return ((max_blocks + c - 1) / c + kConsumers - 1) / kConsumers; };
+  // longest possible sequence
   int best = 1;
   for (int c = 2; c <= 16 && pairs * c <= slots; c *= 2)
     if (rounds(c) < rounds(best)) best = c;
-  // Up to four rounds a block stay with the clusters: a walk that short is all latency, and the flat walk pays for its
-  // page counts, the cut sequences' second kernel and a merge at every sequence's end (64 sequences of 20 to 500
-  // tokens: 33 us flat, 24 one block each).  Longer walks are bound by the memory system, and there an even share of
-  // the pages per block wins, the more so the more the lengths differ (17 sequences of 150 to 6000 tokens: 52 -> 44 us).
-  if (rounds(best) <= 4) return {best, 0};
-  const long long n = slots / Hkv;
-  const size_t need = (size_t)(S - 1 + n) * Hq * kSlotBytes;
-  // the flat walk's page counts have to fit (shared memory, 31 bits), and its partial results the built-in scratch
-  if (S > kMaxFlatSeqs || (long long)S * max_blocks > 0x7fffffffLL || n < 2 ||
-      need > (size_t)UNIGIST_DECODE_STATIC_SCRATCH_BYTES)
-    return {best, 0};
-  return {1, (int)n};
+  // Short walks stay with the clusters: they are all latency, and the flat walk pays for its page counts, the cut sequences'
+  // second kernel and a merge at every sequence's end (64 sequences of 20 to 500 tokens: 33 us flat, 21 one block each).
+  if (rounds(best) <= 4) return {best, 0, false};
+  // Longer walks are bound by the memory system, and there an even share of the pages per block wins, the more so the more
+  // the lengths differ (17 sequences of 150 to 6000 tokens: 41 -> 32 us; 127 of 800 and one of 131072, 16 KV heads: 480 us
+  // in equal parts of every sequence, 1190 one block each, 287 flat; 800 of 4096, 1 KV head: 260, 233, 246).
+  if (n >= 2 && flat_bytes(S, Hq, (int)n) <= ws_bytes) return {1, (int)n, false};
+  // more KV heads than SMs, or less scratch than the flat walk takes: the even split, whose scratch every call brings
+  const int even = decode_num_splits(S, Hkv, max_blocks);
+  return {even, 0, even > 1};
 }
 }  // namespace
 
@@ -529,8 +602,8 @@ size_t decode_min_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks) {
 }
 
 size_t decode_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks) {
-  const DecPlan plan = decode_plan(S, Hq, Hkv, max_blocks);
-  const size_t flat = plan.flat ? ((size_t)(S - 1 + plan.flat) * Hq * kSlotBytes + 255) / 256 * 256 : 0;
+  const DecPlan plan = decode_plan(S, Hq, Hkv, max_blocks, SIZE_MAX);
+  const size_t flat = plan.flat ? (flat_bytes(S, Hq, plan.flat) + 255) / 256 * 256 : 0;
   return std::max(decode_min_scratch_bytes(S, Hq, Hkv, D, max_blocks), flat);
 }
 
@@ -541,11 +614,7 @@ int32_t launch_decode(int S, int Hq, int Hkv, int D, float scale, const void* q,
   (void)D;
   const int G = Hq / Hkv;
   if (G < 1 || G > 8) return fail(UNIGIST_ERR_UNSUPPORTED, "decode supports 1 to 8 query heads per KV head, got %d", G);
-  DecPlan plan = decode_plan(S, Hq, Hkv, max_blocks);
-  if (plan.flat) {  // a caller with the least accepted scratch gets as many shares as it holds
-    const long long fit = (long long)(ws_bytes / ((size_t)Hq * kSlotBytes)) - S + 1;
-    if (fit < plan.flat) plan.flat = fit >= 2 ? (int)fit : 0;
-  }
+  const DecPlan plan = decode_plan(S, Hq, Hkv, max_blocks, ws_bytes);
   // the caches as 2-D tensors [num_blocks * Hkv * 64 tokens, 128 dims], tiles of 64 tokens x 64 dims
   CUtensorMap mk, mv;
   const long long rows = (long long)num_blocks * Hkv * PG;
@@ -558,25 +627,32 @@ int32_t launch_decode(int S, int Hq, int Hkv, int D, float scale, const void* q,
   P.holes = holes;
   P.o = (__nv_bfloat16*)o;
   P.lse = lse;
-  P.part_o = (float*)ws;
-  P.part_ml = reinterpret_cast<float2*>((float*)ws + (size_t)(plan.flat ? S - 1 + plan.flat : 0) * Hq * DD);
+  P.pages_before = (long long*)ws;
+  P.splits = plan.split ? plan.c : 0;
+  P.part_o = reinterpret_cast<float*>((char*)ws + (plan.flat ? flat_counts_bytes(S) : 0));
+  const size_t parts = plan.flat ? flat_slots(S, plan.flat) : (size_t)S * P.splits;
+  P.part_ml = reinterpret_cast<float2*>(P.part_o + parts * Hq * DD);
   P.S = S, P.Hq = Hq, P.Hkv = Hkv, P.G = G, P.num_blocks = num_blocks, P.max_blocks = max_blocks;
   P.holes_stride = holes_stride, P.holes_off = holes_off;
   P.scale_log2 = scale * LOG2E;
   const auto kern = plan.flat ? decode_split_kernel<true> : decode_split_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem::kBytes);
-  if (e == cudaSuccess && plan.c > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  const int cluster = plan.flat || plan.split ? 1 : plan.c;
+  if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return fail(UNIGIST_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   {
     KernelScope ks("decode_split_kernel", st);
-    launch_chained(kern, plan.flat ? dim3(plan.flat, Hkv) : dim3(plan.c, Hkv, S), THREADS, DecSmem::kBytes, st,
-                   plan.flat ? 1 : plan.c, mk, mv, P);
+    launch_chained(kern, plan.flat ? dim3(plan.flat, Hkv) : dim3(plan.c, Hkv, S), THREADS, DecSmem::kBytes, st, cluster, mk, mv,
+                   P);
   }
   if (int32_t rc = check_launch("decode split kernel")) return rc;
-  if (!plan.flat) return UNIGIST_OK;
+  if (!plan.flat && !plan.split) return UNIGIST_OK;
   {
     KernelScope ks("decode_combine_kernel", st);
-    launch_chained(decode_combine_kernel, dim3(S, Hkv), THREADS, 0, st, 1, P, plan.flat);
+    // a block per query head while they are few: with many sequences a sequence has few parts
+    const bool wide = (long long)S * Hq <= 4ll * sm_count();
+    launch_chained(wide ? decode_combine_kernel<true> : decode_combine_kernel<false>, dim3(S, wide ? Hq : Hkv), THREADS, 0, st, 1, P,
+                   plan.flat);
   }
   return check_launch("decode combine kernel");
 }

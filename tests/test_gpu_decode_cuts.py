@@ -1,6 +1,7 @@
-"""Every way a decode call is cut, against the oracle: clusters of 1 to 16 blocks per (sequence, KV head), the flat walk
-over all sequences' pages (fewer pages than shares, sequences inside one share, cut once and cut many times, empty
-ones between them), and the least scratch that is accepted."""
+"""Every way a decode call is cut, against the oracle: clusters of 1 to 16 blocks per (sequence, KV head), the even split
+with a second kernel, the flat walk over all sequences' pages (fewer pages than shares, sequences inside one share, cut once
+and cut many times, empty ones between them, more sequences than a block has threads), and every size of scratch from the
+least that is accepted."""
 import numpy as np
 import pytest
 import torch
@@ -26,12 +27,14 @@ CASES = [
     (4, 4, [40 + 3 * i for i in range(80)], 7),                         # many short walks: one block each
     (1, 1, [(37 * i) % 300 for i in range(300)], 20),                   # three sequences per thread in the page counts
     (1, 1, [(37 * i) % 300 for i in range(384)], 20),                   # ... with the runs ending at the last sequence
+    (1, 1, [(37 * i) % 300 for i in range(769)], 20),                   # seven, the last threads without any
+    (2, 1, [5000] + [(29 * i) % 150 for i in range(1099)] + [64 * 70], 90),  # long sequences among short ones
+    (64, 8, [40 + 7 * (i % 30) for i in range(230)], 80),               # more than 8 MiB of scratch asked for
+    (160, 160, [900, 17], 40),                                          # more KV heads than SMs
 ]
 
 
-@pytest.mark.parametrize("least", [False, True])
-@pytest.mark.parametrize("Hq,Hkv,lens,width", CASES)
-def test_decode_cuts(Hq, Hkv, lens, width, least):
+def _inputs(Hq, Hkv, lens, width):
     S, D = len(lens), 128
     g = torch.Generator().manual_seed(S * 1000 + width)
     used = [-(-n // PG) for n in lens]
@@ -44,13 +47,34 @@ def test_decode_cuts(Hq, Hkv, lens, width, least):
         table[i, :n] = order[at:at + n]
         at += n
     q = torch.randn(S, Hq, D, generator=g).to(torch.bfloat16)
+    return q, kc, vc, table, torch.tensor(lens, dtype=torch.int32)
+
+
+def _check(inputs, o, lse):
+    q, kc, vc, table, lens = inputs
+    Hkv, D = kc.shape[1], 128
+    for i, n in enumerate(lens.tolist()):
+        if n == 0:
+            assert (o[i] == 0).all() and (lse[i] == -np.inf).all()
+            continue
+        kl, vl = (f64(c[table[i, :-(-n // PG)].long()].permute(0, 2, 1, 3).reshape(-1, Hkv, D)[:n]) for c in (kc, vc))
+        oo, ll = oracle.decode(D ** -0.5, f64(q[i:i + 1]), [kl], [vl])
+        check_close(f"O of sequence {i}", f64(o[i:i + 1]), oo, TOL_O_MAX, TOL_O_MEAN)
+        check_close(f"LSE of sequence {i}", f64(lse[i:i + 1]), ll, TOL_LSE)
+
+
+@pytest.mark.parametrize("least", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,lens,width", CASES)
+def test_decode_cuts(Hq, Hkv, lens, width, least):
+    S, D = len(lens), 128
+    inputs = _inputs(Hq, Hkv, lens, width)
     size = ug.unigist_decode_workspace_bytes(S, Hq, Hkv, D, width)
     if least:  # what one partial result per sequence and query head takes, or as much more as the call insists on
         size = -(-S * Hq * (D + 2) * 4 // 256) * 256
     ws = torch.empty(size, dtype=torch.uint8, device=DEV)
     o = torch.full((S, Hq, D), float("nan"), dtype=torch.bfloat16, device=DEV)
     lse = torch.full((S, Hq), float("nan"), dtype=torch.float32, device=DEV)
-    args = [x.to(DEV) for x in (q, kc, vc, table, torch.tensor(lens, dtype=torch.int32))]
+    args = [x.to(DEV) for x in inputs]
     try:
         ug.unigist_decode(*args, o, lse, ws)
     except ug.UnigistError as e:
@@ -60,14 +84,35 @@ def test_decode_cuts(Hq, Hkv, lens, width, least):
         ug.unigist_decode(*args, o, lse, torch.empty(need, dtype=torch.uint8, device=DEV))
     torch.cuda.synchronize()
     ug.unigist_device_status()
-    for i, n in enumerate(lens):
-        if n == 0:
-            assert (o[i] == 0).all() and (lse[i] == -np.inf).all()
+    _check(inputs, o, lse)
+
+
+@pytest.mark.parametrize("Hq,Hkv,lens,width", [(32, 8, [64 * 3 * (i % 5) + 1 for i in range(37)], 144),  # one part each suffices
+                                               (8, 1, [64 * 20 + i for i in range(5)], 300),
+                                               (8, 8, [700] * 40, 47)])
+def test_every_size_of_scratch(Hq, Hkv, lens, width):
+    """From the least that is accepted to more than is asked for, in steps that do not divide the parts."""
+    S, D = len(lens), 128
+    inputs = _inputs(Hq, Hkv, lens, width)
+    args = [x.to(DEV) for x in inputs]
+    o = torch.empty(S, Hq, D, dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty(S, Hq, dtype=torch.float32, device=DEV)
+    with pytest.raises(ug.UnigistError) as e:
+        ug.unigist_decode(*args, o, lse, torch.empty(256, dtype=torch.uint8, device=DEV))
+    least = int(str(e.value).split("decode needs ")[1].split()[0])
+    ideal = ug.unigist_decode_workspace_bytes(S, Hq, Hkv, D, width)
+    assert least <= ideal
+    guard = 4096
+    for size in sorted({least, least + 16, 655360, (least + ideal) // 2 // 16 * 16, ideal - 16, ideal, ideal + 100000}):
+        if size < least:
             continue
-        kl, vl = (f64(c[table[i, :used[i]].long()].permute(0, 2, 1, 3).reshape(-1, Hkv, D)[:n]) for c in (kc, vc))
-        oo, ll = oracle.decode(D ** -0.5, f64(q[i:i + 1]), [kl], [vl])
-        check_close(f"O of sequence {i}", f64(o[i:i + 1]), oo, TOL_O_MAX, TOL_O_MEAN)
-        check_close(f"LSE of sequence {i}", f64(lse[i:i + 1]), ll, TOL_LSE)
+        buf = torch.full((size + guard,), 0xA5, dtype=torch.uint8, device=DEV)
+        o.fill_(float("nan"))
+        lse.fill_(float("nan"))
+        ug.unigist_decode(*args, o, lse, buf[:size])
+        torch.cuda.synchronize()
+        assert (buf[size:] == 0xA5).all()  # nothing behind the workspace
+        _check(inputs, o, lse)
 
 
 @pytest.mark.parametrize("width", [3, 9, 700])  # one block, a cluster, the flat walk
