@@ -13,6 +13,7 @@
 //                   with warp-level mma (m16n8k16, query heads padded to 16 rows), fragments
 //                   fetched with ldmatrix.  The warps merge once, at the end.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "sm100_ptx.cuh"
@@ -568,6 +569,40 @@ size_t flat_counts_bytes(int S) { return ((size_t)S + 1) * sizeof(long long) / 1
 size_t flat_slot_bytes(int Hq) { return (size_t)Hq * (DD + 2) * sizeof(float); }
 size_t flat_bytes(int S, int Hq, int n) { return flat_counts_bytes(S) + (size_t)flat_slots(S, n) * flat_slot_bytes(Hq); }
 
+// Clusters of c = 2, 4, 8 or 16 blocks that the current device holds at once (asked once per device): fewer than its SMs
+// have room for, since a cluster does not leave its group of SMs.  Without a device, what the B200 says.
+int max_clusters(int c) {
+  constexpr int kMaxDevices = 64, kB200[4] = {148, 71, 33, 14};
+  static std::atomic<int> cached[kMaxDevices][4];  // 0 = not asked yet
+  const int i = c == 2 ? 0 : c == 4 ? 1 : c == 8 ? 2 : 3;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+    cudaGetLastError();
+    return kB200[i];
+  }
+  int n = cached[dev][i].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  const auto kern = decode_split_kernel<false>;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = c;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(c);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = DecSmem::kBytes;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem::kBytes) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return kB200[i];
+  }
+  cached[dev][i].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 // How a decode call is cut: into `flat` shares of all pages, or (flat = 0) every (sequence, KV head) into `c` blocks, a
 // cluster or (split) with partial results.  By sizes alone: the lengths are on the device.
 struct DecPlan {
@@ -579,10 +614,11 @@ DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks, size_t ws_bytes) {
   // rounds of three pages (one for each consumer warp) that a block takes for `pages`, and for its share of one sequence
   auto rounds_of = [](long long pages) { return (pages + kConsumers - 1) / kConsumers; };
   auto rounds = [&](int c) { return rounds_of((max_blocks + c - 1) / c); };
-  // few (sequence, KV head) pairs: enough blocks per pair to fill the chip, no more than shorten the walk of the
-  // longest possible sequence
+  // Few (sequence, KV head) pairs: a cluster for each, no larger than shortens the walk of the longest possible sequence
+  // and than the chip holds for all pairs at once (two sequences of 5120 tokens, 8 KV heads: 15.3 us in 16 clusters of 16
+  // of which 14 fit, 10.4 in clusters of 8).
   int best = 1;
-  for (int c = 2; c <= 16 && pairs * c <= slots; c *= 2)
+  for (int c = 2; c <= 16 && pairs <= max_clusters(c); c *= 2)
     if (rounds(c) < rounds(best)) best = c;
   // Short walks stay with the clusters: they are all latency, and the flat walk pays for its page counts, the cut sequences'
   // second kernel and a merge at every sequence's end (64 sequences of 20 to 500 tokens: 33 us flat, 21 one block each).

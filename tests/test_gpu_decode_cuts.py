@@ -30,6 +30,7 @@ CASES = [
     (1, 1, [(37 * i) % 300 for i in range(769)], 20),                   # seven, the last threads without any
     (2, 1, [5000] + [(29 * i) % 150 for i in range(1099)] + [64 * 70], 90),  # long sequences among short ones
     (64, 8, [40 + 7 * (i % 30) for i in range(230)], 80),               # more than 8 MiB of scratch asked for
+    (32, 8, [64 * 79 + 1, 3], 80),                                      # more clusters of 16 than fit
     (160, 160, [900, 17], 40),                                          # more KV heads than SMs
 ]
 
