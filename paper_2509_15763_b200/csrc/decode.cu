@@ -616,13 +616,24 @@ DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks, size_t ws_bytes) {
   auto rounds = [&](int c) { return rounds_of((max_blocks + c - 1) / c); };
   // Few (sequence, KV head) pairs: a cluster for each, no larger than shortens the walk of the longest possible sequence
   // and than the chip holds for all pairs at once (two sequences of 5120 tokens, 8 KV heads: 15.3 us in 16 clusters of 16
-  // of which 14 fit, 10.4 in clusters of 8).
+  // of which 14 fit, 9.3 as below).
   int best = 1;
   for (int c = 2; c <= 16 && pairs <= max_clusters(c); c *= 2)
     if (rounds(c) < rounds(best)) best = c;
+  // Very few pairs and a longer walk: the even split puts more blocks on it than clusters can, which pays for its second
+  // kernel (1.5 us) from three rounds on where it saves one (one sequence, 8 KV heads: 9216 tokens 11.0 -> 9.1 us; 6400
+  // 10.1 -> 8.4).  Past six rounds the flat walk's even shares are worth their page counts and merges (4 sequences of 9216:
+  // 19.3 us in six rounds, 21.4 flat; 8: 40.7 flat), for one sequence, which has no other to even out, past two more than it
+  // takes (65536 tokens, 8 KV heads: 35.7 us split, 37.8 flat; one of 131072, 1 KV head: 35 and 21).
+  if (rounds(best) >= 3) {
+    const int even = decode_num_splits(S, Hkv, max_blocks);
+    const long long most = S == 1 && n >= 2 ? std::max(6ll, rounds_of((max_blocks + n - 1) / n) + 2) : 6;
+    if (pairs * even <= slots && rounds(even) < rounds(best) && rounds(even) <= most) return {even, 0, true};
+  }
   // Short walks stay with the clusters: they are all latency, and the flat walk pays for its page counts, the cut sequences'
-  // second kernel and a merge at every sequence's end (64 sequences of 20 to 500 tokens: 33 us flat, 21 one block each).
-  if (rounds(best) <= 4) return {best, 0, false};
+  // second kernel and a merge at every sequence's end (64 sequences of 20 to 500 tokens: 33 us flat, 21 one block each; 18
+  // of up to 2304 in clusters of two: 17.1 flat, 14.8).
+  if (rounds(best) <= (pairs * best <= slots ? 6 : 4)) return {best, 0, false};
   // Longer walks are bound by the memory system, and there an even share of the pages per block wins, the more so the more
   // the lengths differ (17 sequences of 150 to 6000 tokens: 41 -> 32 us; 127 of 800 and one of 131072, 16 KV heads: 480 us
   // in equal parts of every sequence, 1190 one block each, 287 flat; 800 of 4096, 1 KV head: 260, 233, 246).

@@ -30,6 +30,8 @@ CASES = [
     (1, 1, [(37 * i) % 300 for i in range(769)], 20),                   # seven, the last threads without any
     (2, 1, [5000] + [(29 * i) % 150 for i in range(1099)] + [64 * 70], 90),  # long sequences among short ones
     (64, 8, [40 + 7 * (i % 30) for i in range(230)], 80),               # more than 8 MiB of scratch asked for
+    (8, 1, [64 * 192], 192), (8, 2, [6400, 0], 100), (32, 8, [64 * 99 + 5], 144),  # few pairs: the even split
+    (8, 1, [0], 192), (8, 1, [1], 192),                                 # ... of nothing, of one page
     (32, 8, [64 * 79 + 1, 3], 80),                                      # more clusters of 16 than fit
     (160, 160, [900, 17], 40),                                          # more KV heads than SMs
 ]
@@ -116,7 +118,7 @@ def test_every_size_of_scratch(Hq, Hkv, lens, width):
         _check(inputs, o, lse)
 
 
-@pytest.mark.parametrize("width", [3, 9, 700])  # one block, a cluster, the flat walk
+@pytest.mark.parametrize("width", [3, 9, 100, 700])  # one block, a cluster, the even split, the flat walk
 @pytest.mark.parametrize("n", [1, 130])
 def test_infinities_in_v(width, n):
     """A visible infinity in V comes out as that infinity (both signs in one column: NaN), whatever the rounding of its
