@@ -4,8 +4,8 @@
 //                              dQ accumulator of the fused kernel.
 // head_dim 128: attn_bwd_fused_sm100_kernel (described where it is defined) and dq_convert_kernel.
 // head_dim 64: two kernels (a 64-row dQ^T accumulator would halve the fused kernel's tensor throughput):
-//   attn_bwd_dkdv_sm100_kernel one thread block owns a 128-key tile of one KV head (two blocks of a cluster share a
-//                              sink or gist key tile) and walks every
+//   attn_bwd_dkdv_sm100_kernel one thread block owns a 128-key tile of one KV head (where a walk would be the tail, two
+//                              blocks of a cluster share a sink or gist key tile) and walks every
 //                              128-query tile of every query head of the group that can see it:
 //                              S^T = K Q^T and dP^T = V dO^T (TMEM), P^T = exp2(S^T c - LSE),
 //                              dS^T = P^T o (dP^T - Delta), dV += P^T dO, dK += dS^T Q.  dK and dV
@@ -225,7 +225,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
                            const __grid_constant__ CUtensorMap tm_v_raw, const __grid_constant__ CUtensorMap tm_v_gist,
                            Geom g, int Hq, int Hkv, float scale, const float* __restrict__ lse,
                            const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk,
-                           __nv_bfloat16* __restrict__ dv, int n_sink_kt, int n_gist_kt, int n_raw_kt, int pairs,
+                           __nv_bfloat16* __restrict__ dv, int n_sink_kt, int n_gist_kt, int n_raw_kt, int pairs, int shared,
                            FastDiv heavy_div, FastDiv raw_div, FastDiv hkv_div) {
   using SM = KvSmem<D>;
   extern __shared__ unsigned char smem_dyn[];
@@ -244,21 +244,21 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = Hq / Hkv;
-  // Blocks come in clusters of two.  Sink and gist key tiles are seen by every later query: heaviest, and first over ALL
-  // heads and batch indices (a long walk that starts late is the kernel's tail); the two blocks of a cluster share ONE
-  // such key tile, each walks half of its queries, and they add their dK and dV through distributed shared memory (the
-  // longest walk was 1.3 times an SM's share of all steps on the problem above).  Of the raw key tiles either block of a
-  // cluster takes one of its own.  The tiles of one KV head are neighbours and share its Q and dO.
-  const int n_heavy = n_sink_kt + n_gist_kt, crank = blockIdx.x & 1, cluster = blockIdx.x >> 1;
-  const bool split = cluster < n_heavy * pairs;
+  // Sink and gist key tiles are seen by every later query: heaviest, and first over ALL heads and batch indices (a long walk
+  // that starts late is the kernel's tail).  Where even that leaves a long walk as the tail (dkdv_shares), blocks come in
+  // clusters of two: they share ONE such key tile, each walks half of its queries, and they add their dK and dV through
+  // distributed shared memory; of the raw key tiles either block of a cluster takes one of its own.  The tiles of one KV
+  // head are neighbours and share its Q and dO.
+  const int n_heavy = n_sink_kt + n_gist_kt, crank = shared ? blockIdx.x & 1 : 0, unit = blockIdx.x >> shared;
+  const bool split = shared && unit < n_heavy * pairs;
   int pair, rank;  // pair = batch index * Hkv + KV head
-  if (split) {
-    pair = fdiv(heavy_div, cluster);
-    rank = cluster - pair * n_heavy;
+  if (unit < n_heavy * pairs) {
+    pair = fdiv(heavy_div, unit);
+    rank = unit - pair * n_heavy;
   } else {
-    const int y = cluster - n_heavy * pairs;
+    const int y = unit - n_heavy * pairs;
     pair = fdiv(raw_div, y);
-    rank = n_heavy + 2 * (y - pair * ((n_raw_kt + 1) / 2)) + crank;
+    rank = n_heavy + ((y - pair * ((n_raw_kt + shared) >> shared)) << shared) + crank;
     if (rank >= n_heavy + n_raw_kt) return;  // an odd number of raw key tiles (its cluster never meets)
   }
   const int b = fdiv(hkv_div, pair), hk = pair - b * Hkv;
@@ -1665,6 +1665,21 @@ int32_t launch_dkdv_reduce(const BwdRun& R, int batch, const unigist_problem& p,
   return check_launch("dK/dV reduce kernel");
 }
 
+// Whether two blocks share each sink or gist key tile of the dK / dV kernel: where the longest walk (the first gist key tile's)
+// would otherwise be the kernel's tail.  All blocks' steps are counted to within a tile, per SM; a walk up to 3/4 of that and
+// 22 steps ends under the raw key tiles that are left, and sharing it only costs blocks (us of the whole backward, shared and
+// not; steps of the longest walk / of an SM: 1 x 8190 raw tokens, 16 / 4 heads, 296 / 102: 305 and 456; 2 x 8190, 296 / 205: 529
+// and 577; 2 x 12288, ratio 3, 384 / 396: 1058 and 1150; 4 x 8190, 296 / 411: 1043 and 1005; 8 x 2048, 80 / 105: 301 and 283; 256
+// x 128, 8 / 83: 618 and 422; 1 x 448, one head, 5 / 0: 23.8 and 21.9).
+bool dkdv_shares(const Geom& g, int batch, int Hq, int Hkv) {
+  auto tiles = [](long long rows) { return (rows + 127) / 128; };
+  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n), all = sink + raw + gist, G = Hq / Hkv;
+  // a gist key is seen by the later half of all rows on average, a raw key by k + 1 units and their gists
+  const long long window = std::min(tiles((g.k + 1ll) * g.r) + 1, raw) + std::min(tiles(g.k + 1ll) + 1, gist);
+  const long long steps = (sink * all + gist * (raw + gist + 1) / 2 + raw * window) * Hq * batch / sm_count();
+  return all * G > steps * 3 / 4 + 22;
+}
+
 // The two-kernel backward (head_dim 64; head_dim 128 when dQ has to be the same bit for bit from run to run): a
 // block of the first kernel owns a key tile (dK, dV), a block of the second a query tile (dQ, over 64-key tiles).
 template <int D>
@@ -1694,11 +1709,11 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
   {
     KernelScope ks("attn_bwd_dkdv_sm100_kernel", st);
     const int pairs = B * Hkv, n_heavy = n_sink_t + n_gist_t;
-    const int raw_clusters = (n_raw_t + 1) / 2;
-    launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(2 * (n_heavy + raw_clusters) * pairs), kKvThreads, KvSmem<D>::kBytes,
-                   st, 2, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale, lse, delta,
-        (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, make_fastdiv(n_heavy),
-        make_fastdiv(raw_clusters), make_fastdiv(Hkv));
+    const int shared = dkdv_shares(g, B, Hq, Hkv) ? 1 : 0, raw_units = (n_raw_t + shared) >> shared;
+    launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(((n_heavy + raw_units) * pairs) << shared), kKvThreads, KvSmem<D>::kBytes,
+                   st, 1 << shared, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale,
+                   lse, delta, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, shared,
+                   make_fastdiv(n_heavy), make_fastdiv(raw_units), make_fastdiv(Hkv));
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {

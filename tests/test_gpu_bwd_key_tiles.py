@@ -1,6 +1,6 @@
-"""The two-kernel backward's clusters against the oracle: a sink or gist key tile is walked by two blocks (an odd number of
-query tiles, a single one, so that the second block has none), raw key tiles are dealt out two to a cluster (an odd number
-of them, a single one), heads and batch indices share the block order; twice, bit for bit."""
+"""The two-kernel backward's blocks against the oracle: a sink or gist key tile is walked by one block or shared by the two of
+a cluster (an odd number of query tiles, a single one, so that the second block has none), raw key tiles are then dealt out
+two to a cluster (an odd number of them, a single one), heads and batch indices share the block order; twice, bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -21,6 +21,13 @@ CASES = [
     synth.Workload("two_gist_tiles", 1, 130 * 5, 5, 35, 8, 2, 64, num_sinks=130, seed=505),
     synth.Workload("two_gist_tiles_128", 1, 130 * 5, 5, 35, 4, 2, 128, num_sinks=130, seed=506),
     synth.Workload("odd_raw_128", 2, 3 * 128 + 7, 1, 50, 2, 1, 128, seed=507),
+    # walks of more than 22 steps (query tiles times heads of a group): these are shared
+    synth.Workload("shared_one_tile_each", 1, 9, 3, 6, 12, 1, 64, seed=511),
+    synth.Workload("shared_sinks_only_tile", 1, 4, 4, 4, 8, 1, 64, num_sinks=3, seed=512),
+    synth.Workload("shared_odd_raw_tiles", 2, 3 * 128, 3, 60, 12, 2, 64, seed=513),
+    synth.Workload("shared_odd_raw_ragged", 3, 4 * 128 + 8, 8, 100, 15, 3, 64, num_sinks=1, seed=514),
+    synth.Workload("shared_two_gist_tiles_128", 1, 130 * 5, 5, 35, 8, 2, 128, num_sinks=130, seed=516),
+    synth.Workload("shared_odd_raw_128", 2, 3 * 128 + 7, 1, 50, 8, 1, 128, seed=517),
 ]
 
 
