@@ -287,7 +287,6 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       }
     }
     if (!ok && lane == 0) atomicExch(&g_decode_timeout, 1u);
-    if (kFlat && blockIdx.y == 0) leave_pages_before(P, per, first);  // (under the last pages' products)
   } else {
     // ------------------------------------------------------------ consumer: pages warp, warp + 3, ...
     const int g = lane >> 2, qc = lane & 3;   // query head (row of the padded 16 x 128 Q), column pair
@@ -450,6 +449,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       if (kFlat) named_barrier_sync(1, kConsumers * 32);  // `merge` is free for the next run
     }
     if (!ok && lane == 0) atomicExch(&g_decode_timeout, 1u);
+    if (kFlat && warp == 0 && blockIdx.y == 0) leave_pages_before(P, per, first);
   }
   if constexpr (!kFlat) {
     if (gridDim.x == 1 || P.splits) return;
