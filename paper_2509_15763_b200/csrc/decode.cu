@@ -609,6 +609,7 @@ struct DecPlan {
   int c, flat;
   bool split;
 };
+constexpr int kMaxShortRounds = 4;  // the longest walk that more blocks than fit at once still take as one block each
 DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks, size_t ws_bytes) {
   const long long slots = (long long)sm_count() * 2, pairs = (long long)S * Hkv, n = slots / Hkv;
   // rounds of three pages (one for each consumer warp) that a block takes for `pages`, and for its share of one sequence
@@ -633,7 +634,7 @@ DecPlan decode_plan(int S, int Hq, int Hkv, int max_blocks, size_t ws_bytes) {
   // Short walks stay with the clusters: they are all latency, and the flat walk pays for its page counts, the cut sequences'
   // second kernel and a merge at every sequence's end (64 sequences of 20 to 500 tokens: 33 us flat, 21 one block each; 18
   // of up to 2304 in clusters of two: 17.1 flat, 14.8).
-  if (rounds(best) <= (pairs * best <= slots ? 6 : 4)) return {best, 0, false};
+  if (rounds(best) <= (pairs * best <= slots ? 6 : kMaxShortRounds)) return {best, 0, false};
   // Longer walks are bound by the memory system, and there an even share of the pages per block wins, the more so the more
   // the lengths differ (17 sequences of 150 to 6000 tokens: 41 -> 32 us; 127 of 800 and one of 131072, 16 KV heads: 480 us
   // in equal parts of every sequence, 1190 one block each, 287 flat; 800 of 4096, 1 KV head: 260, 233, 246).
@@ -648,9 +649,11 @@ size_t decode_min_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks) {
   return ((size_t)S * Hq * decode_num_splits(S, Hkv, max_blocks) * (D + 2) * sizeof(float) + 255) / 256 * 256;
 }
 
+// What the plan may use, whichever it is on the device of the call: a size query asks no more of a device than its SM count
+// (the clusters it holds cannot be asked for without making a context on it).
 size_t decode_scratch_bytes(int S, int Hq, int Hkv, int D, int max_blocks) {
-  const DecPlan plan = decode_plan(S, Hq, Hkv, max_blocks, SIZE_MAX);
-  const size_t flat = plan.flat ? (flat_bytes(S, Hq, plan.flat) + 255) / 256 * 256 : 0;
+  const int n = sm_count() * 2 / Hkv;
+  const size_t flat = n >= 2 && max_blocks > kMaxShortRounds * kConsumers ? (flat_bytes(S, Hq, n) + 255) / 256 * 256 : 0;
   return std::max(decode_min_scratch_bytes(S, Hq, Hkv, D, max_blocks), flat);
 }
 

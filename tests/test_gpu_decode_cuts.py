@@ -88,6 +88,10 @@ def test_decode_cuts(Hq, Hkv, lens, width, least):
     torch.cuda.synchronize()
     ug.unigist_device_status()
     _check(inputs, o, lse)
+    if not least and size <= ug.DECODE_STATIC_SCRATCH_BYTES:  # the same cut, bit for bit, with the built-in scratch
+        o2, lse2 = torch.full_like(o, float("nan")), torch.full_like(lse, float("nan"))
+        ug.unigist_decode_static(*args, o2, lse2)
+        assert torch.equal(o, o2) and torch.equal(lse, lse2)
 
 
 @pytest.mark.parametrize("Hq,Hkv,lens,width", [(32, 8, [64 * 3 * (i % 5) + 1 for i in range(37)], 144),  # one part each suffices
