@@ -157,9 +157,10 @@ struct KernelScope {
   int slot;
   cudaStream_t st;
 };
-// Launches a kernel whose first access to global memory comes after pdl_wait(): it may become resident as the one before
-// it on the stream drains, so that launch latency and prologue are hidden.  cluster > 1: blocks along x in clusters of
-// that many.  An error is picked up by check_launch.
+// Launches a kernel whose first access to global memory comes after pdl_wait(): its launch is prepared while the one before
+// it on the stream runs, and its blocks start once the last block of that one has ended (none lets its successor in
+// earlier, see above), so that launch latency is hidden and the prologue runs while the predecessor's writes are made
+// visible.  cluster > 1: blocks along x in clusters of that many.  An error is picked up by check_launch.
 template <typename T>
 struct AsIs {
   using type = T;

@@ -23,6 +23,8 @@ CASES = [
     (1, 3, 40, 1, 3, 2, 2, 5),        # ratio 1
     (2, 0, 120, 8, 1000, 8, 2, 2),    # the window never fills: nothing is ever evicted
     (1, 130, 70, 7, 15, 4, 4, 1),     # sinks over two pages, window of ceil(15 / 7) = 3 units
+    (2, 0, 24, 4, 8, 16, 16, 1),      # 16 and 32 KV heads: a token's rows are more than a block's threads copy at once
+    (1, 2, 20, 4, 4, 32, 32, 2),
 ]
 
 
@@ -146,3 +148,36 @@ def test_append_to_a_length_below_zero_writes_no_row():
         assert (cache[3, :, 5] == 1).all()
         cache[3, :, 5] = 0
         assert (cache == 0).all()
+
+
+@pytest.mark.parametrize("width", [6, 100, 700])  # one block or a cluster, the even split, the flat walk
+@pytest.mark.parametrize("holes", [0, 5, 40])
+def test_freed_slots_are_left_out_however_the_call_is_cut(width, holes):
+    B, Hq, Hkv, D, r = 3, 8, 2, 128, 64
+    p = ug.Problem(B, 2 * r, r, r, Hq, Hkv, D)
+    g = torch.Generator().manual_seed(holes + width)
+    lens = [330, 200, 65]
+    kc, vc = (torch.randn(B * 6, Hkv, PG, D, generator=g).to(torch.bfloat16) for _ in range(2))
+    table = torch.zeros(B, width, dtype=torch.int32)
+    table[:, :6] = torch.randperm(B * 6, generator=g).reshape(B, 6).to(torch.int32)
+    ints = 8 + 2 * r + r  # header, the ring of a window of one unit, the free list
+    state = torch.full((B, ints), -1, dtype=torch.int32)
+    assert ug.unigist_cache_state_bytes(p) >= state.numel() * 4
+    state[:, :5] = 0
+    freed = []
+    for b in range(B):  # the free list: [2] entries, behind the window's ring
+        freed.append(torch.randperm(lens[b], generator=g)[:holes])
+        state[b, 2] = holes
+        state[b, ints - r: ints - r + holes] = freed[b].to(torch.int32)
+    q = torch.randn(B, Hq, D, generator=g).to(torch.bfloat16)
+    o = torch.zeros(B, Hq, D, dtype=torch.bfloat16, device=DEV)
+    lse = torch.zeros(B, Hq, dtype=torch.float32, device=DEV)
+    ws = torch.empty(ug.unigist_decode_workspace_bytes(B, Hq, Hkv, D, width), dtype=torch.uint8, device=DEV)
+    ug.unigist_decode_step(p, *(x.to(DEV) for x in (q, kc, vc, table, torch.tensor(lens, dtype=torch.int32), state)), o, lse, ws)
+    torch.cuda.synchronize()
+    for b in range(B):
+        live = np.setdiff1d(np.arange(lens[b]), freed[b].numpy())
+        kl, vl = (f64(read_cache(c, table[b], lens[b])[live]) for c in (kc, vc))
+        oo, ll = oracle.decode(D ** -0.5, f64(q[b:b + 1]), [kl], [vl])
+        check_close(f"O of sequence {b}", f64(o[b:b + 1]), oo, TOL_O_MAX, TOL_O_MEAN)
+        check_close(f"LSE of sequence {b}", f64(lse[b:b + 1]), ll, TOL_LSE)
