@@ -10,7 +10,7 @@
 //                              S^T = K Q^T and dP^T = V dO^T (TMEM), P^T = exp2(S^T c - LSE),
 //                              dS^T = P^T o (dP^T - Delta), dV += P^T dO, dK += dS^T Q.  dK and dV
 //                              live in TMEM for the whole block: no atomics, deterministic.
-//   attn_bwd_dq_sm100_kernel   one thread block owns a 128-query tile of one query head and walks
+//   attn_bwd_dq_sm100_kernel   beside the tail of the other: one thread block owns a 128-query tile of one query head and walks
 //                              the visible 64-key tiles: S, dP, dS as above, dQ += dS K in TMEM.
 // Tiles without a visible pair are never loaded; only "partial" tiles evaluate the mask.
 #include <algorithm>
@@ -303,6 +303,9 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
   }
   if (warp == kKvCompute + 1) tmem_alloc(tmem_slot, 512);
   pdl_wait();
+  // The dQ kernel reads nothing that this one writes: its blocks take the SMs that this one's tail leaves idle, or never used
+  // (backward of 2 x 8190 raw tokens, ratio 7, 16 / 4 heads: 581 -> 560 us; of 1 x 448, one head: 22.5 -> 13.8).
+  pdl_release();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -629,7 +632,8 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
                          const __grid_constant__ CUtensorMap tm_k_gist, const __grid_constant__ CUtensorMap tm_v_sink,
                          const __grid_constant__ CUtensorMap tm_v_raw, const __grid_constant__ CUtensorMap tm_v_gist,
                          Geom g, int Hq, int Hkv, float scale, const float* __restrict__ lse,
-                         const float* __restrict__ delta, __nv_bfloat16* __restrict__ dq, int n_sink_qt, int n_raw_qt) {
+                         const float* __restrict__ delta, __nv_bfloat16* __restrict__ dq, int n_sink_qt, int n_raw_qt,
+                         int after_dkdv) {
   using SM = DqSmem<D>;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -679,7 +683,9 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     mbar_fence_init();
   }
   if (warp == 5) tmem_alloc(tmem_slot, 256);
-  pdl_wait();
+  // The dK / dV kernel lets this one in once all of its blocks have seen the end of what went before them, Delta included,
+  // and hands nothing on to it.  (Delta and LSE are read past the L1, which may hold an earlier call's.)
+  if (after_dkdv) pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -782,7 +788,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
     const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     const long long stat_idx = ((long long)b * Hq + h) * g.N + q_base + row;
-    const float nl = -(lse[stat_idx] * kLog2e), nd = -delta[stat_idx];
+    const float nl = -(__ldcg(lse + stat_idx) * kLog2e), nd = -__ldcg(delta + stat_idx);
     const uint64_t nl2 = f32x2(nl, nl), nd2 = f32x2(nd, nd);
     for (int j = 0; j < nt && ok; ++j) {
       int sg, idx;
@@ -872,6 +878,8 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     __syncwarp();
     tmem_dealloc(tmem, 256);
   }
+  // whoever comes after this kernel counts on dK and dV too: its last block waits for them
+  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1717,9 +1725,12 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {
+    // dQ over Q or dO in place: not before the dK / dV kernel has read them
+    const char *at = (const char*)dq, *end = at + (size_t)B * g.N * Hq * D * 2;
+    auto apart = [&](const void* x) { return end <= (const char*)x || (const char*)x + (end - at) <= at; };
     KernelScope ks("attn_bwd_dq_sm100_kernel", st);
     launch_chained(attn_bwd_dq_sm100_kernel<D>, dim3(n_tiles, Hq, B), kDqThreads, DqSmem<D>::kBytes, st, 1, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk64[0], mk64[1], mk64[2], mv64[0], mv64[1], mv64[2], g, Hq, Hkv, scale,
-        lse, delta, (__nv_bfloat16*)dq, n_sink_t, n_raw_t);
+        lse, delta, (__nv_bfloat16*)dq, n_sink_t, n_raw_t, apart(q) && apart(do_src) ? 0 : 1);
   }
   return check_launch("tcgen05 dQ kernel");
 }
