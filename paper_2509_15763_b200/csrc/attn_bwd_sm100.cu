@@ -606,7 +606,10 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
 // ------------------------------------------------------------------------------------------------
 // dQ kernel.  Two blocks per SM cover each other's softmax; with head_dim 64 a ring of four K / V stages and a second S
 // buffer leave only dP and dS on the chain of a step (the problem above: 0.38 ms -> 0.285; 0.27 with a row's operands loaded in
-// one go and packed arithmetic; eight compute warps of 32 keys were slower, 0.31).
+// one go and packed arithmetic; eight compute warps of 32 keys were slower, 0.31).  dP of the next step is issued as soon as
+// this step's operands are in registers, so that the chain of a step is the softmax alone (0.261 -> 0.240; fetching dP under
+// the exponentials instead of with the scores lost all of it again; the dK / dV kernel, whose four compute warps per
+// scheduler overlap by themselves, became 2 % slower the same way).
 constexpr int DQ_BM = 128;  // query rows per block
 constexpr int DQ_BN = 64;   // keys per step
 constexpr int kDqThreads = 192;
@@ -641,8 +644,10 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
   constexpr int kSt = SM::kStages;
   const uint32_t sQ = base, sDO = base + SM::kQTile, sK0 = base + 2 * SM::kQTile /* + stage * kKTile */, sV0 = sK0 + kSt * SM::kKTile;
   const uint32_t bars = base + SM::kOffBars;
-  const uint32_t bar_q = bars, bar_s = bars + 8, bar_p = bars + 16, bar_fin = bars + 24, tmem_slot = bars + 32;
+  const uint32_t bar_q = bars, bar_s = bars + 8, bar_fin = bars + 24, tmem_slot = bars + 32;
   const uint32_t full_k = bars + 40, full_v = full_k + 8 * kSt, empty_k = full_v + 8 * kSt, empty_v = empty_k + 8 * kSt;
+  const uint32_t bar_read = empty_v + 8 * kSt;  // S and dP of the step have been read: dP may be overwritten
+  const uint32_t bar_p = bar_read + 8;          // dS is stored (+ 8 * S buffer: step j + 1's may come before the issuer looks for step j's)
   volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen + SM::kOffBars + 32);
 
   const int warp = threadIdx.x >> 5;
@@ -679,6 +684,8 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     for (int i = 0; i < 4 * kSt; ++i) mbar_init(full_k + 8 * i, 1);
     mbar_init(bar_s, 1);
     mbar_init(bar_p, 4);
+    mbar_init(bar_p + 8, 4);
+    mbar_init(bar_read, 4);
     mbar_init(bar_fin, 1);
     mbar_fence_init();
   }
@@ -761,12 +768,15 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       for (int j = 0; j < nt && ok; ++j) {
         const int st = j % kSt;
         const bool has_next = j + 1 < nt;
-        if (SM::kSBufs == 2 && has_next) ok = issue_S(j + 1);  // runs under the softmax of step j
-        ok = ok && mbar_wait_warp(bar_p, j & 1);
+        if (SM::kSBufs == 2 && has_next) {  // the next step's scores and dP run under the softmax of step j
+          ok = issue_S(j + 1) && mbar_wait_warp(bar_read, j & 1);
+          if (!ok) break;
+          tc_fence_after();
+          ok = issue_dP(j + 1);
+        }
+        ok = ok && mbar_wait_warp(bar_p + 8 * (j % SM::kSBufs), (j / SM::kSBufs) & 1);
         if (!ok) break;
         tc_fence_after();
-        if (SM::kSBufs == 2 && has_next) ok = issue_dP(j + 1);  // what the softmax waits for goes before dQ
-        if (!ok) break;
 #pragma unroll
         for (int kk = 0; kk < DQ_BN / 16; ++kk)
           umma_ts(leader, t_dQ, t_S0 + 64 * (j % SM::kSBufs) + kk * 8,
@@ -821,6 +831,10 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
         tmem_ld32(t_dP + lane_base + 32 * c, dv_ + 32 * c);
       }
       tmem_wait_ld();
+      if (SM::kSBufs == 2) {
+        tc_fence_before();
+        mbar_arrive_warp(bar_read);
+      }
 #pragma unroll
       for (int c = 0; c < DQ_BN / 32; ++c) {
         uint32_t pk[16];
@@ -844,7 +858,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
       }
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive_warp(bar_p);
+      mbar_arrive_warp(bar_p + 8 * (j % SM::kSBufs));
     }
     if (ok) ok = mbar_wait_warp(bar_fin, 0);
     if (ok) {
