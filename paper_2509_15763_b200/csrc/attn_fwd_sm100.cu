@@ -4,7 +4,8 @@
 // A thread block runs TWO query streams at once,
 // each a 128-row query tile of one query head: either the same tile of two neighbouring heads of
 // one KV group (when the group size is even: both streams then walk the same key tiles under the
-// same mask), or two neighbouring tiles of one head.  Both streams read the same K / V tiles, which
+// same mask), or two neighbouring tiles of one head; or one stream only, where every stream can have an
+// SM to itself (fwd_mode).  Both streams read the same K / V tiles, which
 // are loaded once into a ring in shared memory.  From the closed-form row intervals each stream
 // derives, per segment, the interval of 128-key tiles that hold a visible pair; the block walks the union
 // (own segment first, downwards from the diagonal, then the other segments) and a stream skips the tiles
@@ -257,10 +258,13 @@ struct FwdRuns {
 constexpr int kMaxRunsPerLaunch = 12;  // 12 units are 20 KB of kernel parameters (the limit is 32 KB)
 static_assert(sizeof(FwdRuns<kMaxRunsPerLaunch>) + 256 <= 32764, "the launch units must fit the kernel parameter space");
 
+// The streams of a block: two tiles of one head, two heads on one tile, or one tile of one head.
+enum { kHeadPair = 0, kSingle = 1, kTilePair = 2 };  // (not kHeadPair: tiles of a unit)
+
 template <int D, int kRuns>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv rdiv, FastDiv hkdiv, float scale_log2,
-                      int pair_heads, int interleaved) {
+                      int mode, int interleaved) {
   int ri = 0, bx, by, bz;
   if constexpr (kRuns == 1) {
     bx = blockIdx.x, by = blockIdx.y, bz = blockIdx.z;
@@ -304,17 +308,17 @@ attn_fwd_sm100_kernel(const __grid_constant__ FwdRuns<kRuns> P, int Hq, FastDiv 
   const int q_seg_base = seg_base(g, qseg);  // shifted position of the segment's row 0
   int qt[2], hh[2];
   bool sv[2];
-  if (pair_heads) {
+  if (mode == kHeadPair) {
     qt[0] = qt[1] = u;
     hh[0] = 2 * by;
     hh[1] = hh[0] + 1;
     sv[0] = sv[1] = true;
   } else {
-    qt[0] = 2 * u;
-    qt[1] = 2 * u + 1;
+    qt[0] = mode * u;
+    qt[1] = qt[0] + 1;
     hh[0] = hh[1] = by;
     sv[0] = true;
-    sv[1] = qt[1] < n_qt;
+    sv[1] = mode == kTilePair && qt[1] < n_qt;
   }
 
   // Barriers, tensor memory and the Q loads come before the rest of the index arithmetic, which then runs
@@ -733,14 +737,32 @@ int32_t encode_map_2d_bf16(CUtensorMap* map, const void* base, long long rows, i
 
 namespace {
 
-// Two streams per block: neighbouring heads of a KV group when the group size is even, otherwise
-// neighbouring query tiles of one head.
-int fwd_pair_heads(const unigist_problem& p) { return (p.num_q_heads / p.num_kv_heads) % 2 == 0 ? 1 : 0; }
+// Query tiles of one sequence and head: sinks, raw, gists.
+struct QueryTiles {
+  int of[3];
+  int total() const { return of[0] + of[1] + of[2]; }
+};
+QueryTiles query_tiles(const Geom& g, const QueryRows* chunk) {
+  QueryTiles t;
+  for (int sg = 0; sg < 3; ++sg) t.of[sg] = (seg_len(g, sg) - (chunk ? chunk->off[sg] : 0) + BM - 1) / BM;
+  return t;
+}
+
+// Two streams per block: neighbouring heads of a KV group when the group size is even, otherwise neighbouring query tiles
+// of one head.  They share the SM's special-function unit, so where all `streams` of a launch can have an SM each they get
+// one: a step of one stream alone takes about two thirds of a step of two (1024 raw tokens, ratio 8, window 128, 16 / 4
+// heads of 128: 23.8 -> 20.6 us).  With more streams than SMs the time of two together counts, and those do better in
+// one block than one after the other.
+int fwd_mode(const unigist_problem& p, long long streams) {
+  if (streams <= sm_count()) return kSingle;
+  return (p.num_q_heads / p.num_kv_heads) % 2 == 0 ? kHeadPair : kTilePair;
+}
+int heads_extent(const unigist_problem& p, int mode) { return mode == kHeadPair ? p.num_q_heads / 2 : p.num_q_heads; }
 
 // Tensor maps and tile counts of one launch unit: `batch` sequences of geometry g whose first rows are
 // q, k, v, o (and lse).  With `chunk` the queries are the tail of each segment only (chunk-wise prefill).
 int32_t fill_fwd_run(FwdRun* R, const Geom& g, const unigist_problem& p, int batch, bool il, const void* q, const void* k,
-                     const void* v, void* o, float* lse, const QueryRows* chunk) {
+                     const void* v, void* o, float* lse, const QueryRows* chunk, int mode) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   if (chunk) {
     R->qr = *chunk;
@@ -756,16 +778,14 @@ int32_t fill_fwd_run(FwdRun* R, const Geom& g, const unigist_problem& p, int bat
     if (int32_t rc = encode_tile_map(&R->k[sg], k, D, Hkv, batch, g.s, g.T, g.r, g.n, il, sg)) return rc;
     if (int32_t rc = encode_tile_map(&R->v[sg], v, D, Hkv, batch, g.s, g.T, g.r, g.n, il, sg)) return rc;
   }
-  const int n_sink_qt = (sq + BM - 1) / BM, n_raw_qt = (Tq + BM - 1) / BM, n_gist_qt = (nq + BM - 1) / BM;
-  const int pair = fwd_pair_heads(p);
-  R->n_sink_units = pair ? n_sink_qt : (n_sink_qt + 1) / 2;
-  R->n_raw_units = pair ? n_raw_qt : (n_raw_qt + 1) / 2;
-  const int n_gist_units = pair ? n_gist_qt : (n_gist_qt + 1) / 2;
-  R->n_units = R->n_sink_units + R->n_raw_units + n_gist_units;
+  const QueryTiles tiles = query_tiles(g, chunk);
+  auto units = [&](int sg) { return mode == kTilePair ? (tiles.of[sg] + 1) / 2 : tiles.of[sg]; };
+  R->n_sink_units = units(kSegSink);
+  R->n_raw_units = units(kSegRaw);
+  R->n_units = R->n_sink_units + R->n_raw_units + units(kSegGist);
   R->g = g;
   R->lse = lse;
-  const int ydim = pair ? Hq / 2 : Hq;
-  R->plane = R->n_units * ydim;
+  R->plane = R->n_units * heads_extent(p, mode);
   R->units_div = make_fastdiv(R->n_units);
   R->plane_div = make_fastdiv(R->plane);
   R->cta_begin = 0;
@@ -773,15 +793,14 @@ int32_t fill_fwd_run(FwdRun* R, const Geom& g, const unigist_problem& p, int bat
 }
 
 template <typename Kern, typename Params>
-int32_t go_fwd(Kern kern, size_t smem, dim3 grid, const Params& P, const unigist_problem& p, float scale, bool il,
+int32_t go_fwd(Kern kern, size_t smem, dim3 grid, const Params& P, const unigist_problem& p, float scale, int mode, bool il,
                cudaStream_t st) {
-  const int Hq = p.num_q_heads, Hkv = p.num_kv_heads, pair = fwd_pair_heads(p);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return fail(UNIGIST_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   {
     KernelScope ks("attn_fwd_sm100_kernel", st);
-    launch_chained(kern, grid, kThreads, smem, st, 1, P, Hq, make_fastdiv(p.ratio),
-                   make_fastdiv(pair ? (Hq / Hkv) / 2 : Hq / Hkv), scale * 1.4426950408889634f, pair, il ? 1 : 0);
+    launch_chained(kern, grid, kThreads, smem, st, 1, P, p.num_q_heads, make_fastdiv(p.ratio),
+                   make_fastdiv(heads_extent(p, mode) / p.num_kv_heads), scale * 1.4426950408889634f, mode, il ? 1 : 0);
   }
   return check_launch("tcgen05 forward kernel");
 }
@@ -793,10 +812,11 @@ int32_t launch_fwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   const bool il = (p.flags & UNIGIST_FLAG_INTERLEAVED) != 0 && !chunk;
   FwdRuns<1> P;
   P.n = 1;
-  if (int32_t rc = fill_fwd_run(&P.run[0], g, p, p.batch, il, q, k, v, o, lse, chunk)) return rc;
-  const dim3 grid(P.run[0].n_units, fwd_pair_heads(p) ? p.num_q_heads / 2 : p.num_q_heads, p.batch);
-  return p.head_dim == 64 ? go_fwd(attn_fwd_sm100_kernel<64, 1>, FwdSmem<64>::kBytes, grid, P, p, scale, il, st)
-                          : go_fwd(attn_fwd_sm100_kernel<128, 1>, FwdSmem<128>::kBytes, grid, P, p, scale, il, st);
+  const int mode = fwd_mode(p, (long long)query_tiles(g, chunk).total() * p.num_q_heads * p.batch);
+  if (int32_t rc = fill_fwd_run(&P.run[0], g, p, p.batch, il, q, k, v, o, lse, chunk, mode)) return rc;
+  const dim3 grid(P.run[0].n_units, heads_extent(p, mode), p.batch);
+  return p.head_dim == 64 ? go_fwd(attn_fwd_sm100_kernel<64, 1>, FwdSmem<64>::kBytes, grid, P, p, scale, mode, il, st)
+                          : go_fwd(attn_fwd_sm100_kernel<128, 1>, FwdSmem<128>::kBytes, grid, P, p, scale, mode, il, st);
 }
 
 int32_t launch_fwd_sm100_runs(const SeqRun* runs, int n_runs, const unigist_problem& p, float scale, const void* q,
@@ -811,12 +831,15 @@ int32_t launch_fwd_sm100_runs(const SeqRun* runs, int n_runs, const unigist_prob
     std::stable_sort(order, order + P.n, [&](int a, int b) {
       return (long long)runs[first + a].g.N * runs[first + a].batch > (long long)runs[first + b].g.N * runs[first + b].batch;
     });
-    long long ctas = 0;
+    long long ctas = 0, streams = 0;
+    for (int i = 0; i < P.n; ++i)
+      streams += (long long)query_tiles(runs[first + i].g, nullptr).total() * p.num_q_heads * runs[first + i].batch;
+    const int mode = fwd_mode(p, streams);
     for (int i = 0; i < P.n; ++i) {
       const SeqRun& r = runs[first + order[i]];
       if (int32_t rc = fill_fwd_run(&P.run[i], r.g, p, r.batch, il, (const char*)q + r.first_row * rq,
                                     (const char*)k + r.first_row * rk, (const char*)v + r.first_row * rk,
-                                    (char*)o + r.first_row * rq, lse + r.first_row * p.num_q_heads, nullptr))
+                                    (char*)o + r.first_row * rq, lse + r.first_row * p.num_q_heads, nullptr, mode))
         return rc;
       P.run[i].cta_begin = (int)ctas;
       ctas += (long long)P.run[i].plane * r.batch;
@@ -824,8 +847,8 @@ int32_t launch_fwd_sm100_runs(const SeqRun* runs, int n_runs, const unigist_prob
     }
     for (int i = P.n; i < kMaxRunsPerLaunch; ++i) P.run[i] = P.run[0];  // unused slots: defined contents, never selected
     const dim3 grid((unsigned)ctas, 1, 1);
-    const int32_t rc = p.head_dim == 64 ? go_fwd(attn_fwd_sm100_kernel<64, kMaxRunsPerLaunch>, FwdSmem<64>::kBytes, grid, P, p, scale, il, st)
-                                        : go_fwd(attn_fwd_sm100_kernel<128, kMaxRunsPerLaunch>, FwdSmem<128>::kBytes, grid, P, p, scale, il, st);
+    const int32_t rc = p.head_dim == 64 ? go_fwd(attn_fwd_sm100_kernel<64, kMaxRunsPerLaunch>, FwdSmem<64>::kBytes, grid, P, p, scale, mode, il, st)
+                                        : go_fwd(attn_fwd_sm100_kernel<128, kMaxRunsPerLaunch>, FwdSmem<128>::kBytes, grid, P, p, scale, mode, il, st);
     if (rc) return rc;
   }
   return UNIGIST_OK;
