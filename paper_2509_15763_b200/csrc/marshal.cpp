@@ -29,6 +29,12 @@ struct Arg {
   operator int32_t*() const { return static_cast<int32_t*>(p); }
 };
 
+// A problem's fields by name.  The names are made once, when the module is loaded (ten strings a call took 0.75 us).
+enum { kBatch, kRawLen, kNumSinks, kRatio, kWindow, kNumQHeads, kNumKvHeads, kHeadDim, kSoftmaxScale, kFlags, kFields };
+constexpr const char* kFieldName[kFields] = {"batch",        "raw_len",  "num_sinks",     "ratio", "window", "num_q_heads",
+                                             "num_kv_heads", "head_dim", "softmax_scale", "flags"};
+PyObject* g_field[kFields];
+
 // The arguments of one call, read left to right (the caller holds a reference to each for the length of the call).
 struct Args {
   PyObject* const* a;
@@ -68,32 +74,35 @@ struct Args {
   }
   unigist_problem problem() {
     PyObject* o = next();
-    auto field = [&](const char* name) {
-      PyObject* v = PyObject_GetAttrString(o, name);
+    auto field = [&](int name) {
+      PyObject* v = PyObject_GetAttr(o, g_field[name]);
       if (!v) throw python_error();
-      PyObject* i = PyNumber_Index(v);  // whatever counts as an integer (numpy's too), as ctypes takes it; no float
+      if (!PyLong_CheckExact(v)) {
+        PyObject* i = PyNumber_Index(v);  // whatever counts as an integer (numpy's too), as ctypes takes it; no float
+        Py_DECREF(v);
+        if (!i) throw python_error();
+        v = i;
+      }
+      const unsigned long long x = PyLong_AsUnsignedLongLongMask(v);
       Py_DECREF(v);
-      if (!i) throw python_error();
-      const unsigned long long x = PyLong_AsUnsignedLongLongMask(i);
-      Py_DECREF(i);
       if (PyErr_Occurred()) throw python_error();
       return x;
     };
     unigist_problem p;
-    p.batch = (int32_t)field("batch");
-    p.raw_len = (int32_t)field("raw_len");
-    p.num_sinks = (int32_t)field("num_sinks");
-    p.ratio = (int32_t)field("ratio");
-    p.window = (int32_t)field("window");
-    p.num_q_heads = (int32_t)field("num_q_heads");
-    p.num_kv_heads = (int32_t)field("num_kv_heads");
-    p.head_dim = (int32_t)field("head_dim");
-    PyObject* s = PyObject_GetAttrString(o, "softmax_scale");
+    p.batch = (int32_t)field(kBatch);
+    p.raw_len = (int32_t)field(kRawLen);
+    p.num_sinks = (int32_t)field(kNumSinks);
+    p.ratio = (int32_t)field(kRatio);
+    p.window = (int32_t)field(kWindow);
+    p.num_q_heads = (int32_t)field(kNumQHeads);
+    p.num_kv_heads = (int32_t)field(kNumKvHeads);
+    p.head_dim = (int32_t)field(kHeadDim);
+    PyObject* s = PyObject_GetAttr(o, g_field[kSoftmaxScale]);
     if (!s) throw python_error();
     p.softmax_scale = (float)PyFloat_AsDouble(s);
     Py_DECREF(s);
     if (PyErr_Occurred()) throw python_error();
-    p.flags = (uint32_t)field("flags");
+    p.flags = (uint32_t)field(kFlags);
     return p;
   }
   std::vector<int32_t> int_list() {
@@ -284,4 +293,8 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, kMethods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit__marshal() {
+  for (int i = 0; i < kFields; ++i)
+    if (!g_field[i] && !(g_field[i] = PyUnicode_InternFromString(kFieldName[i]))) return nullptr;
+  return PyModule_Create(&kModule);
+}
