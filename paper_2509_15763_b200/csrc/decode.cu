@@ -6,7 +6,7 @@
 // K and V are read exactly once (64 sequences of 9216 tokens, 2.4 GB: 6.9 TB/s, the copy rate of the chip being 6.5;
 // one of 1337 tokens: 5.7 us in a graph, 8.5 with two kernels).
 //   producer warp:  per page one K and one V tile (64 tokens x 128 dims, 16 KB each) by TMA, 128-byte
-//                   swizzle, into a 3-stage ring guarded by full / empty mbarriers; two thread blocks
+//                   swizzle, into a 3-stage ring guarded by mbarriers (full / free); two thread blocks
 //                   per SM keep about 128 KB of loads in flight.
 //   consumer warps: three warps, one per ring stage, each takes every third page on its own and keeps a running
 //                   (max, sum, output) for the G query heads of the KV head: S = Q K^T and O += P V
@@ -71,7 +71,7 @@ __device__ __forceinline__ float to_finite(float x) {
 constexpr int kRow = DD + 4;  // a head's result: 128 sums, maximum, sum of the weights (rows of whole 16-byte pieces)
 struct DecSmem {
   static constexpr int kOffBars = STAGES * STAGE_BYTES;
-  static constexpr int kOffMerge = kOffBars + 64;                              // [warps][8 heads][kRow] fp32
+  static constexpr int kOffMerge = kOffBars + 128;                             // [warps][8 heads][kRow] fp32
   static constexpr int kOffFirst = kOffMerge + kConsumers * 8 * kRow * 4;  // [THREADS + 1] 64-bit
   static constexpr int kBytes = kOffFirst + (THREADS + 1) * 8 + 1024 /*align*/;
 };
@@ -215,17 +215,20 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
-  const uint32_t bars = base + DecSmem::kOffBars;  // full[s] at + 8 s, empty[s] at + 8 (STAGES + s)
+  // Barriers, + 8 * stage.  Split by rank, walks are short and bound by latency: a warp has one stage, and the K of its next
+  // page comes under this one's softmax and P V, since K has barriers of its own (8 sequences of 2112 tokens: 11.3 -> 10.7
+  // us).  The flat walk is bound by the memory system, which takes K and V apart badly (64 sequences of 9216: 345 -> 357 us):
+  // there both arrive (full_k) and are free again (free_v) together.
+  constexpr bool kApart = !kFlat;
+  const uint32_t full_k = base + DecSmem::kOffBars, full_v = full_k + 8 * STAGES, free_k = full_v + 8 * STAGES,
+                 free_v = free_k + 8 * STAGES;
   float* merge = reinterpret_cast<float*>(gen + DecSmem::kOffMerge);
   long long* first = reinterpret_cast<long long*>(gen + DecSmem::kOffFirst);
   const int hk = blockIdx.y, G = P.G;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) {
-      mbar_init(bars + 8 * i, 1);
-      mbar_init(bars + 8 * (STAGES + i), 1);
-    }
+    for (int i = 0; i < 4 * STAGES; ++i) mbar_init(full_k + 8 * i, 1);
     mbar_fence_init();
   }
   pdl_wait();  // nothing above touches global memory
@@ -261,30 +264,42 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   if (warp == kConsumers) {
     // ------------------------------------------------------------ producer
     Walk<kFlat> w = start;
-    int i = 0;  // pages loaded so far
+    int i0 = 0;  // ring position of the run's first page
     while (ok && w.next(P)) {
       const int32_t* row = P.table + (long long)w.seq * P.max_blocks;
       int32_t phys_mine = 0;
-      for (int j = 0; j < w.count; ++j, ++i) {
-        if ((j & 31) == 0) {  // the next 32 block-table entries, one per lane
-          phys_mine = j + lane < w.count ? row[w.first + j + lane] : 0;
-          phys_mine = min(max(phys_mine, 0), P.num_blocks - 1);  // never read outside the cache
+      constexpr int kRound = kFlat ? 1 : STAGES;  // the K of a round of pages, then their V
+      for (int j0 = 0; j0 < w.count && ok; j0 += kRound) {
+        int row0[kRound];
+#pragma unroll
+        for (int u = 0; u < kRound; ++u) {
+          const int j = j0 + u;
+          if (j >= w.count) break;
+          if ((j & 31) == 0) {  // the next 32 block-table entries, one per lane
+            phys_mine = j + lane < w.count ? row[w.first + j + lane] : 0;
+            phys_mine = min(max(phys_mine, 0), P.num_blocks - 1);  // never read outside the cache
+          }
+          row0[u] = (__shfl_sync(0xffffffffu, phys_mine, j & 31) * P.Hkv + hk) * PG;
         }
-        const int phys = __shfl_sync(0xffffffffu, phys_mine, j & 31);
-        const int st = i % STAGES, use = i / STAGES;
-        if (use > 0) ok = mbar_wait_warp(bars + 8 * (STAGES + st), (use - 1) & 1);
-        if (!ok) break;
-        if (lane == 0) {
-          const uint32_t full = bars + 8 * st, dst = base + st * STAGE_BYTES;
-          const int row0 = (phys * P.Hkv + hk) * PG;
-          mbar_arrive_expect_tx(full, STAGE_BYTES);
-          tma_load_2d(dst, &tm_k, full, 0, row0);
-          tma_load_2d(dst + SLAB_BYTES, &tm_k, full, 64, row0);
-          tma_load_2d(dst + PAGE_BYTES, &tm_v, full, 0, row0);
-          tma_load_2d(dst + PAGE_BYTES + SLAB_BYTES, &tm_v, full, 64, row0);
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+#pragma unroll
+          for (int u = 0; u < kRound; ++u) {
+            const int i = i0 + j0 + u, st = i % STAGES, use = i / STAGES;
+            if (j0 + u >= w.count || !ok) break;
+            if (use > 0 && (kApart || v == 0)) ok = mbar_wait_warp((kApart && v == 0 ? free_k : free_v) + 8 * st, (use - 1) & 1);
+            if (!ok) break;
+            if (lane == 0) {
+              const uint32_t full = (kApart && v ? full_v : full_k) + 8 * st, dst = base + st * STAGE_BYTES + v * PAGE_BYTES;
+              if (kApart || v == 0) mbar_arrive_expect_tx(full, kApart ? PAGE_BYTES : STAGE_BYTES);
+              tma_load_2d(dst, v ? &tm_v : &tm_k, full, 0, row0[u]);
+              tma_load_2d(dst + SLAB_BYTES, v ? &tm_v : &tm_k, full, 64, row0[u]);
+            }
+            __syncwarp();
+          }
         }
-        __syncwarp();
       }
+      i0 += w.count;
     }
     if (!ok && lane == 0) atomicExch(&g_decode_timeout, 1u);
   } else {
@@ -319,7 +334,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
       if (j < 0) j += STAGES;
       for (; j < w.count && ok; j += kConsumers) {
         const int i = i0 + j, st = i % STAGES, use = i / STAGES;
-        ok = mbar_wait_warp(bars + 8 * st, use & 1);
+        ok = mbar_wait_warp(full_k + 8 * st, use & 1);
         if (!ok) break;
         const uint32_t sK = base + st * STAGE_BYTES, sV = sK + PAGE_BYTES;
         const int tok0 = (w.first + j) * PG;
@@ -346,6 +361,10 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
             mma_bf16(s[nt], qa0[2 * kq], 0u, qa2[2 * kq], 0u, k0, k1);
             mma_bf16(s[nt], qa0[2 * kq + 1], 0u, qa2[2 * kq + 1], 0u, k2, k3);
           }
+        }
+        if (kApart) {  // the next K may come
+          __syncwarp();
+          if (lane == 0) mbar_arrive(free_k + 8 * st);
         }
         // running softmax of row g over the page's 64 tokens (this lane: tokens 8 nt + 2 qc + {0, 1})
         float mx = -INFINITY;
@@ -379,6 +398,8 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
         ps += __shfl_xor_sync(0xffffffffu, ps, 1);
         ps += __shfl_xor_sync(0xffffffffu, ps, 2);
         l_run = l_run * f + ps;
+        if (kApart) ok = mbar_wait_warp(full_v + 8 * st, use & 1);
+        if (!ok) break;
         // O = O f + P V, 4 k-steps of 16 tokens per pair of 8-dim tiles
 #pragma unroll
         for (int np = 0; np < 8; ++np) {  // dim tiles 2 np, 2 np + 1
@@ -398,7 +419,7 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
           o[2 * np + 1][1] = fmaf(o[2 * np + 1][1], f, c1[1] + to_finite(c1[3]));
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bars + 8 * (STAGES + st));  // the stage may be refilled
+        if (lane == 0) mbar_arrive(free_v + 8 * st);
       }
       i0 += w.count;
       // the warps' results for this run meet in shared memory
