@@ -115,7 +115,7 @@ bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int H
 
 // Query rows (numbered inside the raw or the gist segment, inclusive) that see a given key:
 // Eq. 3 read column-wise.  An empty interval has lo > hi.
-__device__ __forceinline__ void key_q_interval(const Geom& g, bool key_is_raw, int key, bool key_valid,
+__device__ __forceinline__ void key_q_interval(const Geom& g, const FastDiv& rdiv, bool key_is_raw, int key, bool key_valid,
                                                bool q_is_raw, int& lo, int& hi) {
   if (!key_valid) {
     lo = 1;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void key_q_interval(const Geom& g, bool key_is_raw, i
     return;
   }
   if (key_is_raw) {
-    const int u = key / g.r;
+    const int u = fdiv(rdiv, key);
     if (q_is_raw) {
       lo = key;
       hi = min(g.T - 1, (u + g.k + 1) * g.r - 1);
@@ -144,7 +144,7 @@ __device__ __forceinline__ void key_q_interval(const Geom& g, bool key_is_raw, i
 
 // Query rows of segment qseg (numbered inside it, inclusive) that see key `key` of segment kseg:
 // Eq. 3 read column-wise, sinks included.  An empty interval has lo > hi.
-__device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key, bool key_valid, int qseg, int& lo,
+__device__ __forceinline__ void key_q_interval3(const Geom& g, const FastDiv& rdiv, int kseg, int key, bool key_valid, int qseg, int& lo,
                                                 int& hi) {
   lo = 1;
   hi = 0;
@@ -155,7 +155,7 @@ __device__ __forceinline__ void key_q_interval3(const Geom& g, int kseg, int key
     return;
   }
   if (qseg == kSegSink) return;  // sink queries see sinks only
-  key_q_interval(g, kseg == kSegRaw, key, true, qseg == kSegRaw, lo, hi);
+  key_q_interval(g, rdiv, kseg == kSegRaw, key, true, qseg == kSegRaw, lo, hi);
 }
 
 // One 32-query chunk of P^T for one key: p = 2^(s * c + nl[q]), nl = -LSE in log2 units; kMasked: bit e of `bits` says
@@ -226,7 +226,7 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
                            Geom g, int Hq, int Hkv, float scale, const float* __restrict__ lse,
                            const float* __restrict__ delta, __nv_bfloat16* __restrict__ dk,
                            __nv_bfloat16* __restrict__ dv, int n_sink_kt, int n_gist_kt, int n_raw_kt, int pairs, int shared,
-                           FastDiv heavy_div, FastDiv raw_div, FastDiv hkv_div) {
+                           FastDiv heavy_div, FastDiv raw_div, FastDiv hkv_div, FastDiv rdiv) {
   using SM = KvSmem<D>;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -272,14 +272,14 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
   // query tiles that see this key tile, per query segment: first tile and count, and the bounds inside which a
   // tile is "full" (seen by the last key from t_lo on, by the first key up to t_hi)
   int lo_a, hi_a, lo_b, hi_b;
-  key_q_interval3(g, kseg, key_a, true, kSegRaw, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegRaw, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegRaw, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegRaw, lo_b, hi_b);
   const int n_raw_q = hi_b >= lo_a ? hi_b / KV_BN - lo_a / KV_BN + 1 : 0, rq_lo = lo_a / KV_BN, raw_t_lo = lo_b, raw_t_hi = hi_a;
-  key_q_interval3(g, kseg, key_a, true, kSegGist, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegGist, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegGist, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegGist, lo_b, hi_b);
   const int n_gist_q = hi_b >= lo_a ? hi_b / KV_BN - lo_a / KV_BN + 1 : 0, gq_lo = lo_a / KV_BN, gist_t_lo = lo_b, gist_t_hi = hi_a;
-  key_q_interval3(g, kseg, key_a, true, kSegSink, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegSink, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegSink, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegSink, lo_b, hi_b);
   const int n_sink_q = hi_b >= lo_a ? hi_b / KV_BN - lo_a / KV_BN + 1 : 0, sq_lo = lo_a / KV_BN, sink_t_lo = lo_b, sink_t_hi = hi_a;
   // this block's part of the walk: query tiles [t_begin, t_end) in the order of the steps below
   const int n_tiles = n_raw_q + n_gist_q + n_sink_q, t_half = (n_tiles + 1) / 2;
@@ -463,9 +463,9 @@ attn_bwd_dkdv_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const 
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
     const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     int my_lo_r, my_hi_r, my_lo_g, my_hi_g, my_lo_s, my_hi_s;  // queries that see this key, per query segment
-    key_q_interval3(g, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
-    key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
-    key_q_interval3(g, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
 
     StepIter cur{t_begin, 0};
     for (int it = 0; it < n_iter && ok; ++it, advance(cur)) {
@@ -636,7 +636,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
                          const __grid_constant__ CUtensorMap tm_v_raw, const __grid_constant__ CUtensorMap tm_v_gist,
                          Geom g, int Hq, int Hkv, float scale, const float* __restrict__ lse,
                          const float* __restrict__ delta, __nv_bfloat16* __restrict__ dq, int n_sink_qt, int n_raw_qt,
-                         int after_dkdv) {
+                         int after_dkdv, FastDiv rdiv) {
   using SM = DqSmem<D>;
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -659,7 +659,8 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
   const int q_len = seg_len(g, qseg);
   const int q_base = seg_base(g, qseg);
   const int row_a = qt * DQ_BM, row_b = min(row_a + DQ_BM - 1, q_len - 1);
-  const RowIv iv_a = row_intervals(g, q_base + row_a), iv_b = row_intervals(g, q_base + row_b);
+  auto div_r = [&](int x) { return fdiv(rdiv, x); };
+  const RowIv iv_a = row_intervals_with(g, q_base + row_a, div_r), iv_b = row_intervals_with(g, q_base + row_b, div_r);
   // visible 64-key tiles: sink tiles [0, n_sink), raw tiles [raw_lo, raw_lo + n_raw), gist tiles [0, n_gist)
   const int n_sink = iv_b.hi_sink >= 0 ? iv_b.hi_sink / DQ_BN + 1 : 0;
   const int raw_lo = iv_a.lo_raw / DQ_BN, n_raw = iv_b.hi_raw >= iv_a.lo_raw ? iv_b.hi_raw / DQ_BN - raw_lo + 1 : 0;
@@ -794,7 +795,7 @@ attn_bwd_dq_sm100_kernel(const __grid_constant__ CUtensorMap tm_q_sink, const __
     const int r_in_tile = threadIdx.x;
     const int row = min(row_a + r_in_tile, row_b);
     const bool valid = row_a + r_in_tile <= row_b;
-    const RowIv my = row_intervals(g, q_base + row);
+    const RowIv my = row_intervals_with(g, q_base + row, div_r);
     const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
     const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     const long long stat_idx = ((long long)b * Hq + h) * g.N + q_base + row;
@@ -1048,14 +1049,14 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
   // query tiles that see this key tile, per query segment: [first tile, count], and the bounds inside
   // which a tile is "full" (seen by the last key from t_lo on, by the first key up to t_hi)
   int lo_a, hi_a, lo_b, hi_b;
-  key_q_interval3(g, kseg, key_a, true, kSegRaw, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegRaw, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegRaw, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegRaw, lo_b, hi_b);
   const int n_raw_q = hi_b >= lo_a ? hi_b / 128 - lo_a / 128 + 1 : 0, rq_lo = lo_a / 128, raw_t_lo = lo_b, raw_t_hi = hi_a;
-  key_q_interval3(g, kseg, key_a, true, kSegGist, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegGist, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegGist, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegGist, lo_b, hi_b);
   const int n_gist_q = hi_b >= lo_a ? hi_b / 128 - lo_a / 128 + 1 : 0, gq_lo = lo_a / 128, gist_t_lo = lo_b, gist_t_hi = hi_a;
-  key_q_interval3(g, kseg, key_a, true, kSegSink, lo_a, hi_a);
-  key_q_interval3(g, kseg, key_b, true, kSegSink, lo_b, hi_b);
+  key_q_interval3(g, rdiv, kseg, key_a, true, kSegSink, lo_a, hi_a);
+  key_q_interval3(g, rdiv, kseg, key_b, true, kSegSink, lo_b, hi_b);
   const int n_sink_q = hi_b >= lo_a ? hi_b / 128 - lo_a / 128 + 1 : 0, sq_lo = lo_a / 128, sink_t_lo = lo_b, sink_t_hi = hi_a;
   // this block's part of the walk: tiles [t_begin, t_end) of the order below (all of them for a raw key tile)
   const int n_tiles = n_raw_q + n_gist_q + n_sink_q;
@@ -1349,9 +1350,9 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
     const uint64_t scale2 = f32x2(scale * kLog2e, scale * kLog2e);
     int my_lo_r, my_hi_r, my_lo_g, my_hi_g, my_lo_s, my_hi_s;  // queries that see this key, per query segment
-    key_q_interval3(g, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
-    key_q_interval3(g, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
-    key_q_interval3(g, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegRaw, my_lo_r, my_hi_r);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegGist, my_lo_g, my_hi_g);
+    key_q_interval3(g, rdiv, kseg, key, key_valid, kSegSink, my_lo_s, my_hi_s);
     // this thread's row of the dS^T tile in shared memory: slab hf, row krow, 16-byte chunks swizzled by row
     unsigned char* ds_row = gen + SM::kOffDS + hf * SM::kSlab + krow * 128;
     const int swz = krow & 7;
@@ -1475,13 +1476,13 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
 }
 
 // Number of 128-query tiles that see a key tile [key_a, key_b] of segment kseg (all query segments).
-__device__ __forceinline__ int count_q_tiles(const Geom& g, int kseg, int key_a, int key_b) {
+__device__ __forceinline__ int count_q_tiles(const Geom& g, const FastDiv& rdiv, int kseg, int key_a, int key_b) {
   int n = 0;
 #pragma unroll
   for (int qseg = 0; qseg < 3; ++qseg) {
     int lo_a, hi_a, lo_b, hi_b;
-    key_q_interval3(g, kseg, key_a, true, qseg, lo_a, hi_a);
-    key_q_interval3(g, kseg, key_b, true, qseg, lo_b, hi_b);
+    key_q_interval3(g, rdiv, kseg, key_a, true, qseg, lo_a, hi_a);
+    key_q_interval3(g, rdiv, kseg, key_b, true, qseg, lo_b, hi_b);
     n += hi_b >= lo_a ? hi_b / 128 - lo_a / 128 + 1 : 0;
   }
   return n;
@@ -1493,14 +1494,14 @@ __device__ __forceinline__ int count_q_tiles(const Geom& g, int kseg, int key_a,
 __global__ void __launch_bounds__(128)
 dkdv_reduce_kernel(Geom g, int interleaved, int Hkv, int n_sink_kt, int n_gist_kt, int n_chunks, int chunk_tiles,
                    const float* __restrict__ partial, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                   float scale) {
+                   float scale, FastDiv rdiv) {
   pdl_wait();
   const int rank = blockIdx.x >> 3, row0 = (blockIdx.x & 7) * 16, hk = blockIdx.y, b = blockIdx.z;
   const int n_heavy_kt = n_sink_kt + n_gist_kt;
   const int kseg = rank < n_sink_kt ? kSegSink : kSegGist;
   const int kt = rank - (kseg == kSegSink ? 0 : n_sink_kt);
   const int key_a = kt * 128, key_b = min(key_a + 127, seg_len(g, kseg) - 1);
-  const int n_tiles = count_q_tiles(g, kseg, key_a, key_b);
+  const int n_tiles = count_q_tiles(g, rdiv, kseg, key_a, key_b);
   if (n_tiles <= chunk_tiles) return;  // a single chunk: the fused kernel stored dK, dV itself
   const int chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1682,7 +1683,7 @@ int32_t launch_dkdv_reduce(const BwdRun& R, int batch, const unigist_problem& p,
   {
     KernelScope ks("dkdv_reduce_kernel", st);
     launch_chained(dkdv_reduce_kernel, dim3((R.n_sink_kt + R.n_gist_kt) * 8, p.num_kv_heads, batch), 128, 0, st, 1, R.g, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_kv_heads, R.n_sink_kt, R.n_gist_kt, R.n_chunks,
-        R.chunk_tiles, R.partial, R.dk, R.dv, scale);
+        R.chunk_tiles, R.partial, R.dk, R.dv, scale, make_fastdiv(p.ratio));
   }
   return check_launch("dK/dV reduce kernel");
 }
@@ -1735,7 +1736,7 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
     launch_chained(attn_bwd_dkdv_sm100_kernel<D>, dim3(((n_heavy + raw_units) * pairs) << shared), kKvThreads, KvSmem<D>::kBytes,
                    st, 1 << shared, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk[0], mk[1], mk[2], mv[0], mv[1], mv[2], g, Hq, Hkv, scale,
                    lse, delta, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, n_sink_t, n_gist_t, n_raw_t, pairs, shared,
-                   make_fastdiv(n_heavy), make_fastdiv(raw_units), make_fastdiv(Hkv));
+                   make_fastdiv(n_heavy), make_fastdiv(raw_units), make_fastdiv(Hkv), make_fastdiv(g.r));
   }
   if (int32_t rc = check_launch("tcgen05 dK/dV kernel")) return rc;
   {
@@ -1744,7 +1745,7 @@ int32_t launch_two_kernels(const Geom& g, const unigist_problem& p, float scale,
     auto apart = [&](const void* x) { return end <= (const char*)x || (const char*)x + (end - at) <= at; };
     KernelScope ks("attn_bwd_dq_sm100_kernel", st);
     launch_chained(attn_bwd_dq_sm100_kernel<D>, dim3(n_tiles, Hq, B), kDqThreads, DqSmem<D>::kBytes, st, 1, mq[0], mq[1], mq[2], md[0], md[1], md[2], mk64[0], mk64[1], mk64[2], mv64[0], mv64[1], mv64[2], g, Hq, Hkv, scale,
-        lse, delta, (__nv_bfloat16*)dq, n_sink_t, n_raw_t, apart(q) && apart(do_src) ? 0 : 1);
+        lse, delta, (__nv_bfloat16*)dq, n_sink_t, n_raw_t, apart(q) && apart(do_src) ? 0 : 1, make_fastdiv(g.r));
   }
   return check_launch("tcgen05 dQ kernel");
 }
