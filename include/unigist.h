@@ -174,7 +174,8 @@ int32_t unigist_attn_fwd(const unigist_problem* p, const void* q, const void* k,
  * whatever order the blocks arrive: its last bit may differ between runs (UNIGIST_FLAG_DETERMINISTIC_DQ trades
  * speed for a fixed order).  workspace:
  * unigist_workspace_bytes(p, UNIGIST_OP_BWD) bytes (Delta, a bf16 copy of an fp32 dO, and for head_dim 128 the
- * fp32 dQ accumulator and the chunks' partial dK / dV), 16-byte aligned.
+ * fp32 dQ accumulator and the chunks' partial dK / dV), 16-byte aligned.  Less is accepted, down to a size without those
+ * partial sums that only spread a walk over idle SMs: the call is then slower, dK / dV may differ in their last bits.
  */
 int32_t unigist_attn_bwd(const unigist_problem* p, const void* q, const void* k, const void* v,
                          const void* o, const float* lse, const void* d_o, void* dq, void* dk,

@@ -198,7 +198,7 @@ size_t unigist_workspace_bytes(const unigist_problem* p, int32_t op) {
       // the fp32 dQ accumulator and the chunks' partial dK / dV
       return bwd_scratch_bytes((long long)p->batch * g.N, p->num_q_heads, p->head_dim,
                                (p->flags & UNIGIST_FLAG_DOUT_FP32) != 0, bwd_is_fused(p->head_dim, p->flags)) +
-             bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, bwd_is_fused(p->head_dim, p->flags));
+             bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, bwd_is_fused(p->head_dim, p->flags), true);
     case UNIGIST_OP_COMPACT: {
       const size_t L = (size_t)g.s + g.n + (size_t)g.k * g.r;
       return align_up(2 * (size_t)p->batch * L * p->num_kv_heads * p->head_dim * 2, 256);
@@ -313,12 +313,16 @@ int32_t unigist_attn_bwd(const unigist_problem* p, const void* q, const void* k,
     if (!aligned16(x)) return fail(UNIGIST_ERR_ALIGNMENT, "tensor pointers must be 16-byte aligned");
   if (reinterpret_cast<uintptr_t>(lse) & 3) return fail(UNIGIST_ERR_ALIGNMENT, "lse must be 4-byte aligned");
   if (int32_t rc = check_interleaved(p, g)) return rc;
-  const size_t need = unigist_workspace_bytes(p, UNIGIST_OP_BWD);
+  // a small problem's walks are spread over more blocks where there is room for their partial sums, which is not asked for
+  const size_t full = unigist_workspace_bytes(p, UNIGIST_OP_BWD);
+  const bool fused = bwd_is_fused(p->head_dim, p->flags);
+  const size_t need = full - bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, fused, true) +
+                      bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, fused, false);
   if (!workspace || ws_bytes < need)
     return fail(UNIGIST_ERR_WORKSPACE, "backward needs %zu bytes of workspace, got %zu", need,
                 ws_bytes);
   // the fused kernel for head_dim 128, the two-kernel path for head_dim 64; both on the tensor cores
-  return launch_bwd_sm100(g, *p, scale, q, k, v, o, lse, d_o, dq, dk, dv, workspace, (cudaStream_t)stream);
+  return launch_bwd_sm100(g, *p, scale, q, k, v, o, lse, d_o, dq, dk, dv, workspace, ws_bytes >= full, (cudaStream_t)stream);
 }
 
 // ---- cross-document masking: a packed sample is a list of independent sequences -------------------------------
@@ -395,7 +399,7 @@ size_t unigist_docs_workspace_bytes(const unigist_problem* p, int32_t op, int32_
     for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t, int32_t) {
       Geom g;
       if (check_problem(&run, &g, nullptr) == UNIGIST_OK)
-        need += bwd_partial_bytes(g, run.batch, run.num_q_heads, run.num_kv_heads, true);
+        need += bwd_partial_bytes(g, run.batch, run.num_q_heads, run.num_kv_heads, true, false);
       return (int32_t)UNIGIST_OK;
     });
     return need;
