@@ -1607,20 +1607,25 @@ int32_t launch_convert(const TokRuns<kRuns>& T, const unigist_problem& p, long l
   return check_launch("dQ convert kernel");
 }
 
+int tiles(long long rows) { return (int)((rows + 127) / 128); }
+// Query tiles that a raw key tile's walk has at most: k + 1 units and their gists.
+long long raw_walk(const Geom& g) {
+  return std::min(tiles((g.k + 1ll) * g.r) + 1, tiles(g.T)) + std::min(tiles(g.k + 1ll) + 1, tiles(g.n));
+}
+
 // How the walk of a sink or gist key tile over its query tiles is cut (head_dim 128).  Not at all while the rows
 // one KV head's blocks sweep (Q, dO and the fp32 dQ of its G query heads: 1 KB per token and head) fit in three
 // quarters of the L2: however the blocks start, what one has read is still there for the next.  Otherwise into at
 // most four chunks of at least 16 query tiles, fewer where the chunks' fp32 partial sums would take more than
 // half the room of the dQ accumulator.
 // Where the longest sink or gist walk, and not the load of an SM, is the kernel's time (a step is about 2 us), that walk is
-// cut too, if the workspace has room (spread): into chunks of half of an SM's load, no shorter than a raw key tile's walk,
+// cut too, if the workspace has room (load >= 0, the steps of the launch per SM): into chunks of half of an SM's load, no shorter than a raw key tile's walk,
 // where that saves at least eight steps; the second kernel and the partial sums cost about 5 us (us of the whole backward,
 // uncut and cut: 512 raw tokens, ratio 4, 32 / 8 heads 63 and 54; 1024, 16 / 4 heads 92 and 51; 4096, ratio 16, window 128, 16
 // / 2 heads 598 and 130; 4096, window 1024, 32 / 8 heads 382 and 320; 9000, window 128 811 and 520; 16384, window 1024, longest
 // walk 576 steps, load 571: not cut).
 // -> tiles per chunk, number of chunks of the longest walk (1 = no cutting, no partial sums).
-void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, bool spread, int* n_chunks, int* chunk_tiles) {
-  auto tiles = [](long long rows) { return (int)((rows + 127) / 128); };
+void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, long long load, int* n_chunks, int* chunk_tiles) {
   const int n_raw = tiles(g.T), n_gist = tiles(g.n), n_heavy = tiles(g.s) + n_gist;
   const int max_tiles = n_heavy + n_raw;  // the first sink / gist key tile is seen by every query tile
   const size_t dq_bytes = (size_t)batch * g.N * Hq * 128 * sizeof(float);
@@ -1629,13 +1634,8 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, bool spread, int* n
   while (C > 1 && ((max_tiles + C - 1) / C < 16 ||
                    (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2))
     --C;
-  if (spread && C == 1 && n_heavy > 0) {
-    // steps: a gist key is seen by the later half of all rows on average, a raw key by k + 1 units and their gists
-    const long long G = Hq / Hkv, longest = max_tiles * G;
-    const long long window = std::min(tiles((g.k + 1ll) * g.r) + 1, n_raw) + std::min(tiles(g.k + 1ll) + 1, n_gist);
-    const long long load = ((long long)(n_heavy - n_gist) * max_tiles + (long long)n_gist * (n_raw + n_gist + 1) / 2 +
-                            n_raw * window) * Hq * batch / sm_count();
-    const long long target = std::max(window * G, load / 2);
+  if (load >= 0 && C == 1 && n_heavy > 0) {
+    const long long G = Hq / Hkv, longest = max_tiles * G, target = std::max(raw_walk(g) * G, load / 2);
     if (longest - std::max(target, load) >= 8) C = (int)((longest + target - 1) / target);
     while (C > 1 && (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2) --C;
   }
@@ -1648,7 +1648,7 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, bool spread, int* n
 // interleaved tensors, and reduction maps over the fp32 dQ tensor (always shifted).
 int32_t fill_bwd_run(BwdRun* R, const Geom& g, const unigist_problem& p, int batch, const void* q, const void* do_src,
                      const void* k, const void* v, float* dq32, const float* lse, const float* delta, void* dk, void* dv,
-                     float* partial, bool spread) {
+                     float* partial, long long load) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   const bool il = (p.flags & UNIGIST_FLAG_INTERLEAVED) != 0;
   for (int sg = 0; sg < 3; ++sg) {
@@ -1667,7 +1667,7 @@ int32_t fill_bwd_run(BwdRun* R, const Geom& g, const unigist_problem& p, int bat
   R->n_sink_kt = (g.s + 127) / 128;
   R->n_gist_kt = (g.n + 127) / 128;
   R->n_raw_kt = (g.T + 127) / 128;
-  bwd_chunking(g, batch, Hq, Hkv, spread, &R->n_chunks, &R->chunk_tiles);
+  bwd_chunking(g, batch, Hq, Hkv, load, &R->n_chunks, &R->chunk_tiles);
   R->partial = partial;
   const int n_heavy = R->n_sink_kt + R->n_gist_kt;
   R->heavy_plane = n_heavy * R->n_chunks * Hkv;
@@ -1712,11 +1712,8 @@ int32_t launch_dkdv_reduce(const BwdRun& R, int batch, const unigist_problem& p,
 // and 577; 2 x 12288, ratio 3, 384 / 396: 1058 and 1150; 4 x 8190, 296 / 411: 1043 and 1005; 8 x 2048, 80 / 105: 301 and 283; 256
 // x 128, 8 / 83: 618 and 422; 1 x 448, one head, 5 / 0: 23.8 and 21.9).
 bool dkdv_shares(const Geom& g, int batch, int Hq, int Hkv) {
-  auto tiles = [](long long rows) { return (rows + 127) / 128; };
-  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n), all = sink + raw + gist, G = Hq / Hkv;
-  // a gist key is seen by the later half of all rows on average, a raw key by k + 1 units and their gists
-  const long long window = std::min(tiles((g.k + 1ll) * g.r) + 1, raw) + std::min(tiles(g.k + 1ll) + 1, gist);
-  const long long steps = (sink * all + gist * (raw + gist + 1) / 2 + raw * window) * Hq * batch / sm_count();
+  const long long all = tiles(g.s) + tiles(g.T) + tiles(g.n), G = Hq / Hkv;
+  const long long steps = bwd_steps(g, batch, Hq) / sm_count();
   return all * G > steps * 3 / 4 + 22;
 }
 
@@ -1776,10 +1773,16 @@ size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool f
   return b;
 }
 
-size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, bool spread) {
+// A gist key is seen by the later half of all rows on average.
+long long bwd_steps(const Geom& g, int batch, int Hq) {
+  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
+  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk(g)) * Hq * batch;
+}
+
+size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, long long load) {
   if (!fused) return 0;
   int C, tiles;
-  bwd_chunking(g, batch, Hq, Hkv, spread, &C, &tiles);
+  bwd_chunking(g, batch, Hq, Hkv, load, &C, &tiles);
   if (C <= 1) return 0;
   const size_t n_heavy = (g.s + 127) / 128 + (g.n + 127) / 128;
   return align256((size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float));
@@ -1787,7 +1790,7 @@ size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, 
 
 int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, const void* q, const void* k,
                          const void* v, const void* o, const float* lse, const void* d_o, void* dq, void* dk,
-                         void* dv, void* workspace, bool spread, cudaStream_t st) {
+                         void* dv, void* workspace, long long load, cudaStream_t st) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads, B = p.batch;
   const bool f32 = (p.flags & UNIGIST_FLAG_DOUT_FP32) != 0;
   const long long tokens = (long long)B * g.N;
@@ -1809,7 +1812,7 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   P.n = 1;
   P.total_heavy = 0;  // not used with the (blocks, 1, batch) grid
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true));
-  if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, spread)) return rc;
+  if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, load)) return rc;
   if (int32_t rc = launch_fused(P, dim3(P.run[0].plane, 1, B), p, scale, st)) return rc;
   if (int32_t rc = launch_dkdv_reduce(P.run[0], B, p, scale, st)) return rc;
   return launch_convert(T, p, tokens, sc, dq, scale, st);
@@ -1819,7 +1822,7 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
 // units share one launch of the prep, fused and convert kernels.
 int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, const unigist_problem& p, float scale,
                               const void* q, const void* k, const void* v, const void* o, const float* lse,
-                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, cudaStream_t st) {
+                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load, cudaStream_t st) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   const bool f32 = (p.flags & UNIGIST_FLAG_DOUT_FP32) != 0;
   const BwdScratch sc = carve_scratch(workspace, tokens, Hq, D, f32, true);
@@ -1831,7 +1834,7 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
     char* at = static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true);
     for (int i = 0; i < n_runs; ++i) {
       partial_of[i] = reinterpret_cast<float*>(at);
-      at += bwd_partial_bytes(runs[i].g, runs[i].batch, Hq, Hkv, true, false);
+      at += bwd_partial_bytes(runs[i].g, runs[i].batch, Hq, Hkv, true, load);
     }
   }
   for (int first = 0; first < n_runs; first += kMaxRunsPerLaunch) {
@@ -1857,7 +1860,7 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
                                     (const char*)do_src + r.first_row * rq, (const char*)k + r.first_row * rk,
                                     (const char*)v + r.first_row * rk, sc.dq32 + r.first_row * Hq * D,
                                     lse + r.first_row * Hq, sc.delta + r.first_row * Hq, (char*)dk + r.first_row * rk,
-                                    (char*)dv + r.first_row * rk, partial_of[first + order[i]], false))
+                                    (char*)dv + r.first_row * rk, partial_of[first + order[i]], load))
         return rc;
       ctas += (long long)P.run[i].plane * r.batch;
       if (ctas > 0x7fffffffLL) return fail(UNIGIST_ERR_SHAPE, "packed sample too large for one grid");

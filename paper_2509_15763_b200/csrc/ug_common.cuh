@@ -219,12 +219,12 @@ int32_t launch_fwd_sm100_runs(const SeqRun* runs, int n_runs, const unigist_prob
 int32_t fwd_sm100_take_timeout(bool* timed_out);
 int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, const void* q,
                          const void* k, const void* v, const void* o, const float* lse,
-                         const void* d_o, void* dq, void* dk, void* dv, void* workspace, bool spread,
+                         const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load,
                          cudaStream_t st);
 // The same over a packed sample (head_dim 128; `runs` in token order, `tokens` = rows of the packed tensors).
 int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, const unigist_problem& p, float scale,
                               const void* q, const void* k, const void* v, const void* o, const float* lse,
-                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, cudaStream_t st);
+                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load, cudaStream_t st);
 // The fused backward serves head_dim 128 unless a fixed dQ summation order is asked for; otherwise two kernels.
 inline bool bwd_is_fused(int D, uint32_t flags) { return D == 128 && !(flags & UNIGIST_FLAG_DETERMINISTIC_DQ); }
 // Bytes of backward scratch for `tokens` packed tokens: Delta, the bf16 copy of an fp32 dO, and for the fused
@@ -232,8 +232,11 @@ inline bool bwd_is_fused(int D, uint32_t flags) { return D == 128 && !(flags & U
 size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool fused);
 // Bytes behind that scratch for the fp32 partial dK / dV of the sink and gist key tiles whose walk over the
 // queries is cut into chunks (0 where nothing is cut, or the backward is not the fused one), for `batch` sequences
-// of geometry g.  spread: as the cuts of a small problem want it; without, the least that is accepted.
-size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, bool spread);
+// of geometry g.  load: the steps of the call per SM, which say where a walk is worth cutting, or -1 for the least that is
+// accepted.
+size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, long long load);
+// Steps (key tile, query tile, query head) of `batch` sequences, to within a tile a walk.
+long long bwd_steps(const Geom& g, int batch, int Hq);
 int32_t bwd_sm100_take_timeout(bool* timed_out);
 int32_t launch_compact_gather(const Geom& g, const unigist_problem& p, const void* k,
                               const void* v, void* kc, void* vc, int num_blocks,

@@ -62,3 +62,28 @@ def test_without_room_for_partial_sums(w):
     assert torch.equal(uncut[1], between[1]) and torch.equal(uncut[2], between[2])
     with pytest.raises(ug.UnigistError):
         bwd(least - 16)
+
+
+@pytest.mark.parametrize("docs", [[1024, 64], [32, 1200, 1200, 8]], ids=str)
+def test_packed_sample(docs):
+    p = ug.Problem(1, 8, 8, 64, 8, 1, 128, num_sinks=2)
+    n = ug.unigist_docs_total_len(p, docs)
+    g = torch.Generator(device=DEV).manual_seed(610 + len(docs))
+    q, k, v, do = (torch.randn(1, n, h, 128, generator=g, device=DEV).bfloat16() for h in (8, 1, 1, 8))
+    o, lse = torch.empty_like(q), torch.empty(8 * n, device=DEV)
+    ug.unigist_attn_fwd_docs(p, docs, q, k, v, o, lse)
+    al = lambda x: -(-x // 256) * 256
+    full, least = ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, docs), al(n * 8 * 4) + al(n * 8 * 128 * 4)
+    assert full > least
+    got = []
+    for size in (full, full, least):
+        ws = torch.full((size + 4096,), 7, dtype=torch.uint8, device=DEV)
+        got.append([torch.full_like(x, float("nan")) for x in (q, k, v)])
+        ug.unigist_attn_bwd_docs(p, docs, q, k, v, o, lse, do, *got[-1], ws[:size])
+        ug.unigist_device_status()
+        assert bool((ws[size:] == 7).all())
+    assert torch.equal(got[0][1], got[1][1]) and torch.equal(got[0][2], got[1][2])
+    for a, b in zip(got[0], got[2]):
+        assert float((a.float() - b.float()).norm()) <= 2 ** -8 * float(b.float().norm())
+    with pytest.raises(ug.UnigistError):
+        ug.unigist_attn_bwd_docs(p, docs, q, k, v, o, lse, do, *got[0], ws[:least - 16])
