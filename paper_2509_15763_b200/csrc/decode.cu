@@ -208,18 +208,19 @@ struct Walk {
 // kFlat = true: grid (n, Hkv); block x takes the x-th of n equal shares of all sequences' pages laid end to end, so
 // that sequences of any lengths keep every block equally busy; a sequence that lies inside one share is finished
 // there, one that is cut leaves a partial result per share in its flat_slot, for decode_combine_kernel.
-template <bool kFlat>
+// kApart: a stage's K and V arrive and are free again each by itself, instead of together (full_k, free_v).  A warp has one
+// stage; with barriers of its own the K of its next page comes under this one's softmax and P V.  That pays where walks are
+// short and bound by latency and a warp takes more than one page (8 sequences of 2112 tokens: 11.3 -> 10.6 us); with one page
+// a warp it only costs (one of 1337: 5.38 -> 5.41), and a long walk is bound by the memory system, which takes K and V apart
+// badly (past six rounds of pages: one of 65536, 44.5 -> 45.3 us; flat, 64 of 9216: 345 -> 357).
+template <bool kFlat, bool kApart>
 __global__ void __launch_bounds__(THREADS, 2)
 decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                     const __grid_constant__ DecParams P) {
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
-  // Barriers, + 8 * stage.  Split by rank, walks are short and bound by latency: a warp has one stage, and the K of its next
-  // page comes under this one's softmax and P V, since K has barriers of its own (8 sequences of 2112 tokens: 11.3 -> 10.7
-  // us).  The flat walk is bound by the memory system, which takes K and V apart badly (64 sequences of 9216: 345 -> 357 us):
-  // there both arrive (full_k) and are free again (free_v) together.
-  constexpr bool kApart = !kFlat;
+  // barriers, + 8 * stage
   const uint32_t full_k = base + DecSmem::kOffBars, full_v = full_k + 8 * STAGES, free_k = full_v + 8 * STAGES,
                  free_v = free_k + 8 * STAGES;
   float* merge = reinterpret_cast<float*>(gen + DecSmem::kOffMerge);
@@ -268,34 +269,53 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
     while (ok && w.next(P)) {
       const int32_t* row = P.table + (long long)w.seq * P.max_blocks;
       int32_t phys_mine = 0;
-      constexpr int kRound = kFlat ? 1 : STAGES;  // the K of a round of pages, then their V
-      for (int j0 = 0; j0 < w.count && ok; j0 += kRound) {
-        int row0[kRound];
-#pragma unroll
-        for (int u = 0; u < kRound; ++u) {
-          const int j = j0 + u;
-          if (j >= w.count) break;
-          if ((j & 31) == 0) {  // the next 32 block-table entries, one per lane
-            phys_mine = j + lane < w.count ? row[w.first + j + lane] : 0;
-            phys_mine = min(max(phys_mine, 0), P.num_blocks - 1);  // never read outside the cache
+      auto entries = [&](int j) {  // the next 32 block-table entries, one per lane
+        if (j & 31) return;
+        phys_mine = j + lane < w.count ? row[w.first + j + lane] : 0;
+        phys_mine = min(max(phys_mine, 0), P.num_blocks - 1);  // never read outside the cache
+      };
+      auto row_of = [&](int j) { return (__shfl_sync(0xffffffffu, phys_mine, j & 31) * P.Hkv + hk) * PG; };
+      if constexpr (!kApart) {
+        for (int j = 0; j < w.count; ++j) {
+          entries(j);
+          const int row0 = row_of(j), i = i0 + j, st = i % STAGES, use = i / STAGES;
+          if (use > 0) ok = mbar_wait_warp(free_v + 8 * st, (use - 1) & 1);
+          if (!ok) break;
+          if (lane == 0) {
+            const uint32_t full = full_k + 8 * st, dst = base + st * STAGE_BYTES;
+            mbar_arrive_expect_tx(full, STAGE_BYTES);
+            tma_load_2d(dst, &tm_k, full, 0, row0);
+            tma_load_2d(dst + SLAB_BYTES, &tm_k, full, 64, row0);
+            tma_load_2d(dst + PAGE_BYTES, &tm_v, full, 0, row0);
+            tma_load_2d(dst + PAGE_BYTES + SLAB_BYTES, &tm_v, full, 64, row0);
           }
-          row0[u] = (__shfl_sync(0xffffffffu, phys_mine, j & 31) * P.Hkv + hk) * PG;
+          __syncwarp();
         }
+      } else {
+        for (int j0 = 0; j0 < w.count && ok; j0 += STAGES) {  // the K of a round of pages, then their V
+          int row0[STAGES];
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
+          for (int u = 0; u < STAGES; ++u) {
+            if (j0 + u >= w.count) break;
+            entries(j0 + u);
+            row0[u] = row_of(j0 + u);
+          }
 #pragma unroll
-          for (int u = 0; u < kRound; ++u) {
-            const int i = i0 + j0 + u, st = i % STAGES, use = i / STAGES;
-            if (j0 + u >= w.count || !ok) break;
-            if (use > 0 && (kApart || v == 0)) ok = mbar_wait_warp((kApart && v == 0 ? free_k : free_v) + 8 * st, (use - 1) & 1);
-            if (!ok) break;
-            if (lane == 0) {
-              const uint32_t full = (kApart && v ? full_v : full_k) + 8 * st, dst = base + st * STAGE_BYTES + v * PAGE_BYTES;
-              if (kApart || v == 0) mbar_arrive_expect_tx(full, kApart ? PAGE_BYTES : STAGE_BYTES);
-              tma_load_2d(dst, v ? &tm_v : &tm_k, full, 0, row0[u]);
-              tma_load_2d(dst + SLAB_BYTES, v ? &tm_v : &tm_k, full, 64, row0[u]);
+          for (int v = 0; v < 2; ++v) {
+#pragma unroll
+            for (int u = 0; u < STAGES; ++u) {
+              const int i = i0 + j0 + u, st = i % STAGES, use = i / STAGES;
+              if (j0 + u >= w.count || !ok) break;
+              if (use > 0) ok = mbar_wait_warp((v ? free_v : free_k) + 8 * st, (use - 1) & 1);
+              if (!ok) break;
+              if (lane == 0) {
+                const uint32_t full = (v ? full_v : full_k) + 8 * st, dst = base + st * STAGE_BYTES + v * PAGE_BYTES;
+                mbar_arrive_expect_tx(full, PAGE_BYTES);
+                tma_load_2d(dst, v ? &tm_v : &tm_k, full, 0, row0[u]);
+                tma_load_2d(dst + SLAB_BYTES, v ? &tm_v : &tm_k, full, 64, row0[u]);
+              }
+              __syncwarp();
             }
-            __syncwarp();
           }
         }
       }
@@ -603,7 +623,7 @@ int max_clusters(int c) {
   }
   int n = cached[dev][i].load(std::memory_order_relaxed);
   if (n > 0) return n;
-  const auto kern = decode_split_kernel<false>;
+  const auto kern = decode_split_kernel<false, false>;
   cudaLaunchAttribute at = {};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = c;
@@ -706,7 +726,9 @@ int32_t launch_decode(int S, int Hq, int Hkv, int D, float scale, const void* q,
   P.S = S, P.Hq = Hq, P.Hkv = Hkv, P.G = G, P.num_blocks = num_blocks, P.max_blocks = max_blocks;
   P.holes_stride = holes_stride, P.holes_off = holes_off;
   P.scale_log2 = scale * LOG2E;
-  const auto kern = plan.flat ? decode_split_kernel<true> : decode_split_kernel<false>;
+  const int walk = (max_blocks + plan.c - 1) / plan.c;  // pages a block takes of the longest possible sequence
+  const bool apart = !plan.flat && walk > kConsumers && walk <= 6 * kConsumers;
+  const auto kern = plan.flat ? decode_split_kernel<true, false> : apart ? decode_split_kernel<false, true> : decode_split_kernel<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem::kBytes);
   const int cluster = plan.flat || plan.split ? 1 : plan.c;
   if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
