@@ -1488,37 +1488,69 @@ __device__ __forceinline__ int count_q_tiles(const Geom& g, const FastDiv& rdiv,
   return n;
 }
 
+// The launch units of a fused backward whose walks were cut, for the kernel below.
+struct ReduceRun {
+  Geom g;
+  const float* partial;
+  __nv_bfloat16 *dk, *dv;
+  int n_sink_kt, n_gist_kt, n_chunks, chunk_tiles;
+  int begin;  // first block of this unit (flat grid)
+};
+template <int kRuns>
+struct ReduceRuns {
+  ReduceRun run[kRuns];
+  int n;
+};
+
 // dK, dV of the sink and gist key tiles whose walk was cut into several chunks: the chunks' fp32 partial sums
 // added in chunk order (the same bits on every run), scaled, rounded to bf16 and stored at the keys' rows.
-// One block per (16 rows of a heavy key tile, KV head, batch index), a warp per key row.
+// The units of a packed sample go in one launch (each by itself cost 5 - 7 us a unit: twelve documents of about 500 tokens, 16 / 2
+// heads, 226 -> 147 us for the whole backward).  Bound by the latency of the chunks' loads: a warp takes one key row, four chunks
+// of dK and dV in flight (with four rows a warp 11264 raw tokens, 19 chunks, took 288 us instead of 261).
+constexpr int kReduceBlocks = 32;  // per heavy key tile, KV head and sequence
+template <int kRuns>
 __global__ void __launch_bounds__(128)
-dkdv_reduce_kernel(Geom g, int interleaved, int Hkv, int n_sink_kt, int n_gist_kt, int n_chunks, int chunk_tiles,
-                   const float* __restrict__ partial, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                   float scale, FastDiv rdiv) {
+dkdv_reduce_kernel(const __grid_constant__ ReduceRuns<kRuns> P, int interleaved, int Hkv, float scale, FastDiv rdiv) {
   pdl_wait();
-  const int rank = blockIdx.x >> 3, row0 = (blockIdx.x & 7) * 16, hk = blockIdx.y, b = blockIdx.z;
+  int ri = 0, bx = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
+  if constexpr (kRuns > 1) {
+    while (ri + 1 < P.n && (int)blockIdx.x >= P.run[ri + 1].begin) ++ri;
+    const int heavy = (P.run[ri].n_sink_kt + P.run[ri].n_gist_kt) * kReduceBlocks, plane = heavy * Hkv;
+    bx -= P.run[ri].begin;
+    b = bx / plane;
+    bx -= b * plane;
+    hk = bx / heavy;
+    bx -= hk * heavy;
+  }
+  const ReduceRun& R = P.run[ri];
+  const Geom& g = R.g;
+  const int n_sink_kt = R.n_sink_kt, n_gist_kt = R.n_gist_kt, n_chunks = R.n_chunks, chunk_tiles = R.chunk_tiles;
+  const int rank = bx / kReduceBlocks, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int krow = bx % kReduceBlocks * 4 + warp;
   const int n_heavy_kt = n_sink_kt + n_gist_kt;
   const int kseg = rank < n_sink_kt ? kSegSink : kSegGist;
   const int kt = rank - (kseg == kSegSink ? 0 : n_sink_kt);
   const int key_a = kt * 128, key_b = min(key_a + 127, seg_len(g, kseg) - 1);
   const int n_tiles = count_q_tiles(g, rdiv, kseg, key_a, key_b);
-  if (n_tiles <= chunk_tiles) return;  // a single chunk: the fused kernel stored dK, dV itself
+  if (n_tiles <= chunk_tiles || key_a + krow > key_b) return;  // a single chunk: the fused kernel stored dK, dV itself
   const int chunks = (n_tiles + chunk_tiles - 1) / chunk_tiles;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float* base = partial + ((((long long)b * Hkv + hk) * n_heavy_kt + rank) * n_chunks) * 2 * 128 * 128;
-  for (int krow = row0 + warp; krow < row0 + 16 && key_a + krow <= key_b; krow += 4) {
-    const long long tok = (long long)b * g.N + seg_row_to_token(g, interleaved != 0, kseg, key_a + krow);
+  const float* base = R.partial + ((((long long)b * Hkv + hk) * n_heavy_kt + rank) * n_chunks) * 2 * 128 * 128;
+  const long long tok = (long long)b * g.N + seg_row_to_token(g, interleaved != 0, kseg, key_a + krow);
+  float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+#pragma unroll 4
+  for (int c = 0; c < chunks; ++c) {
 #pragma unroll
     for (int which = 0; which < 2; ++which) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int c = 0; c < chunks; ++c) {
-        const float4 x = __ldcs(reinterpret_cast<const float4*>(base + ((long long)(c * 2 + which) * 128 + krow) * 128) + lane);
-        acc.x += x.x, acc.y += x.y, acc.z += x.z, acc.w += x.w;
-      }
-      const float mul = which == 0 ? scale : 1.f;
-      __nv_bfloat16* dst = (which == 0 ? dk : dv) + (tok * Hkv + hk) * 128 + lane * 4;
-      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc.x * mul, acc.y * mul), pack_bf16(acc.z * mul, acc.w * mul));
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(base + ((long long)(c * 2 + which) * 128 + krow) * 128) + lane);
+      acc[which].x += x.x, acc[which].y += x.y, acc[which].z += x.z, acc[which].w += x.w;
     }
+  }
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    const float mul = which == 0 ? scale : 1.f;
+    __nv_bfloat16* dst = (which == 0 ? R.dk : R.dv) + (tok * Hkv + hk) * 128 + lane * 4;
+    *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[which].x * mul, acc[which].y * mul),
+                                                pack_bf16(acc[which].z * mul, acc[which].w * mul));
   }
 }
 
@@ -1694,13 +1726,22 @@ int32_t launch_fused(const BwdRuns<kRuns>& P, dim3 grid, const unigist_problem& 
   return check_launch("tcgen05 fused backward kernel");
 }
 
-// Adds up the chunks' partial dK / dV of one launch unit (nothing to do where no key tile has several chunks).
-int32_t launch_dkdv_reduce(const BwdRun& R, int batch, const unigist_problem& p, float scale, cudaStream_t st) {
-  if (R.n_chunks <= 1) return UNIGIST_OK;
+// Adds a unit to the reduce kernel's, from block `begin` on, if its walks were cut.  -> its blocks per KV head and sequence.
+template <int kRuns>
+int add_reduce_run(ReduceRuns<kRuns>* P, const BwdRun& R, int begin) {
+  if (R.n_chunks <= 1) return 0;
+  P->run[P->n++] = {R.g, R.partial, R.dk, R.dv, R.n_sink_kt, R.n_gist_kt, R.n_chunks, R.chunk_tiles, begin};
+  return (R.n_sink_kt + R.n_gist_kt) * kReduceBlocks;
+}
+
+// Adds up the chunks' partial dK / dV of the units that were cut (nothing to do where no key tile has several chunks).
+template <int kRuns>
+int32_t launch_dkdv_reduce(const ReduceRuns<kRuns>& P, dim3 grid, const unigist_problem& p, float scale, cudaStream_t st) {
+  if (P.n == 0) return UNIGIST_OK;
   {
     KernelScope ks("dkdv_reduce_kernel", st);
-    launch_chained(dkdv_reduce_kernel, dim3((R.n_sink_kt + R.n_gist_kt) * 8, p.num_kv_heads, batch), 128, 0, st, 1, R.g, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_kv_heads, R.n_sink_kt, R.n_gist_kt, R.n_chunks,
-        R.chunk_tiles, R.partial, R.dk, R.dv, scale, make_fastdiv(p.ratio));
+    launch_chained(dkdv_reduce_kernel<kRuns>, grid, 128, 0, st, 1, P, (p.flags & UNIGIST_FLAG_INTERLEAVED) ? 1 : 0, p.num_kv_heads,
+                   scale, make_fastdiv(p.ratio));
   }
   return check_launch("dK/dV reduce kernel");
 }
@@ -1814,7 +1855,10 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true));
   if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, load)) return rc;
   if (int32_t rc = launch_fused(P, dim3(P.run[0].plane, 1, B), p, scale, st)) return rc;
-  if (int32_t rc = launch_dkdv_reduce(P.run[0], B, p, scale, st)) return rc;
+  ReduceRuns<1> C;
+  C.n = 0;
+  const int reduce_blocks = add_reduce_run(&C, P.run[0], 0);
+  if (int32_t rc = launch_dkdv_reduce(C, dim3(reduce_blocks, Hkv, B), p, scale, st)) return rc;
   return launch_convert(T, p, tokens, sc, dq, scale, st);
 }
 
@@ -1876,7 +1920,15 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
       P.run[i].raw_begin = at;
       at += P.run[i].raw_plane * runs[first + order[i]].batch;
     }
+    ReduceRuns<kMaxRunsPerLaunch> C;
+    C.n = 0;
+    long long reduce_ctas = 0;
+    for (int i = 0; i < n; ++i) {
+      reduce_ctas += (long long)add_reduce_run(&C, P.run[i], (int)reduce_ctas) * Hkv * runs[first + order[i]].batch;
+      if (reduce_ctas > 0x7fffffffLL) return fail(UNIGIST_ERR_SHAPE, "packed sample too large for one grid");
+    }
     for (int i = n; i < kMaxRunsPerLaunch; ++i) T.run[i] = T.run[0], P.run[i] = P.run[0];  // never selected
+    for (int i = C.n; i < kMaxRunsPerLaunch; ++i) C.run[i] = ReduceRun();
     // the per-token kernels of this launch see the tensors from packed token tok_lo on
     BwdScratch part = sc;
     if (part.do_bf16) part.do_bf16 += tok_lo * Hq * D;
@@ -1885,8 +1937,7 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
     if (int32_t rc = launch_prep(T, p, tok_hi - tok_lo, (const char*)d_o + tok_lo * rdo, (const char*)o + tok_lo * rq, part, st))
       return rc;
     if (int32_t rc = launch_fused(P, dim3((unsigned)ctas, 1, 1), p, scale, st)) return rc;
-    for (int i = 0; i < n; ++i)
-      if (int32_t rc = launch_dkdv_reduce(P.run[i], runs[first + order[i]].batch, p, scale, st)) return rc;
+    if (int32_t rc = launch_dkdv_reduce(C, dim3((unsigned)reduce_ctas, 1, 1), p, scale, st)) return rc;
     if (int32_t rc = launch_convert(T, p, tok_hi - tok_lo, part, (char*)dq + tok_lo * rq, scale, st)) return rc;
   }
   return UNIGIST_OK;

@@ -87,3 +87,30 @@ def test_packed_sample(docs):
         assert float((a.float() - b.float()).norm()) <= 2 ** -8 * float(b.float().norm())
     with pytest.raises(ug.UnigistError):
         ug.unigist_attn_bwd_docs(p, docs, q, k, v, o, lse, do, *got[0], ws[:least - 16])
+
+
+@pytest.mark.parametrize("sinks", [0, 130])
+def test_packed_sample_with_several_cut_documents(sinks):
+    """The partial sums of all units that are cut (runs of several sequences and several KV heads among them) are added by one
+    kernel: at most four launches in all, and eight where a sample has more than twelve units."""
+    p, ratio = ug.Problem(1, 8, 8, 64, 16, 2, 128, num_sinks=sinks), 8
+    for docs, launches in (([1200, 1200, 1024, 64, 904], 4), ([1200 - ratio * i for i in range(12)] + [1600, 8], 8)):
+        n = ug.unigist_docs_total_len(p, docs)
+        g = torch.Generator(device=DEV).manual_seed(620 + len(docs) + sinks)
+        q, k, v, do = (torch.randn(1, n, h, 128, generator=g, device=DEV).bfloat16() for h in (16, 2, 2, 16))
+        o, lse = torch.empty_like(q), torch.empty(16 * n, device=DEV)
+        ug.unigist_attn_fwd_docs(p, docs, q, k, v, o, lse)
+        al = lambda x: -(-x // 256) * 256
+        full, least = ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, docs), al(n * 16 * 4) + al(n * 16 * 128 * 4)
+        assert full > least
+        got = []
+        for size in (full, least):
+            ws = torch.full((size + 4096,), 7, dtype=torch.uint8, device=DEV)
+            got.append([torch.full_like(x, float("nan")) for x in (q, k, v)])
+            before = ug.unigist_launch_count()
+            ug.unigist_attn_bwd_docs(p, docs, q, k, v, o, lse, do, *got[-1], ws[:size])
+            assert ug.unigist_launch_count() - before <= launches
+            ug.unigist_device_status()
+            assert bool((ws[size:] == 7).all())
+        for a, b in zip(*got):
+            assert float((a.float() - b.float()).norm()) <= 2 ** -8 * float(b.float().norm())
