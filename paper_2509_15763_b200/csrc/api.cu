@@ -150,6 +150,17 @@ int32_t check_interleaved(const unigist_problem* p, const Geom& g) {
   return UNIGIST_OK;
 }
 
+// The backward's workspace for one problem: its scratch, and the partial sums of cut walks behind it.
+size_t bwd_scratch(const Geom& g, const unigist_problem* p) {
+  return bwd_scratch_bytes((long long)p->batch * g.N, p->num_q_heads, p->head_dim, (p->flags & UNIGIST_FLAG_DOUT_FP32) != 0,
+                           bwd_is_fused(p->head_dim, p->flags));
+}
+size_t bwd_partials(const Geom& g, const unigist_problem* p, bool spread) {
+  if (!bwd_is_fused(p->head_dim, p->flags)) return 0;
+  const SeqRun unit = {g, p->batch, 0};
+  return bwd_partial_bytes(&unit, 1, p->num_q_heads, p->num_kv_heads, spread);
+}
+
 }  // namespace ug
 
 using namespace ug;
@@ -196,10 +207,8 @@ size_t unigist_workspace_bytes(const unigist_problem* p, int32_t op) {
     case UNIGIST_OP_BWD:
       // Delta [B,Hq,N] fp32, a bf16 copy of dO when it arrives as fp32, and for the fused tensor-core backward
       // the fp32 dQ accumulator and the chunks' partial dK / dV
-      return bwd_scratch_bytes((long long)p->batch * g.N, p->num_q_heads, p->head_dim,
-                               (p->flags & UNIGIST_FLAG_DOUT_FP32) != 0, bwd_is_fused(p->head_dim, p->flags)) +
-             bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, bwd_is_fused(p->head_dim, p->flags),
-                               bwd_steps(g, p->batch, p->num_q_heads) / sm_count());
+      return bwd_scratch(g, p) +
+             bwd_partials(g, p, true);
     case UNIGIST_OP_COMPACT: {
       const size_t L = (size_t)g.s + g.n + (size_t)g.k * g.r;
       return align_up(2 * (size_t)p->batch * L * p->num_kv_heads * p->head_dim * 2, 256);
@@ -314,17 +323,14 @@ int32_t unigist_attn_bwd(const unigist_problem* p, const void* q, const void* k,
     if (!aligned16(x)) return fail(UNIGIST_ERR_ALIGNMENT, "tensor pointers must be 16-byte aligned");
   if (reinterpret_cast<uintptr_t>(lse) & 3) return fail(UNIGIST_ERR_ALIGNMENT, "lse must be 4-byte aligned");
   if (int32_t rc = check_interleaved(p, g)) return rc;
-  // long walks are cut where there is room for their partial sums, which is not asked for
-  const size_t full = unigist_workspace_bytes(p, UNIGIST_OP_BWD);
-  const bool fused = bwd_is_fused(p->head_dim, p->flags);
-  const long long load = bwd_steps(g, p->batch, p->num_q_heads) / sm_count();
-  const size_t need = full - bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, fused, load) +
-                      bwd_partial_bytes(g, p->batch, p->num_q_heads, p->num_kv_heads, fused, -1);
+  // walks are spread over idle SMs where there is room for their partial sums, which is not asked for
+  const bool spread = workspace && ws_bytes >= unigist_workspace_bytes(p, UNIGIST_OP_BWD);
+  const size_t need = spread ? 0 : bwd_scratch(g, p) + bwd_partials(g, p, false);
   if (!workspace || ws_bytes < need)
     return fail(UNIGIST_ERR_WORKSPACE, "backward needs %zu bytes of workspace, got %zu", need,
                 ws_bytes);
   // the fused kernel for head_dim 128, the two-kernel path for head_dim 64; both on the tensor cores
-  return launch_bwd_sm100(g, *p, scale, q, k, v, o, lse, d_o, dq, dk, dv, workspace, ws_bytes >= full ? load : -1, (cudaStream_t)stream);
+  return launch_bwd_sm100(g, *p, scale, q, k, v, o, lse, d_o, dq, dk, dv, workspace, spread, (cudaStream_t)stream);
 }
 
 // ---- cross-document masking: a packed sample is a list of independent sequences -------------------------------
@@ -382,27 +388,28 @@ int32_t doc_runs(const unigist_problem* p, int32_t num_docs, const int32_t* doc_
   return rc;
 }
 
-// Steps of the packed sample's fused backward per SM, and its workspace: one scratch layout over all packed tokens, then the
-// runs' partial dK / dV.
-long long docs_load(const unigist_problem* p, int32_t num_docs, const int32_t* doc_raw_len) {
-  long long steps = 0;
-  for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t, int32_t) {
-    Geom g;
-    if (check_problem(&run, &g, nullptr) == UNIGIST_OK) steps += bwd_steps(g, run.batch, run.num_q_heads);
+// Workspace of the packed sample's fused backward: one scratch layout over all packed tokens, then the partial sums of the
+// runs, launch by launch.
+size_t docs_bwd_bytes(const unigist_problem* p, int32_t num_docs, const int32_t* doc_raw_len, bool spread) {
+  SeqRun launch[kMaxRunsPerLaunch];
+  int n = 0;
+  int64_t tokens = 0;
+  size_t partials = 0;
+  auto flush = [&]() {
+    partials += bwd_partial_bytes(launch, n, p->num_q_heads, p->num_kv_heads, spread);
+    n = 0;
+  };
+  for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t base, int32_t) {
+    tokens = base + ((int64_t)run.num_sinks + run.raw_len + run.raw_len / run.ratio) * run.batch;
+    SeqRun& r = launch[n];
+    if (check_problem(&run, &r.g, nullptr) != UNIGIST_OK) return (int32_t)UNIGIST_OK;  // refused when it is launched
+    r.batch = run.batch;
+    r.first_row = base;
+    if (++n == kMaxRunsPerLaunch) flush();
     return (int32_t)UNIGIST_OK;
   });
-  return steps / sm_count();
-}
-size_t docs_bwd_bytes(const unigist_problem* p, int32_t num_docs, const int32_t* doc_raw_len, long long load) {
-  size_t need = bwd_scratch_bytes(unigist_docs_total_len(p, num_docs, doc_raw_len), p->num_q_heads, p->head_dim,
-                                  (p->flags & UNIGIST_FLAG_DOUT_FP32) != 0, true);
-  for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t, int32_t) {
-    Geom g;
-    if (check_problem(&run, &g, nullptr) == UNIGIST_OK)
-      need += bwd_partial_bytes(g, run.batch, run.num_q_heads, run.num_kv_heads, true, load);
-    return (int32_t)UNIGIST_OK;
-  });
-  return need;
+  flush();
+  return bwd_scratch_bytes(tokens, p->num_q_heads, p->head_dim, (p->flags & UNIGIST_FLAG_DOUT_FP32) != 0, true) + partials;
 }
 
 }  // namespace
@@ -418,7 +425,7 @@ int64_t unigist_docs_total_len(const unigist_problem* p, int32_t num_docs, const
 size_t unigist_docs_workspace_bytes(const unigist_problem* p, int32_t op, int32_t num_docs, const int32_t* doc_raw_len) {
   if (check_docs(p, num_docs, doc_raw_len) != UNIGIST_OK) return 0;
   if (op != UNIGIST_OP_BWD) return 0;
-  if (bwd_is_fused(p->head_dim, p->flags)) return docs_bwd_bytes(p, num_docs, doc_raw_len, docs_load(p, num_docs, doc_raw_len));
+  if (bwd_is_fused(p->head_dim, p->flags)) return docs_bwd_bytes(p, num_docs, doc_raw_len, true);
   size_t need = 0;  // head_dim 64: one launch set per run, each with its own slice
   for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t, int32_t) {
     need += align_up(unigist_workspace_bytes(&run, op), 256);
@@ -453,9 +460,11 @@ int32_t unigist_attn_bwd_docs(const unigist_problem* p, int32_t num_docs, const 
   for (const void* x : ptrs)
     if (!aligned16(x)) return fail(UNIGIST_ERR_ALIGNMENT, "tensor pointers must be 16-byte aligned");
   if (reinterpret_cast<uintptr_t>(lse) & 3) return fail(UNIGIST_ERR_ALIGNMENT, "lse must be 4-byte aligned");
-  const size_t full = unigist_docs_workspace_bytes(p, UNIGIST_OP_BWD, num_docs, doc_raw_len);
   const bool fused = bwd_is_fused(p->head_dim, p->flags);
-  const size_t need = fused ? docs_bwd_bytes(p, num_docs, doc_raw_len, -1) : full;
+  const size_t full = fused ? docs_bwd_bytes(p, num_docs, doc_raw_len, true)
+                            : unigist_docs_workspace_bytes(p, UNIGIST_OP_BWD, num_docs, doc_raw_len);
+  const bool spread = ws_bytes >= full;
+  const size_t need = fused && !spread ? docs_bwd_bytes(p, num_docs, doc_raw_len, false) : full;
   if (!workspace || ws_bytes < need)
     return fail(UNIGIST_ERR_WORKSPACE, "backward over documents needs %zu bytes of 16-byte aligned workspace, got %zu", need,
                 ws_bytes);
@@ -466,7 +475,7 @@ int32_t unigist_attn_bwd_docs(const unigist_problem* p, int32_t num_docs, const 
   const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->head_dim);
   if (fused)
     return launch_bwd_sm100_runs(runs.data(), (int)runs.size(), tokens, *p, scale, q, k, v, o, lse, d_o, dq, dk, dv,
-                                 workspace, ws_bytes >= full ? docs_load(p, num_docs, doc_raw_len) : -1, (cudaStream_t)stream);
+                                 workspace, spread, (cudaStream_t)stream);
   // the two-kernel backward (head_dim 64, or a fixed summation order asked for): the runs one after the other on the caller's stream
   const size_t rq = (size_t)p->num_q_heads * p->head_dim * 2, rk = (size_t)p->num_kv_heads * p->head_dim * 2;
   const size_t rdo = (p->flags & UNIGIST_FLAG_DOUT_FP32) ? 2 * rq : rq;

@@ -964,7 +964,6 @@ struct BwdRuns {
   int n;
   int total_heavy;  // flat grid: blocks of the sink / gist range
 };
-constexpr int kMaxRunsPerLaunch = 12;  // 12 units are 24 KB of kernel parameters (the limit is 32 KB)
 static_assert(sizeof(BwdRuns<kMaxRunsPerLaunch>) + 256 <= 32764, "the launch units must fit the kernel parameter space");
 
 template <int kRuns>
@@ -1644,6 +1643,11 @@ int tiles(long long rows) { return (int)((rows + 127) / 128); }
 long long raw_walk(const Geom& g) {
   return std::min(tiles((g.k + 1ll) * g.r) + 1, tiles(g.T)) + std::min(tiles(g.k + 1ll) + 1, tiles(g.n));
 }
+// Steps (key tile, query tile, query head) of `batch` sequences.  A gist key is seen by the later half of all rows on average.
+long long bwd_steps(const Geom& g, int batch, int Hq) {
+  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
+  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk(g)) * Hq * batch;
+}
 
 // How the walk of a sink or gist key tile over its query tiles is cut (head_dim 128).  Not at all while the rows
 // one KV head's blocks sweep (Q, dO and the fp32 dQ of its G query heads: 1 KB per token and head) fit in three
@@ -1746,6 +1750,19 @@ int32_t launch_dkdv_reduce(const ReduceRuns<kRuns>& P, dim3 grid, const unigist_
   return check_launch("dK/dV reduce kernel");
 }
 
+// Bytes of a unit's partial sums, and what a launch holds per SM (the load that the cut goes by).
+size_t unit_partial_bytes(const SeqRun& r, int Hq, int Hkv, long long load) {
+  int C, chunk_tiles;
+  bwd_chunking(r.g, r.batch, Hq, Hkv, load, &C, &chunk_tiles);
+  if (C <= 1) return 0;
+  return align256((size_t)r.batch * Hkv * (tiles(r.g.s) + tiles(r.g.n)) * C * 2 * 128 * 128 * sizeof(float));
+}
+long long launch_load(const SeqRun* runs, int n_runs, int Hq) {
+  long long steps = 0;
+  for (int i = 0; i < n_runs; ++i) steps += bwd_steps(runs[i].g, runs[i].batch, Hq);
+  return steps / sm_count();
+}
+
 // Whether two blocks share each sink or gist key tile of the dK / dV kernel: where the longest walk (the first gist key tile's)
 // would otherwise be the kernel's tail.  All blocks' steps are counted to within a tile, per SM; a walk up to 3/4 of that and
 // 22 steps ends under the raw key tiles that are left, and sharing it only costs blocks (us of the whole backward, shared and
@@ -1814,24 +1831,16 @@ size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool f
   return b;
 }
 
-// A gist key is seen by the later half of all rows on average.
-long long bwd_steps(const Geom& g, int batch, int Hq) {
-  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
-  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk(g)) * Hq * batch;
-}
-
-size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, long long load) {
-  if (!fused) return 0;
-  int C, tiles;
-  bwd_chunking(g, batch, Hq, Hkv, load, &C, &tiles);
-  if (C <= 1) return 0;
-  const size_t n_heavy = (g.s + 127) / 128 + (g.n + 127) / 128;
-  return align256((size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float));
+size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool spread) {
+  const long long load = spread ? launch_load(runs, n_runs, Hq) : -1;
+  size_t b = 0;
+  for (int i = 0; i < n_runs; ++i) b += unit_partial_bytes(runs[i], Hq, Hkv, load);
+  return b;
 }
 
 int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, const void* q, const void* k,
                          const void* v, const void* o, const float* lse, const void* d_o, void* dq, void* dk,
-                         void* dv, void* workspace, long long load, cudaStream_t st) {
+                         void* dv, void* workspace, bool spread, cudaStream_t st) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads, B = p.batch;
   const bool f32 = (p.flags & UNIGIST_FLAG_DOUT_FP32) != 0;
   const long long tokens = (long long)B * g.N;
@@ -1853,6 +1862,8 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   P.n = 1;
   P.total_heavy = 0;  // not used with the (blocks, 1, batch) grid
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true));
+  const SeqRun unit = {g, B, 0};
+  const long long load = spread ? launch_load(&unit, 1, Hq) : -1;
   if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, load)) return rc;
   if (int32_t rc = launch_fused(P, dim3(P.run[0].plane, 1, B), p, scale, st)) return rc;
   ReduceRuns<1> C;
@@ -1866,23 +1877,23 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
 // units share one launch of the prep, fused and convert kernels.
 int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, const unigist_problem& p, float scale,
                               const void* q, const void* k, const void* v, const void* o, const float* lse,
-                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load, cudaStream_t st) {
+                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, bool spread, cudaStream_t st) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   const bool f32 = (p.flags & UNIGIST_FLAG_DOUT_FP32) != 0;
   const BwdScratch sc = carve_scratch(workspace, tokens, Hq, D, f32, true);
   const void* do_src = f32 ? static_cast<const void*>(sc.do_bf16) : d_o;
   const size_t rq = (size_t)Hq * D * 2, rk = (size_t)Hkv * D * 2;
-  // the chunks' partial dK / dV: one slice per run, behind the scratch of the packed tokens
-  std::vector<float*> partial_of(n_runs);
-  {
-    char* at = static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true);
-    for (int i = 0; i < n_runs; ++i) {
-      partial_of[i] = reinterpret_cast<float*>(at);
-      at += bwd_partial_bytes(runs[i].g, runs[i].batch, Hq, Hkv, true, load);
-    }
-  }
+  // the chunks' partial dK / dV: one slice per run, in token order, behind the scratch of the packed tokens
+  char* partial_at = static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true);
   for (int first = 0; first < n_runs; first += kMaxRunsPerLaunch) {
     const int n = n_runs - first < kMaxRunsPerLaunch ? n_runs - first : kMaxRunsPerLaunch;
+    // the launches run one after the other: what one SM has to do in each goes by its own units
+    const long long load = spread ? launch_load(runs + first, n, Hq) : -1;
+    float* partial_of[kMaxRunsPerLaunch];
+    for (int i = 0; i < n; ++i) {
+      partial_of[i] = reinterpret_cast<float*>(partial_at);
+      partial_at += unit_partial_bytes(runs[first + i], Hq, Hkv, load);
+    }
     // the runs of one launch hold consecutive packed tokens [tok_lo, tok_hi)
     const long long tok_lo = runs[first].first_row;
     const long long tok_hi = runs[first + n - 1].first_row + (long long)runs[first + n - 1].g.N * runs[first + n - 1].batch;
@@ -1904,7 +1915,7 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
                                     (const char*)do_src + r.first_row * rq, (const char*)k + r.first_row * rk,
                                     (const char*)v + r.first_row * rk, sc.dq32 + r.first_row * Hq * D,
                                     lse + r.first_row * Hq, sc.delta + r.first_row * Hq, (char*)dk + r.first_row * rk,
-                                    (char*)dv + r.first_row * rk, partial_of[first + order[i]], load))
+                                    (char*)dv + r.first_row * rk, partial_of[order[i]], load))
         return rc;
       ctas += (long long)P.run[i].plane * r.batch;
       if (ctas > 0x7fffffffLL) return fail(UNIGIST_ERR_SHAPE, "packed sample too large for one grid");

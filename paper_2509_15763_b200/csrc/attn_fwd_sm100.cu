@@ -255,7 +255,6 @@ struct FwdRuns {
   FwdRun run[kRuns];
   int n;
 };
-constexpr int kMaxRunsPerLaunch = 12;  // 12 units are 20 KB of kernel parameters (the limit is 32 KB)
 static_assert(sizeof(FwdRuns<kMaxRunsPerLaunch>) + 256 <= 32764, "the launch units must fit the kernel parameter space");
 
 // The streams of a block: two tiles of one head, two heads on one tile, or one tile of one head.

@@ -209,6 +209,7 @@ int32_t launch_fwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
 // A run of `batch` consecutive sequences of one geometry inside packed [N_total, heads, D] tensors (a packed
 // sample under cross-document masking), starting at packed row first_row.  The *_runs launchers take the
 // tensors' base pointers and put up to twelve runs into one launch.
+constexpr int kMaxRunsPerLaunch = 12;  // 12 units are 20 or 24 KB of kernel parameters (the limit is 32 KB)
 struct SeqRun {
   Geom g;
   int batch;
@@ -219,24 +220,21 @@ int32_t launch_fwd_sm100_runs(const SeqRun* runs, int n_runs, const unigist_prob
 int32_t fwd_sm100_take_timeout(bool* timed_out);
 int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, const void* q,
                          const void* k, const void* v, const void* o, const float* lse,
-                         const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load,
+                         const void* d_o, void* dq, void* dk, void* dv, void* workspace, bool spread,
                          cudaStream_t st);
 // The same over a packed sample (head_dim 128; `runs` in token order, `tokens` = rows of the packed tensors).
 int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, const unigist_problem& p, float scale,
                               const void* q, const void* k, const void* v, const void* o, const float* lse,
-                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, long long load, cudaStream_t st);
+                              const void* d_o, void* dq, void* dk, void* dv, void* workspace, bool spread, cudaStream_t st);
 // The fused backward serves head_dim 128 unless a fixed dQ summation order is asked for; otherwise two kernels.
 inline bool bwd_is_fused(int D, uint32_t flags) { return D == 128 && !(flags & UNIGIST_FLAG_DETERMINISTIC_DQ); }
 // Bytes of backward scratch for `tokens` packed tokens: Delta, the bf16 copy of an fp32 dO, and for the fused
 // backward the fp32 dQ accumulator.
 size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool fused);
 // Bytes behind that scratch for the fp32 partial dK / dV of the sink and gist key tiles whose walk over the
-// queries is cut into chunks (0 where nothing is cut, or the backward is not the fused one), for `batch` sequences
-// of geometry g.  load: the steps of the call per SM, which say where a walk is worth cutting, or -1 for the least that is
-// accepted.
-size_t bwd_partial_bytes(const Geom& g, int batch, int Hq, int Hkv, bool fused, long long load);
-// Steps (key tile, query tile, query head) of `batch` sequences, to within a tile a walk.
-long long bwd_steps(const Geom& g, int batch, int Hq);
+// queries is cut into chunks (0 where nothing is cut), for the units of ONE launch of the fused backward.  spread: walks that are
+// cut only to spread them over idle SMs too; without them, the least that is accepted.
+size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool spread);
 int32_t bwd_sm100_take_timeout(bool* timed_out);
 int32_t launch_compact_gather(const Geom& g, const unigist_problem& p, const void* k,
                               const void* v, void* kc, void* vc, int num_blocks,

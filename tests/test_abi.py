@@ -126,3 +126,22 @@ def test_backward_workspace_sizes_hold_every_part():
     assert n_tot == sum(t + t // 4 for t in docs)
     assert ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, docs) == al(4 * n_tot * 4) + al(n_tot * 4 * 128 * 4)
     assert ug.unigist_docs_workspace_bytes(p, ug.OP_FWD, docs) == 0
+
+
+@pytest.mark.parametrize("sinks", [0, 5])
+def test_packed_backward_workspace_goes_by_launch(sinks):
+    """Up to twelve runs of equal documents share a launch, and the launches follow each other: where a long document's walks are
+    cut goes by the documents of its own launch, so the partial sums of a sample are those of its launches one by one."""
+    p, (hq, hkv, dim) = ug.Problem(1, 8, 8, 128, 16, 2, 128, num_sinks=sinks), (16, 2, 128)
+
+    def partial_sums(docs):
+        n, al = ug.unigist_docs_total_len(p, docs), lambda x: -(-x // 256) * 256
+        return ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, docs) - al(n * hq * 4) - al(n * hq * dim * 4)
+
+    first = [2048 + 8 * i for i in range(11)] + [4000, 4000]         # twelve runs
+    second = [4096] + [200 + 8 * i for i in range(11)]
+    third = [3000]
+    assert partial_sums(second) > 0 and partial_sums(third) > 0
+    assert partial_sums(first + second + third) == sum(map(partial_sums, (first, second, third)))
+    one = ug.Problem(1, 3000, 8, 128, hq, hkv, dim, num_sinks=sinks)  # a sample of one document is the problem itself
+    assert ug.unigist_workspace_bytes(one, ug.OP_BWD) == ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, third)
