@@ -158,7 +158,7 @@ size_t bwd_scratch(const Geom& g, const unigist_problem* p) {
 size_t bwd_partials(const Geom& g, const unigist_problem* p, bool spread) {
   if (!bwd_is_fused(p->head_dim, p->flags)) return 0;
   const SeqRun unit = {g, p->batch, 0};
-  return bwd_partial_bytes(&unit, 1, p->num_q_heads, p->num_kv_heads, spread);
+  return bwd_partial_bytes(&unit, 1, p->num_q_heads, p->num_kv_heads, true, spread);
 }
 
 }  // namespace ug
@@ -396,7 +396,7 @@ size_t docs_bwd_bytes(const unigist_problem* p, int32_t num_docs, const int32_t*
   int64_t tokens = 0;
   size_t partials = 0;
   auto flush = [&]() {
-    partials += bwd_partial_bytes(launch, n, p->num_q_heads, p->num_kv_heads, spread);
+    partials += bwd_partial_bytes(launch, n, p->num_q_heads, p->num_kv_heads, false, spread);
     n = 0;
   };
   for_each_doc_run(p, num_docs, doc_raw_len, [&](const unigist_problem& run, int64_t base, int32_t) {

@@ -115,7 +115,7 @@ bwd_prep_kernel(const __grid_constant__ TokRuns<kRuns> P, int interleaved, int H
 
 // Query rows (numbered inside the raw or the gist segment, inclusive) that see a given key:
 // Eq. 3 read column-wise.  An empty interval has lo > hi.
-__device__ __forceinline__ void key_q_interval(const Geom& g, const FastDiv& rdiv, bool key_is_raw, int key, bool key_valid,
+__host__ __device__ __forceinline__ void key_q_interval(const Geom& g, const FastDiv& rdiv, bool key_is_raw, int key, bool key_valid,
                                                bool q_is_raw, int& lo, int& hi) {
   if (!key_valid) {
     lo = 1;
@@ -144,7 +144,7 @@ __device__ __forceinline__ void key_q_interval(const Geom& g, const FastDiv& rdi
 
 // Query rows of segment qseg (numbered inside it, inclusive) that see key `key` of segment kseg:
 // Eq. 3 read column-wise, sinks included.  An empty interval has lo > hi.
-__device__ __forceinline__ void key_q_interval3(const Geom& g, const FastDiv& rdiv, int kseg, int key, bool key_valid, int qseg, int& lo,
+__host__ __device__ __forceinline__ void key_q_interval3(const Geom& g, const FastDiv& rdiv, int kseg, int key, bool key_valid, int qseg, int& lo,
                                                 int& hi) {
   lo = 1;
   hi = 0;
@@ -1475,7 +1475,7 @@ attn_bwd_fused_sm100_kernel(const __grid_constant__ BwdRuns<kRuns> P, int Hq, in
 }
 
 // Number of 128-query tiles that see a key tile [key_a, key_b] of segment kseg (all query segments).
-__device__ __forceinline__ int count_q_tiles(const Geom& g, const FastDiv& rdiv, int kseg, int key_a, int key_b) {
+__host__ __device__ __forceinline__ int count_q_tiles(const Geom& g, const FastDiv& rdiv, int kseg, int key_a, int key_b) {
   int n = 0;
 #pragma unroll
   for (int qseg = 0; qseg < 3; ++qseg) {
@@ -1639,14 +1639,39 @@ int32_t launch_convert(const TokRuns<kRuns>& T, const unigist_problem& p, long l
 }
 
 int tiles(long long rows) { return (int)((rows + 127) / 128); }
-// Query tiles that a raw key tile's walk has at most: k + 1 units and their gists.
-long long raw_walk(const Geom& g) {
-  return std::min(tiles((g.k + 1ll) * g.r) + 1, tiles(g.T)) + std::min(tiles(g.k + 1ll) + 1, tiles(g.n));
-}
-// Steps (key tile, query tile, query head) of `batch` sequences.  A gist key is seen by the later half of all rows on average.
-long long bwd_steps(const Geom& g, int batch, int Hq) {
-  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
-  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk(g)) * Hq * batch;
+// What a launch of the fused backward holds besides its longest walk, in steps (key tile, query tile, query head).
+struct LaunchLoad {
+  long long end;       // when the SMs would be through if no walk outlasted the others and the long ones were cut
+  long long late;      // when the last sink and gist key tiles start
+  long long raw_walk;  // longest walk of a raw key tile
+};
+// in_turn: one problem, whose sequences' blocks follow each other; otherwise all sink and gist key tiles come first.
+constexpr int kBlockSteps = 2;  // the fixed part of a block, in steps
+LaunchLoad launch_load(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_turn) {
+  const long long G = Hq / Hkv, sms = sm_count();
+  long long steps = 0, raw_walk = 0, blocks = 0, before_last = 0;
+  for (int i = 0; i < n_runs; ++i) {
+    const Geom& g = runs[i].g;
+    const FastDiv rdiv = make_fastdiv(g.r);
+    const long long n_heavy = tiles(g.s) + tiles(g.n), n_raw = tiles(g.T);
+    long long n_steps = 0, n_blocks = 0;
+    for (int kseg = 0; kseg < 3; ++kseg)
+      for (int key = 0; key < seg_len(g, kseg); key += 128) {
+        const int n = count_q_tiles(g, rdiv, kseg, key, std::min(key + 127, seg_len(g, kseg) - 1));
+        n_steps += n;
+        n_blocks += kseg != kSegRaw && n > (n_heavy + n_raw + 1) / 2 ? 2 : 1;  // (if it is cut, two at least)
+        if (kseg == kSegRaw) raw_walk = std::max(raw_walk, n * G);
+      }
+    steps += n_steps * Hq * runs[i].batch;
+    blocks += n_blocks * Hkv * runs[i].batch;
+    before_last = ((n_heavy + n_raw) * (runs[i].batch - 1) + n_heavy) * Hkv;
+  }
+  LaunchLoad load;
+  load.raw_walk = raw_walk;
+  load.end = (steps + kBlockSteps * blocks) / sms;
+  load.late = in_turn && before_last > sms ? std::max(0ll, load.end - load.end / runs[0].batch - raw_walk / 2) : 0;
+  if (blocks > sms) load.end += raw_walk / 2;  // blocks that start when others end do not end together
+  return load;
 }
 
 // How the walk of a sink or gist key tile over its query tiles is cut (head_dim 128).  Not at all while the rows
@@ -1654,14 +1679,16 @@ long long bwd_steps(const Geom& g, int batch, int Hq) {
 // quarters of the L2: however the blocks start, what one has read is still there for the next.  Otherwise into at
 // most four chunks of at least 16 query tiles, fewer where the chunks' fp32 partial sums would take more than
 // half the room of the dQ accumulator.
-// Where the longest sink or gist walk, and not the load of an SM, is the kernel's time (a step is about 2 us), that walk is
-// cut too, if the workspace has room (load >= 0, the steps of the launch per SM): into chunks of half of an SM's load, no shorter than a raw key tile's walk,
-// where that saves at least eight steps; the second kernel and the partial sums cost about 5 us (us of the whole backward,
-// uncut and cut: 512 raw tokens, ratio 4, 32 / 8 heads 63 and 54; 1024, 16 / 4 heads 92 and 51; 4096, ratio 16, window 128, 16
-// / 2 heads 598 and 130; 4096, window 1024, 32 / 8 heads 382 and 320; 9000, window 128 811 and 520; 16384, window 1024, longest
-// walk 576 steps, load 571: not cut).
+// Where the longest sink or gist walk would outlast the rest of the launch by eight steps or more (a step is about 2 us), that
+// walk is cut too, if the workspace has room (load != nullptr): into chunks of half of the time the rest takes, no shorter than
+// the longest raw key tile's walk; the second kernel and the partial sums cost about 5 us.  Whole backward, us, uncut and cut;
+// steps of the longest walk / of the rest: 512 raw tokens, ratio 4, window 64, 32 / 8 heads 61 and 50, 22 / 4; 1024, ratio 8,
+// window 128, 16 / 4 heads 91 and 47, 38 / 4; 4096, ratio 16, 16 / 2 heads 597 and 107, 274 / 16; 9000, ratio 8, 32 / 8 heads 805
+// and 509, 322 / 150; 4096, window 1024 378 and 310, 146 / 112; 16384 578 / 598, not cut; 4 x 384, ratio 16, window 128, 128
+// sinks, 64 / 8 heads 147 and 167, 42 / 44, not cut.  Over 1367 problems that it cuts, of 128 - 24000 tokens: half the uncut time
+// on average, 3 % above the best number of chunks, one slower than uncut by more than 3 %.
 // -> tiles per chunk, number of chunks of the longest walk (1 = no cutting, no partial sums).
-void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, long long load, int* n_chunks, int* chunk_tiles) {
+void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, const LaunchLoad* load, int* n_chunks, int* chunk_tiles) {
   const int n_raw = tiles(g.T), n_gist = tiles(g.n), n_heavy = tiles(g.s) + n_gist;
   const int max_tiles = n_heavy + n_raw;  // the first sink / gist key tile is seen by every query tile
   const size_t dq_bytes = (size_t)batch * g.N * Hq * 128 * sizeof(float);
@@ -1670,9 +1697,10 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, long long load, int
   while (C > 1 && ((max_tiles + C - 1) / C < 16 ||
                    (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2))
     --C;
-  if (load >= 0 && C == 1 && n_heavy > 0) {
-    const long long G = Hq / Hkv, longest = max_tiles * G, target = std::max(raw_walk(g) * G, load / 2);
-    if (longest - std::max(target, load) >= 8) C = (int)((longest + target - 1) / target);
+  if (load && C == 1 && n_heavy > 0) {
+    const long long longest = (long long)max_tiles * (Hq / Hkv), target = std::max(load->raw_walk, load->end / 2);
+    const long long start = load->late + kBlockSteps;
+    if (start + longest - std::max(start + target, load->end) >= 8) C = (int)((longest + target - 1) / target);
     while (C > 1 && (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2) --C;
   }
   *chunk_tiles = (max_tiles + C - 1) / C;
@@ -1684,7 +1712,7 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, long long load, int
 // interleaved tensors, and reduction maps over the fp32 dQ tensor (always shifted).
 int32_t fill_bwd_run(BwdRun* R, const Geom& g, const unigist_problem& p, int batch, const void* q, const void* do_src,
                      const void* k, const void* v, float* dq32, const float* lse, const float* delta, void* dk, void* dv,
-                     float* partial, long long load) {
+                     float* partial, const LaunchLoad* load) {
   const int D = p.head_dim, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   const bool il = (p.flags & UNIGIST_FLAG_INTERLEAVED) != 0;
   for (int sg = 0; sg < 3; ++sg) {
@@ -1750,17 +1778,20 @@ int32_t launch_dkdv_reduce(const ReduceRuns<kRuns>& P, dim3 grid, const unigist_
   return check_launch("dK/dV reduce kernel");
 }
 
-// Bytes of a unit's partial sums, and what a launch holds per SM (the load that the cut goes by).
-size_t unit_partial_bytes(const SeqRun& r, int Hq, int Hkv, long long load) {
+// Bytes of a unit's partial sums.
+size_t unit_partial_bytes(const SeqRun& r, int Hq, int Hkv, const LaunchLoad* load) {
   int C, chunk_tiles;
   bwd_chunking(r.g, r.batch, Hq, Hkv, load, &C, &chunk_tiles);
   if (C <= 1) return 0;
   return align256((size_t)r.batch * Hkv * (tiles(r.g.s) + tiles(r.g.n)) * C * 2 * 128 * 128 * sizeof(float));
 }
-long long launch_load(const SeqRun* runs, int n_runs, int Hq) {
-  long long steps = 0;
-  for (int i = 0; i < n_runs; ++i) steps += bwd_steps(runs[i].g, runs[i].batch, Hq);
-  return steps / sm_count();
+
+// Steps (key tile, query tile, query head) of `batch` sequences, estimated: a raw key tile's walk is taken as the longest that it
+// can be, k + 1 units and their gists; a gist key is seen by the later half of all rows on average.
+long long bwd_steps(const Geom& g, int batch, int Hq) {
+  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
+  const long long raw_walk = std::min(tiles((g.k + 1ll) * g.r) + 1, tiles(g.T)) + std::min(tiles(g.k + 1ll) + 1, tiles(g.n));
+  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk) * Hq * batch;
 }
 
 // Whether two blocks share each sink or gist key tile of the dK / dV kernel: where the longest walk (the first gist key tile's)
@@ -1831,10 +1862,11 @@ size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool f
   return b;
 }
 
-size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool spread) {
-  const long long load = spread ? launch_load(runs, n_runs, Hq) : -1;
+size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_turn, bool spread) {
+  LaunchLoad load;
+  if (spread) load = launch_load(runs, n_runs, Hq, Hkv, in_turn);
   size_t b = 0;
-  for (int i = 0; i < n_runs; ++i) b += unit_partial_bytes(runs[i], Hq, Hkv, load);
+  for (int i = 0; i < n_runs; ++i) b += unit_partial_bytes(runs[i], Hq, Hkv, spread ? &load : nullptr);
   return b;
 }
 
@@ -1863,8 +1895,10 @@ int32_t launch_bwd_sm100(const Geom& g, const unigist_problem& p, float scale, c
   P.total_heavy = 0;  // not used with the (blocks, 1, batch) grid
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + bwd_scratch_bytes(tokens, Hq, D, f32, true));
   const SeqRun unit = {g, B, 0};
-  const long long load = spread ? launch_load(&unit, 1, Hq) : -1;
-  if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, load)) return rc;
+  LaunchLoad load;
+  if (spread) load = launch_load(&unit, 1, Hq, Hkv, true);
+  if (int32_t rc = fill_bwd_run(&P.run[0], g, p, B, q, do_src, k, v, sc.dq32, lse, delta, dk, dv, partial, spread ? &load : nullptr))
+    return rc;
   if (int32_t rc = launch_fused(P, dim3(P.run[0].plane, 1, B), p, scale, st)) return rc;
   ReduceRuns<1> C;
   C.n = 0;
@@ -1888,7 +1922,9 @@ int32_t launch_bwd_sm100_runs(const SeqRun* runs, int n_runs, long long tokens, 
   for (int first = 0; first < n_runs; first += kMaxRunsPerLaunch) {
     const int n = n_runs - first < kMaxRunsPerLaunch ? n_runs - first : kMaxRunsPerLaunch;
     // the launches run one after the other: what one SM has to do in each goes by its own units
-    const long long load = spread ? launch_load(runs + first, n, Hq) : -1;
+    LaunchLoad launch;
+    if (spread) launch = launch_load(runs + first, n, Hq, Hkv, false);
+    const LaunchLoad* load = spread ? &launch : nullptr;
     float* partial_of[kMaxRunsPerLaunch];
     for (int i = 0; i < n; ++i) {
       partial_of[i] = reinterpret_cast<float*>(partial_at);

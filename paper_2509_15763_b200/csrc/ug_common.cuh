@@ -232,9 +232,9 @@ inline bool bwd_is_fused(int D, uint32_t flags) { return D == 128 && !(flags & U
 // backward the fp32 dQ accumulator.
 size_t bwd_scratch_bytes(long long tokens, int Hq, int D, bool dout_fp32, bool fused);
 // Bytes behind that scratch for the fp32 partial dK / dV of the sink and gist key tiles whose walk over the
-// queries is cut into chunks (0 where nothing is cut), for the units of ONE launch of the fused backward.  spread: walks that are
-// cut only to spread them over idle SMs too; without them, the least that is accepted.
-size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool spread);
+// queries is cut into chunks (0 where nothing is cut), for the units of ONE launch of the fused backward.  in_turn: one problem,
+// not a packed sample.  spread: walks that are cut only to spread them over idle SMs too; without them, the least that is accepted.
+size_t bwd_partial_bytes(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_turn, bool spread);
 int32_t bwd_sm100_take_timeout(bool* timed_out);
 int32_t launch_compact_gather(const Geom& g, const unigist_problem& p, const void* k,
                               const void* v, void* kc, void* vc, int num_blocks,

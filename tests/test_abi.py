@@ -145,3 +145,20 @@ def test_packed_backward_workspace_goes_by_launch(sinks):
     assert partial_sums(first + second + third) == sum(map(partial_sums, (first, second, third)))
     one = ug.Problem(1, 3000, 8, 128, hq, hkv, dim, num_sinks=sinks)  # a sample of one document is the problem itself
     assert ug.unigist_workspace_bytes(one, ug.OP_BWD) == ug.unigist_docs_workspace_bytes(p, ug.OP_BWD, third)
+
+
+@pytest.mark.parametrize("problem,cut", [
+    # a walk that does not outlast what fills the other SMs is left whole (uncut and cut, us: 147 and 167, 108 and 119, 153 and 160)
+    ((4, 384, 16, 128, 64, 8, 128), False), ((8, 792, 8, 512, 8, 2, 128), False), ((4, 472, 8, 64, 64, 8, 0), False),
+    # (104 and 129: the blocks no longer fit the SMs at once)
+    ((8, 288, 16, 128, 32, 4, 0), False),
+    # 560 steps for every SM, 576 in the longest walk
+    ((1, 16384, 8, 1024, 32, 8, 0), False),
+    # 83 and 72, 261 and 203 (the last sequence's walks start late), 693 and 487, 92 and 46
+    ((4, 128, 8, 128, 64, 8, 128), True), ((4, 760, 8, 64, 64, 8, 0), True), ((8, 4352, 16, 512, 8, 2, 4), True),
+    ((1, 1024, 8, 128, 16, 4, 0), True)], ids=str)
+def test_walks_are_cut_where_they_outlast_the_rest(problem, cut):
+    batch, raw, ratio, window, hq, hkv, sinks = problem
+    p, al = ug.Problem(batch, raw, ratio, window, hq, hkv, 128, num_sinks=sinks), lambda x: -(-x // 256) * 256
+    rows = batch * ug.unigist_total_len(p) * hq
+    assert (ug.unigist_workspace_bytes(p, ug.OP_BWD) > al(rows * 4) + al(rows * 128 * 4)) == cut
