@@ -1679,14 +1679,15 @@ LaunchLoad launch_load(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_
 // quarters of the L2: however the blocks start, what one has read is still there for the next.  Otherwise into at
 // most four chunks of at least 16 query tiles, fewer where the chunks' fp32 partial sums would take more than
 // half the room of the dQ accumulator.
-// Where the longest sink or gist walk would outlast the rest of the launch by eight steps or more (a step is about 2 us), that
-// walk is cut too, if the workspace has room (load != nullptr): into chunks of half of the time the rest takes, no shorter than
-// the longest raw key tile's walk; the second kernel and the partial sums cost about 5 us.  Whole backward, us, uncut and cut;
-// steps of the longest walk / of the rest: 512 raw tokens, ratio 4, window 64, 32 / 8 heads 61 and 50, 22 / 4; 1024, ratio 8,
-// window 128, 16 / 4 heads 91 and 47, 38 / 4; 4096, ratio 16, 16 / 2 heads 597 and 107, 274 / 16; 9000, ratio 8, 32 / 8 heads 805
-// and 509, 322 / 150; 4096, window 1024 378 and 310, 146 / 112; 16384 578 / 598, not cut; 4 x 384, ratio 16, window 128, 128
-// sinks, 64 / 8 heads 147 and 167, 42 / 44, not cut.  Over 1367 problems that it cuts, of 128 - 24000 tokens: half the uncut time
-// on average, 3 % above the best number of chunks, one slower than uncut by more than 3 %.
+// Where the longest sink or gist walk, or chunk of one, would outlast the rest of the launch by eight steps or more (a step is
+// about 2 us), the walks are cut further, if the workspace has room (load != nullptr): into chunks of half of the time the rest
+// takes, no shorter than the longest raw key tile's walk; the second kernel and the partial sums cost about 5 us.  Whole
+// backward, us, uncut and cut; steps of the longest walk / of the rest: 512 raw tokens, ratio 4, window 64, 32 / 8 heads 61 and
+// 50, 22 / 4; 1024, ratio 8, window 128, 16 / 4 heads 91 and 47, 38 / 4; 4096, ratio 16, 16 / 2 heads 597 and 107, 274 / 16; 9000,
+// ratio 8, 32 / 8 heads 805 and 509, 322 / 150; 4096, window 1024 378 and 310, 146 / 112; 16384 578 / 598, not cut; 4 x 384,
+// ratio 16, window 128, 128 sinks, 64 / 8 heads 147 and 167, 42 / 44, not cut; 11520, ratio 16, 16 / 2 heads, past the L2, 497 in
+// the four chunks of 192 steps that the L2 asks for and 271 in chunks of 48.  Over 1367 problems that it cuts, of 128 - 24000
+// tokens: half the uncut time on average, 3 % above the best number of chunks, one slower than uncut by more than 3 %.
 // -> tiles per chunk, number of chunks of the longest walk (1 = no cutting, no partial sums).
 void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, const LaunchLoad* load, int* n_chunks, int* chunk_tiles) {
   const int n_raw = tiles(g.T), n_gist = tiles(g.n), n_heavy = tiles(g.s) + n_gist;
@@ -1697,11 +1698,12 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, const LaunchLoad* l
   while (C > 1 && ((max_tiles + C - 1) / C < 16 ||
                    (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2))
     --C;
-  if (load && C == 1 && n_heavy > 0) {
-    const long long longest = (long long)max_tiles * (Hq / Hkv), target = std::max(load->raw_walk, load->end / 2);
+  if (load && n_heavy > 0) {
+    const long long G = Hq / Hkv, longest = (max_tiles + C - 1) / C * G, target = std::max(load->raw_walk, load->end / 2);
     const long long start = load->late + kBlockSteps;
-    if (start + longest - std::max(start + target, load->end) >= 8) C = (int)((longest + target - 1) / target);
-    while (C > 1 && (size_t)batch * Hkv * n_heavy * C * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2) --C;
+    int more = start + longest - std::max(start + target, load->end) >= 8 ? (int)((max_tiles * G + target - 1) / target) : C;
+    while (more > C && (size_t)batch * Hkv * n_heavy * more * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2) --more;
+    C = std::max(C, more);
   }
   *chunk_tiles = (max_tiles + C - 1) / C;
   *n_chunks = (max_tiles + *chunk_tiles - 1) / *chunk_tiles;

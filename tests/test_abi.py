@@ -162,3 +162,16 @@ def test_walks_are_cut_where_they_outlast_the_rest(problem, cut):
     p, al = ug.Problem(batch, raw, ratio, window, hq, hkv, 128, num_sinks=sinks), lambda x: -(-x // 256) * 256
     rows = batch * ug.unigist_total_len(p) * hq
     assert (ug.unigist_workspace_bytes(p, ug.OP_BWD) > al(rows * 4) + al(rows * 128 * 4)) == cut
+
+
+@pytest.mark.parametrize("raw", [11520, 12288, 16384])
+def test_chunks_do_not_jump_where_the_l2_rule_begins(raw):
+    """One KV head's rows outgrow the L2 between 11264 and 11520 raw tokens here, and from there on walks are cut for that reason;
+    they are still cut as short as the idle SMs ask."""
+    def chunk_tiles(raw):
+        p, al = ug.Problem(1, raw, 16, 128, 16, 2, 128), lambda x: -(-x // 256) * 256
+        rows, gist = ug.unigist_total_len(p) * 16, -(-raw // 16 // 128)
+        chunks = (ug.unigist_workspace_bytes(p, ug.OP_BWD) - al(rows * 4) - al(rows * 128 * 4)) // (2 * gist * 2 * 128 * 128 * 4)
+        return (-(-raw // 128) + gist) / chunks
+
+    assert chunk_tiles(raw) <= 1.2 * raw / 11264 * chunk_tiles(11264)
