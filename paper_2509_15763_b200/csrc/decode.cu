@@ -211,7 +211,7 @@ struct Walk {
 // kApart: a stage's K and V arrive and are free again each by itself, instead of together (full_k, free_v).  A warp has one
 // stage; with barriers of its own the K of its next page comes under this one's softmax and P V.  That pays where walks are
 // short and bound by latency and a warp takes more than one page (8 sequences of 2112 tokens: 11.3 -> 10.6 us); with one page
-// a warp it only costs (one of 1337: 5.38 -> 5.41), and a long walk is bound by the memory system, which takes K and V apart
+// a warp it only costs (one of 1337: 5.39 -> 5.41), and a long walk is bound by the memory system, which takes K and V apart
 // badly (past six rounds of pages: one of 65536, 44.5 -> 45.3 us; flat, 64 of 9216: 345 -> 357).
 template <bool kFlat, bool kApart>
 __global__ void __launch_bounds__(THREADS, 2)
@@ -220,16 +220,16 @@ decode_split_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_const
   extern __shared__ unsigned char smem_dyn[];
   const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* gen = smem_dyn + (base - smem_u32(smem_dyn));
-  // barriers, + 8 * stage
-  const uint32_t full_k = base + DecSmem::kOffBars, full_v = full_k + 8 * STAGES, free_k = full_v + 8 * STAGES,
-                 free_v = free_k + 8 * STAGES;
+  // barriers, + 8 * stage; together, a stage's K and V use full_k and free_v only, which come first
+  const uint32_t full_k = base + DecSmem::kOffBars, free_v = full_k + 8 * STAGES, full_v = free_v + 8 * STAGES,
+                 free_k = full_v + 8 * STAGES;
   float* merge = reinterpret_cast<float*>(gen + DecSmem::kOffMerge);
   long long* first = reinterpret_cast<long long*>(gen + DecSmem::kOffFirst);
   const int hk = blockIdx.y, G = P.G;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 4 * STAGES; ++i) mbar_init(full_k + 8 * i, 1);
+    for (int i = 0; i < (kApart ? 4 : 2) * STAGES; ++i) mbar_init(full_k + 8 * i, 1);
     mbar_fence_init();
   }
   pdl_wait();  // nothing above touches global memory
