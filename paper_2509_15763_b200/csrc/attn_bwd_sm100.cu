@@ -1639,6 +1639,26 @@ int32_t launch_convert(const TokRuns<kRuns>& T, const unigist_problem& p, long l
 }
 
 int tiles(long long rows) { return (int)((rows + 127) / 128); }
+// The walks of one sequence's key tiles for one query head: steps (key tile, query tile) of all, steps of the longest raw key
+// tile's, and how many blocks they take if the sink and gist ones are cut into two at least.
+struct Walks {
+  long long steps;
+  int longest_raw, blocks;
+};
+Walks count_walks(const Geom& g) {
+  const FastDiv rdiv = make_fastdiv(g.r);
+  const int all = tiles(g.s) + tiles(g.T) + tiles(g.n);
+  Walks w = {0, 0, 0};
+  for (int kseg = 0; kseg < 3; ++kseg)
+    for (int key = 0; key < seg_len(g, kseg); key += 128) {
+      const int n = count_q_tiles(g, rdiv, kseg, key, std::min(key + 127, seg_len(g, kseg) - 1));
+      w.steps += n;
+      w.blocks += kseg != kSegRaw && n > (all + 1) / 2 ? 2 : 1;
+      if (kseg == kSegRaw) w.longest_raw = std::max(w.longest_raw, n);
+    }
+  return w;
+}
+
 // What a launch of the fused backward holds besides its longest walk, in steps (key tile, query tile, query head).
 struct LaunchLoad {
   long long end;       // when the SMs would be through if no walk outlasted the others and the long ones were cut
@@ -1652,18 +1672,11 @@ LaunchLoad launch_load(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_
   long long steps = 0, raw_walk = 0, blocks = 0, before_last = 0;
   for (int i = 0; i < n_runs; ++i) {
     const Geom& g = runs[i].g;
-    const FastDiv rdiv = make_fastdiv(g.r);
+    const Walks w = count_walks(g);
     const long long n_heavy = tiles(g.s) + tiles(g.n), n_raw = tiles(g.T);
-    long long n_steps = 0, n_blocks = 0;
-    for (int kseg = 0; kseg < 3; ++kseg)
-      for (int key = 0; key < seg_len(g, kseg); key += 128) {
-        const int n = count_q_tiles(g, rdiv, kseg, key, std::min(key + 127, seg_len(g, kseg) - 1));
-        n_steps += n;
-        n_blocks += kseg != kSegRaw && n > (n_heavy + n_raw + 1) / 2 ? 2 : 1;  // (if it is cut, two at least)
-        if (kseg == kSegRaw) raw_walk = std::max(raw_walk, n * G);
-      }
-    steps += n_steps * Hq * runs[i].batch;
-    blocks += n_blocks * Hkv * runs[i].batch;
+    steps += w.steps * Hq * runs[i].batch;
+    blocks += (long long)w.blocks * Hkv * runs[i].batch;
+    raw_walk = std::max(raw_walk, w.longest_raw * G);
     before_last = ((n_heavy + n_raw) * (runs[i].batch - 1) + n_heavy) * Hkv;
   }
   LaunchLoad load;
@@ -1788,24 +1801,16 @@ size_t unit_partial_bytes(const SeqRun& r, int Hq, int Hkv, const LaunchLoad* lo
   return align256((size_t)r.batch * Hkv * (tiles(r.g.s) + tiles(r.g.n)) * C * 2 * 128 * 128 * sizeof(float));
 }
 
-// Steps (key tile, query tile, query head) of `batch` sequences, estimated: a raw key tile's walk is taken as the longest that it
-// can be, k + 1 units and their gists; a gist key is seen by the later half of all rows on average.
-long long bwd_steps(const Geom& g, int batch, int Hq) {
-  const long long sink = tiles(g.s), raw = tiles(g.T), gist = tiles(g.n);
-  const long long raw_walk = std::min(tiles((g.k + 1ll) * g.r) + 1, tiles(g.T)) + std::min(tiles(g.k + 1ll) + 1, tiles(g.n));
-  return (sink * (sink + raw + gist) + gist * (raw + gist + 1) / 2 + raw * raw_walk) * Hq * batch;
-}
-
-// Whether two blocks share each sink or gist key tile of the dK / dV kernel: where the longest walk (the first gist key tile's)
-// would otherwise be the kernel's tail.  All blocks' steps are counted to within a tile, per SM; a walk up to 3/4 of that and
-// 22 steps ends under the raw key tiles that are left, and sharing it only costs blocks (us of the whole backward, shared and
-// not; steps of the longest walk / of an SM: 1 x 8190 raw tokens, 16 / 4 heads, 296 / 102: 305 and 456; 2 x 8190, 296 / 205: 529
-// and 577; 2 x 12288, ratio 3, 384 / 396: 1058 and 1150; 4 x 8190, 296 / 411: 1043 and 1005; 8 x 2048, 80 / 105: 301 and 283; 256
-// x 128, 8 / 83: 618 and 422; 1 x 448, one head, 5 / 0: 23.8 and 21.9).
+// Whether two blocks share each sink or gist key tile of the dK / dV kernel: where the longest walk (the first sink or gist key
+// tile's) would otherwise be the time.  The dQ blocks fill the SMs that the tail of that kernel leaves idle, and they are about as
+// much work again: up to twice the steps of an SM, and eight, a walk is hidden, and sharing it only costs blocks (us of the whole
+// backward, shared and not; steps of the longest walk / of an SM: 1 x 8190 raw tokens, ratio 7, window 700, 16 / 4 heads, 296 / 100:
+// 252 and 325; 2 x 8190, 296 / 201: 494 and 487; 4 x 8190, 296 / 400: 1043 and 1022; 2 x 12288, ratio 3, 512 / 658: 1577 and 1548;
+// 8 x 2048, ratio 8, 72 / 121: 363 and 352; 256 x 128, 8 / 111: 612 and 422; 1 x 592, 32 / 8 heads, 24 / 4: 28.1 and 36.9; 1 x 448,
+// one head, 5 / 0: 15.9 and 14.1).  Over 1931 problems of 128 - 24000 tokens 0.3 % above the better of the two.
 bool dkdv_shares(const Geom& g, int batch, int Hq, int Hkv) {
-  const long long all = tiles(g.s) + tiles(g.T) + tiles(g.n), G = Hq / Hkv;
-  const long long steps = bwd_steps(g, batch, Hq) / sm_count();
-  return all * G > steps * 3 / 4 + 22;
+  const long long longest = (long long)(tiles(g.s) + tiles(g.T) + tiles(g.n)) * (Hq / Hkv);
+  return longest > 2 * (count_walks(g).steps * Hq * batch / sm_count()) + 8;
 }
 
 // The two-kernel backward (head_dim 64; head_dim 128 when dQ has to be the same bit for bit from run to run): a

@@ -21,7 +21,8 @@ CASES = [
     synth.Workload("two_gist_tiles", 1, 130 * 5, 5, 35, 8, 2, 64, num_sinks=130, seed=505),
     synth.Workload("two_gist_tiles_128", 1, 130 * 5, 5, 35, 4, 2, 128, num_sinks=130, seed=506),
     synth.Workload("odd_raw_128", 2, 3 * 128 + 7, 1, 50, 2, 1, 128, seed=507),
-    # walks of more than 22 steps (query tiles times heads of a group): these are shared
+    synth.Workload("whole_odd_raw_128", 2, 3 * 128 + 7, 1, 50, 1, 1, 128, seed=508),
+    # walks of more than 8 steps (query tiles times heads of a group): these, and some of the above, are shared
     synth.Workload("shared_one_tile_each", 1, 9, 3, 6, 12, 1, 64, seed=511),
     synth.Workload("shared_sinks_only_tile", 1, 4, 4, 4, 8, 1, 64, num_sinks=3, seed=512),
     synth.Workload("shared_odd_raw_tiles", 2, 3 * 128, 3, 60, 12, 2, 64, seed=513),
