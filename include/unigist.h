@@ -168,14 +168,17 @@ int32_t unigist_attn_fwd(const unigist_problem* p, const void* q, const void* k,
  * q, k, v, o, lse as in the forward; d_o [B,N,Hq,D] device bf16 (fp32 with
  * UNIGIST_FLAG_DOUT_FP32); dq [B,N,Hq,D], dk, dv [B,N,Hkv,D] device bf16, all shifted.
  * dK/dV are accumulated without atomics: a key tile is owned by one thread block, or, where very many queries see
- * it (sink and gist keys of a long sequence), by one block per chunk of those queries whose fp32 partial sums a
- * small kernel, or the two blocks of a cluster, add in a fixed order; either way they are the same bit for bit from run to run.  For head_dim 128
+ * it (sink and gist keys of a long sequence, or of a call that leaves SMs idle), by one block per chunk of those queries
+ * whose fp32 partial sums a small kernel, or the two blocks of a cluster, add in a fixed order; either way they are the
+ * same bit for bit from run to run.  The chunks go by the whole call (batch and heads, the documents of a packed sample,
+ * the workspace): a sequence alone and in a batch may differ in the last bits of dK and dV.  For head_dim 128
  * dQ is the sum, over the key tiles that see a query tile, of fp32 partial tiles reduced into the workspace in
  * whatever order the blocks arrive: its last bit may differ between runs (UNIGIST_FLAG_DETERMINISTIC_DQ trades
  * speed for a fixed order).  workspace:
  * unigist_workspace_bytes(p, UNIGIST_OP_BWD) bytes (Delta, a bf16 copy of an fp32 dO, and for head_dim 128 the
  * fp32 dQ accumulator and the chunks' partial dK / dV), 16-byte aligned.  Less is accepted, down to a size without those
- * partial sums that only spread a walk over idle SMs: the call is then slower, dK / dV may differ in their last bits.
+ * partial sums that only spread a walk over idle SMs: the call is then slower, dK / dV may differ in their last bits (a size
+ * in between is taken like the least).
  */
 int32_t unigist_attn_bwd(const unigist_problem* p, const void* q, const void* k, const void* v,
                          const void* o, const float* lse, const void* d_o, void* dq, void* dk,
@@ -194,7 +197,8 @@ int32_t unigist_attn_bwd(const unigist_problem* p, const void* q, const void* k,
  * units, of equal or different lengths, share ONE launch of each kernel (every thread block finds its document
  * from its block index; the units' tensor maps travel as kernel parameters), a sample with more units takes one
  * launch per twelve.  Everything is enqueued on `stream`.  For head_dim 64 the backward runs its two kernels once
- * per unit.  workspace (backward only): unigist_docs_workspace_bytes bytes.
+ * per unit.  workspace (backward only): unigist_docs_workspace_bytes bytes; for head_dim 128 less is accepted as by
+ * unigist_attn_bwd, with the same effect.
  * Errors as for unigist_attn_fwd / unigist_attn_bwd, raised before the first launch where the list is malformed.
  */
 int64_t unigist_docs_total_len(const unigist_problem* p, int32_t num_docs, const int32_t* doc_raw_len);

@@ -134,12 +134,13 @@ __host__ __device__ inline int seg_row_to_token(const Geom& g, bool interleaved,
 
 // Programmatic dependent launch: returns when the kernel before this one on the stream has completed and its writes are
 // visible; every thread calls it before its first access to global memory (in a kernel launched without the attribute it
-// does nothing).
+// does nothing).  The one exception is the dQ kernel beside dK / dV (after_dkdv == 0), see pdl_release.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel on the stream start once every block of this one has called it or ended.  Only where that kernel can
 // work before this one is done: blocks that just sit on the SMs and wait made a training pass 2 - 4 % longer.  Such a kernel
-// reads nothing that this one writes, reads what came before this one past the L1, and its last block calls pdl_wait(), so
-// that its own end still stands for everything before it on the stream.
+// reads nothing that this one writes and writes nothing that this one still reads (the host compares their buffers), reads what
+// came before this one past the L1, and its last block calls pdl_wait(), so that its own end still stands for everything before it
+// on the stream.
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Host side helpers (api.cu).
@@ -161,7 +162,8 @@ struct KernelScope {
   int slot;
   cudaStream_t st;
 };
-// Launches a kernel whose first access to global memory comes after pdl_wait(): its launch is prepared while the one before
+// Launches a kernel whose first access to global memory comes after pdl_wait() (or whose predecessor calls pdl_release() for it,
+// under the conditions there): its launch is prepared while the one before
 // it on the stream runs, and its blocks start once the last block of that one has ended (or has let its successor in
 // earlier, see above), so that launch latency is hidden and the prologue runs while the predecessor's writes are made
 // visible.  cluster > 1: blocks along x in clusters of that many.  An error is picked up by check_launch.
