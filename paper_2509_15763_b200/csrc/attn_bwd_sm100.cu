@@ -1699,7 +1699,8 @@ LaunchLoad launch_load(const SeqRun* runs, int n_runs, int Hq, int Hkv, bool in_
 // 50, 22 / 4; 1024, ratio 8, window 128, 16 / 4 heads 91 and 47, 38 / 4; 4096, ratio 16, 16 / 2 heads 597 and 107, 274 / 16; 9000,
 // ratio 8, 32 / 8 heads 805 and 509, 322 / 150; 4096, window 1024 378 and 310, 146 / 112; 16384 578 / 598, not cut; 4 x 384,
 // ratio 16, window 128, 128 sinks, 64 / 8 heads 147 and 167, 42 / 44, not cut; 11520, ratio 16, 16 / 2 heads, past the L2, 497 in
-// the four chunks of 192 steps that the L2 asks for and 271 in chunks of 48.  Over 1367 problems that it cuts, of 128 - 24000
+// the four chunks of 192 steps that the L2 asks for and 271 in chunks of 48 (chunks are cut again only if they outlast the rest by
+// an eighth: 33012, ratio 4, window 64, 8 / 1 heads, in 4 and 9 chunks, 1770 and 1931).  Over 1367 problems that it cuts, of 128 - 24000
 // tokens: half the uncut time on average, 3 % above the best number of chunks, one slower than uncut by more than 3 %.
 // -> tiles per chunk, number of chunks of the longest walk (1 = no cutting, no partial sums).
 void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, const LaunchLoad* load, int* n_chunks, int* chunk_tiles) {
@@ -1713,8 +1714,8 @@ void bwd_chunking(const Geom& g, int batch, int Hq, int Hkv, const LaunchLoad* l
     --C;
   if (load && n_heavy > 0) {
     const long long G = Hq / Hkv, longest = (max_tiles + C - 1) / C * G, target = std::max(load->raw_walk, load->end / 2);
-    const long long start = load->late + kBlockSteps;
-    int more = start + longest - std::max(start + target, load->end) >= 8 ? (int)((max_tiles * G + target - 1) / target) : C;
+    const long long start = load->late + kBlockSteps, least = C > 1 ? std::max(8ll, load->end / 8) : 8;
+    int more = start + longest - std::max(start + target, load->end) >= least ? (int)((max_tiles * G + target - 1) / target) : C;
     while (more > C && (size_t)batch * Hkv * n_heavy * more * 2 * 128 * 128 * sizeof(float) > dq_bytes / 2) --more;
     C = std::max(C, more);
   }
